@@ -1,0 +1,426 @@
+"""Performance cases: the work that users of the library have it do, each
+through the package's public entry points.
+
+Kinds of case (``"kind"``):
+
+* ``nve``    ``System.step`` and ``System.state``: velocity-Verlet NVE of an LJ
+             liquid or an EAM metal, then the state read back.
+* ``batch``  the same for a batch of independent LJ replicas in one handle.
+* ``eval``   ``System.set_state``, ``compute_forces`` and ``energy_virial`` at
+             coordinates the caller supplies (Monte Carlo moves, minimisers,
+             re-evaluating a stored trajectory, another program's integrator).
+* ``match``  a force-matching step through autograd (``LJForces`` /
+             ``EAMForces``): forces, squared-error loss, gradients of positions
+             and potential parameters.
+
+Sizes, densities, temperatures, cut-offs and time steps are those of the
+repository's own workloads (``synth``, ``bench.py``, the tests); ``draw`` spreads
+them over the ranges between.
+"""
+from __future__ import annotations
+
+import math
+
+import numpy as np
+import torch
+
+import paper_1009_4330_gb300 as md
+
+RHO, TEMP, DT, SKIN = 0.8442, 1.44, 0.005, 0.3              # LJ liquid
+EAM = (4.95, 1.0, 0.5, -0.2, 0.02)                          # rc, A, c0, c1, c2 (eV, Angstrom)
+EAM_A, EAM_MASS, EAM_SKIN, EAM_DT = 3.615, 63.55, 0.5, 1.0  # Angstrom, amu, Angstrom, fs
+FTM2V, KB = 9.64853321e-3, 8.617333262e-5
+KA_EPS, KA_SIG = (1.0, 1.5, 0.5), (1.0, 0.8, 0.88)          # binary mixture, pairs AA, AB, BB
+KA_RHO = 1.2
+
+
+def listed():
+    return [
+        # the smallest system of the batch workload alone: launches and latency set its step
+        {"name": "nve_lj500_mixed", "kind": "nve", "pot": "lj", "n": 500, "prec": "mixed", "rc": 2.5, "steps": 20,
+         "tpa": 1, "list": "full", "types": 1},
+        # the small reference system: 4,000 atoms in double precision, 100 steps to a call
+        {"name": "nve_lj4000_fp64", "kind": "nve", "pot": "lj", "n": 4000, "prec": "fp64", "rc": 2.5, "steps": 100,
+         "tpa": 8, "list": "full", "types": 1},
+        # an ordinary system of a production run, with a ragged size
+        {"name": "nve_lj32771_mixed", "kind": "nve", "pot": "lj", "n": 32771, "prec": "mixed", "rc": 2.5, "steps": 50,
+         "tpa": 1, "list": "full", "types": 1},
+        # the headline liquid, 864,000 atoms, at both of its cut-offs
+        {"name": "nve_lj864k_mixed", "kind": "nve", "pot": "lj", "n": 864000, "prec": "mixed", "rc": 2.5, "steps": 20,
+         "tpa": 1, "list": "full", "types": 1},
+        {"name": "nve_lj864k_rc5_mixed", "kind": "nve", "pot": "lj", "n": 864000, "prec": "mixed", "rc": 5.0,
+         "steps": 10, "tpa": 1, "list": "full", "types": 1},
+        # double precision at size, with the half list that the set-up benchmark picks there
+        {"name": "nve_lj256k_fp64_half", "kind": "nve", "pot": "lj", "n": 256000, "prec": "fp64", "rc": 2.5,
+         "steps": 10, "tpa": 4, "list": "half", "types": 1},
+        # the EAM metal, mixed (500,000 atoms) and double precision (108,000 atoms)
+        {"name": "nve_eam500k_mixed", "kind": "nve", "pot": "eam", "n": 500000, "prec": "mixed", "steps": 20, "tpa": 1},
+        {"name": "nve_eam108k_fp64", "kind": "nve", "pot": "eam", "n": 108000, "prec": "fp64", "steps": 10, "tpa": 1},
+        # ensemble sampling: 512 replicas of 500 to 20,000 atoms advanced together
+        {"name": "batch512_mixed", "kind": "batch", "n_rep": 512, "lo": 500, "hi": 20000, "prec": "mixed", "rc": 2.5,
+         "steps": 10, "tpa": 1},
+        # coordinates from outside, a binary mixture: forces, energy and virial at each set
+        {"name": "eval_lj100003_mixed", "kind": "eval", "pot": "lj", "n": 100003, "prec": "mixed", "rc": 2.5, "tpa": 1,
+         "list": "full", "types": 2},
+        # force matching: the 32,768-atom binary mixture, and the EAM metal
+        {"name": "match_lj32768_mixed", "kind": "match", "pot": "lj", "n": 32768, "prec": "mixed", "rc": 2.5, "tpa": 1,
+         "types": 2},
+        {"name": "match_eam108k_mixed", "kind": "match", "pot": "eam", "n": 108000, "prec": "mixed", "tpa": 1},
+    ]
+
+
+def _log(rng, lo, hi):
+    return int(round(math.exp(rng.uniform(math.log(lo), math.log(hi)))))
+
+
+def draw(rng):
+    kind = rng.choice(["nve", "nve", "nve", "batch", "eval", "match"])
+    prec = rng.choice(["mixed", "mixed", "fp64"])
+    slow = 15.0 if prec == "fp64" else 1.0  # double precision costs about so much more
+    if kind == "batch":
+        n_rep = _log(rng, 4, 512 if prec == "mixed" else 64)
+        return {"kind": "batch", "n_rep": n_rep, "lo": 500, "hi": _log(rng, 2000, 20000), "prec": prec, "rc": 2.5,
+                "steps": rng.randint(3, 10), "tpa": rng.choice([1, 1, 2])}
+    pot = rng.choice(["lj", "lj", "eam"])
+    tpa = rng.choice([1, 1, 1, 2, 4]) if prec == "mixed" else rng.choice([1, 4, 8])
+    most = 500000 if pot == "eam" else 864000
+    if kind == "match":
+        most = 108000 if pot == "eam" else 200000
+    n = _log(rng, 512 if pot == "lj" else 864, most if prec == "mixed" else min(most, 256000))
+    case = {"kind": kind, "pot": pot, "n": n, "prec": prec, "tpa": tpa}
+    if pot == "lj":
+        rc = 2.5
+        if kind != "match" and n >= 4000 and rng.random() < 0.3:
+            rc = round(rng.uniform(2.5, 5.0), 2)
+        case.update(rc=rc, types=rng.choice([1, 1, 2]))
+        if kind != "match":
+            case["list"] = rng.choice(["full", "half"]) if prec == "fp64" else "full"
+    if kind == "nve":
+        work = n * (case.get("rc", 2.5) / 2.5) ** 3 * slow
+        case["steps"] = max(2, min(rng.randint(5, 100), int(3.0e7 / work)))
+    return case
+
+
+# ------------------------------------------------------------------ inputs --
+
+def _rng(case, seed):
+    return np.random.default_rng([int(seed) % (1 << 32), int(case.get("n", case.get("n_rep", 0)))])
+
+
+def _sites(n, L, rng):
+    """n of the sites of the smallest fcc lattice holding them in a cube of edge L, chosen at random."""
+    m = max(1, int(math.ceil((n / 4.0) ** (1.0 / 3.0) - 1e-12)))
+    g = np.arange(m)
+    cells = np.stack(np.meshgrid(g, g, g, indexing="ij"), axis=-1).reshape(-1, 3)
+    basis = np.array([[0.0, 0.0, 0.0], [0.5, 0.5, 0.0], [0.5, 0.0, 0.5], [0.0, 0.5, 0.5]])
+    x = ((cells[:, None, :] + basis + 0.25) * (L / m)).reshape(-1, 3)
+    return x[np.sort(rng.permutation(x.shape[0])[:n])] if n < x.shape[0] else x
+
+
+def _velocities(n, kt_over_m, rng):
+    """Maxwell-Boltzmann velocities without net momentum."""
+    v = rng.standard_normal((n, 3)) * math.sqrt(kt_over_m)
+    return v - v.mean(axis=0)
+
+
+def _dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a), device="cuda")
+
+
+def _liquid(n, rho, jitter, rng):
+    L = (n / rho) ** (1.0 / 3.0)
+    return np.mod(_sites(n, L, rng) + rng.normal(0.0, jitter, (n, 3)), L), L
+
+
+def _matrix(aa, ab, bb):
+    return np.array([[aa, ab], [ab, bb]])
+
+
+def _inputs(case, seed):
+    """Positions, velocities, box edge, types and the potential's parameters of a single system, from the seed alone."""
+    rng = _rng(case, seed)
+    n = case["n"]
+    if case["pot"] == "eam":
+        L = EAM_A * (n / 4.0) ** (1.0 / 3.0)
+        x = np.mod(_sites(n, L, rng) + rng.normal(0.0, 0.1, (n, 3)), L)
+        v = _velocities(n, KB * 300.0 * FTM2V / EAM_MASS, rng)
+        return {"x": x, "v": v, "L": L, "types": np.zeros(n, np.int32), "mass": EAM_MASS, "rc": EAM[0],
+                "skin": EAM_SKIN, "dt": EAM_DT, "ftm2v": FTM2V, "params": np.array(EAM)}
+    mix = case["types"] == 2
+    x, L = _liquid(n, KA_RHO if mix and case["kind"] == "match" else RHO, 0.05 if case["kind"] == "match" else 0.03, rng)
+    v = _velocities(n, TEMP, rng)
+    t = np.zeros(n, np.int32)
+    if mix:
+        t[rng.permutation(n)[:int(round(0.2 * n))]] = 1
+    eps = _matrix(*KA_EPS) if mix else np.ones((1, 1))
+    sig = _matrix(*KA_SIG) if mix else np.ones((1, 1))
+    return {"x": x, "v": v, "L": L, "types": t, "mass": 1.0, "rc": case["rc"], "skin": SKIN, "dt": DT, "ftm2v": 1.0,
+            "eps": eps, "sig": sig}
+
+
+def _start_params(case, d, seed):
+    """Learnable starting values, up to 10 % away from the true ones."""
+    rng = np.random.default_rng([int(seed) % (1 << 32), 77])
+    if case["pot"] == "eam":
+        p = np.array(EAM) * (1.0 + rng.uniform(-0.1, 0.1, 5))
+        p[0] = EAM[0]
+        return (p,)
+    iu = np.triu_indices(case["types"])
+    return tuple(m[iu] * (1.0 + rng.uniform(-0.1, 0.1, iu[0].size)) for m in (d["eps"], d["sig"]))
+
+
+def _reference_forces(case, seed):
+    """The forces that a force-matching step is fitted to (any numbers of their size do)."""
+    rng = np.random.default_rng([int(seed) % (1 << 32), 78])
+    return rng.normal(0.0, 0.5 if case["pot"] == "eam" else 20.0, (case["n"], 3))
+
+
+def _replicas(case, seed):
+    sizes = np.random.default_rng(1004).uniform(math.log(case["lo"]), math.log(case["hi"]), case["n_rep"])
+    sizes = np.rint(np.exp(sizes)).astype(int)  # of the case alone; what is in the replicas is the seed's
+    rng = _rng(case, seed)
+    reps = []
+    for n in sizes:
+        L = (n / RHO) ** (1.0 / 3.0)
+        reps.append({"x": _sites(int(n), L, rng), "v": _velocities(int(n), TEMP, rng), "box": np.full(3, L)})
+    return reps
+
+
+def _system(case, d):
+    kw = dict(skin=d["skin"], dt=d["dt"], mass=d["mass"], ftm2v=d["ftm2v"], precision=case["prec"], tpa=case["tpa"])
+    box = np.full(3, d["L"])
+    if case["pot"] == "eam":
+        return md.System.eam(_dev(d["x"]), _dev(d["v"]), box, eam_params=d["params"], **kw)
+    return md.System.lj(_dev(d["x"]), _dev(d["v"]), box, eps=d["eps"], sig=d["sig"], types=_dev(d["types"]),
+                        n_types=case["types"], cutoff=d["rc"], list=case.get("list", "full"),
+                        **{**kw, "mass": [1.0] * case["types"]})
+
+
+def prepare(case, seed):
+    if case["kind"] == "batch":
+        reps = _replicas(case, seed)
+        for r in reps:
+            r["x"], r["v"] = _dev(r["x"]), _dev(r["v"])
+        s = md.System.batch(reps, params=md.lj_params(1.0, 1.0, 1), cutoff=case["rc"], skin=SKIN, dt=DT, mass=1.0,
+                            precision=case["prec"], tpa=case["tpa"])
+        return {"case": case, "system": s}
+    d = _inputs(case, seed)
+    state = {"case": case, "system": _system(case, d)}
+    if case["kind"] == "eval":
+        state["x"], state["v"] = _dev(d["x"]), _dev(d["v"])
+    if case["kind"] == "match":
+        state["x"] = _dev(d["x"]).requires_grad_()
+        state["theta"] = [_dev(p).requires_grad_() for p in _start_params(case, d, seed)]
+        state["target"] = _dev(_reference_forces(case, seed))
+    return state
+
+
+def run(state):
+    case, s = state["case"], state["system"]
+    if case["kind"] in ("nve", "batch"):
+        s.step(case["steps"])
+        x, v, f = s.state()
+        return {"x": x, "v": v, "f": f}
+    if case["kind"] == "eval":
+        s.set_state(x=state["x"], v=state["v"])
+        return {"f": s.compute_forces(), "ev": s.energy_virial()}
+    fn = md.EAMForces if case["pot"] == "eam" else md.LJForces
+    f = fn.apply(s, state["x"], *state["theta"])
+    loss = ((f - state["target"]) ** 2).sum()
+    grads = torch.autograd.grad(loss, [state["x"], *state["theta"]])
+    return {"f": f.detach(), "gx": grads[0], "gp": list(grads[1:])}
+
+
+def _neighbours(rho, rc):
+    return 4.0 / 3.0 * math.pi * rc ** 3 * rho
+
+
+def work(case):
+    """Operations: each pair within the cut-off evaluated once (23 for an LJ
+    pair, 35 for an EAM one, 30 more for its share of a backward pass).  Bytes:
+    positions and velocities read and written in every step, and the inputs and
+    outputs of the call."""
+    if case["kind"] == "batch":
+        lo, hi = case["lo"], case["hi"]
+        n = case["n_rep"] * (hi - lo) / math.log(hi / lo)
+    else:
+        n = case["n"]
+    eam = case.get("pot") == "eam"
+    if eam:
+        pairs = n * _neighbours(4.0 / EAM_A ** 3, EAM[0]) / 2.0
+    else:
+        dense = case["kind"] == "match" and case["types"] == 2
+        pairs = n * _neighbours(KA_RHO if dense else RHO, case["rc"]) / 2.0
+    flops = pairs * (35.0 if eam else 23.0)
+    if case["kind"] in ("nve", "batch"):
+        return {"bytes": case["steps"] * 96.0 * n + 72.0 * n, "flops": case["steps"] * flops}
+    if case["kind"] == "eval":
+        return {"bytes": 72.0 * n, "flops": flops}
+    return {"bytes": 96.0 * n, "flops": flops + 30.0 * pairs}
+
+
+# ------------------------------------------------- the same in plain torch --
+
+def _pairs(x, L, r):
+    """Every ordered pair (i, j) closer than r in a periodic cube of edge L."""
+    n, dev = x.shape[0], x.device
+    nb = int(L // r)
+    out = []
+
+    def keep(i, j, ok):
+        d = x[i] - x[j]
+        d -= L * torch.round(d / L)
+        ok = ok & ((d * d).sum(-1) < r * r) & (i != j)
+        out.append((i.expand(ok.shape)[ok], j.expand(ok.shape)[ok]))
+
+    if nb < 4 or n < 3000:
+        al = torch.arange(n, device=dev)
+        for a in range(0, n, 1024):
+            i = al[a:a + 1024, None]
+            keep(i, al[None, :], torch.ones((i.shape[0], n), dtype=torch.bool, device=dev))
+    else:
+        c = torch.clamp((torch.remainder(x, L) * (nb / L)).long(), 0, nb - 1)
+        cell = (c[:, 2] * nb + c[:, 1]) * nb + c[:, 0]
+        order = torch.argsort(cell)
+        count = torch.bincount(cell, minlength=nb ** 3)
+        first = torch.cumsum(count, 0) - count
+        width = int(count.max())
+        slot = torch.arange(width, device=dev)
+        table = order[torch.clamp(first[:, None] + slot, max=n - 1)]
+        full = slot < count[:, None]
+        al = torch.arange(nb ** 3, device=dev)
+        cx, cy, cz = al % nb, (al // nb) % nb, al // (nb * nb)
+        chunk = max(1, int(4.0e7 / width ** 2))
+        for k in range(27):
+            other = (((cz + k // 9 - 1) % nb) * nb + (cy + k // 3 % 3 - 1) % nb) * nb + (cx + k % 3 - 1) % nb
+            for a in range(0, nb ** 3, chunk):
+                s = slice(a, a + chunk)
+                keep(table[s][:, :, None], table[other[s]][:, None, :], full[s][:, :, None] & full[other[s]][:, None, :])
+    return torch.cat([p[0] for p in out]), torch.cat([p[1] for p in out])
+
+
+PIECE = 1 << 24
+
+
+class _Exact:
+    """Forces, energy and virial of one system in FP64 over a list of ordered pairs."""
+
+    def __init__(self, case, d):
+        self.case, self.L, self.rc = case, d["L"], d["rc"]
+        self.types = _dev(d["types"]).long()
+        if "params" in d:
+            self.p = _dev(d["params"])
+        else:
+            self.eps, self.sig = _dev(d["eps"]), _dev(d["sig"])
+        self.x0 = None
+
+    def list_for(self, x, slack):
+        if self.x0 is None or slack == 0 or float(((x - self.x0) ** 2).sum(1).max()) > (0.5 * slack) ** 2:
+            self.x0 = x.detach().clone()
+            self.i, self.j = _pairs(self.x0, self.L, self.rc + slack)
+
+    def sep(self, x, s):
+        i, j = self.i[s], self.j[s]
+        d = x[i] - x[j]
+        d = d - self.L * torch.round(d.detach() / self.L)
+        r2 = (d * d).sum(1)
+        ok = r2.detach() < self.rc ** 2
+        return i[ok], j[ok], d[ok], r2[ok]
+
+    def pieces(self):
+        return [slice(a, a + PIECE) for a in range(0, self.i.numel(), PIECE)]
+
+    def coefficient(self, i, j, r2, fp=None):
+        """-U'(r)/r and the pair energy"""
+        if fp is None:
+            e, g = self.eps[self.types[i], self.types[j]], self.sig[self.types[i], self.types[j]]
+            s6 = (g * g / r2) ** 3
+            return 24.0 * e * (2.0 * s6 * s6 - s6) / r2, 4.0 * e * (s6 * s6 - s6)
+        r = torch.sqrt(r2)
+        t = self.rc - r
+        poly = self.p[2] + r * (self.p[3] + r * self.p[4])
+        dphi = t * (t * (self.p[3] + 2.0 * self.p[4] * r) - 2.0 * poly)
+        return -(dphi - 2.0 * t * (fp[i] + fp[j])) / r, t * t * poly
+
+    def embedding(self, x):
+        rho = torch.zeros(x.shape[0], dtype=x.dtype, device=x.device)
+        for s in self.pieces():
+            i, _, _, r2 = self.sep(x, s)
+            rho = rho.index_add(0, i, (self.rc - torch.sqrt(r2)) ** 2)
+        safe = torch.where(rho > 0, rho, torch.ones_like(rho))
+        return torch.where(rho > 0, -0.5 * self.p[1] / torch.sqrt(safe), torch.zeros_like(rho))
+
+    def forces(self, x):
+        fp = self.embedding(x) if self.case.get("pot") == "eam" else None
+        f = torch.zeros_like(x)
+        for s in self.pieces():
+            i, j, d, r2 = self.sep(x, s)
+            f = f.index_add(0, i, d * self.coefficient(i, j, r2, fp)[0][:, None])
+        return f
+
+    def energy_virial(self, x, v, mass):
+        """Of an LJ system: Epot, Ekin, Wxx, Wyy, Wzz, Wxy, Wxz, Wyz."""
+        out = torch.zeros(8, dtype=x.dtype, device=x.device)
+        out[1] = 0.5 * mass * (v * v).sum()
+        for s in self.pieces():
+            i, j, d, r2 = self.sep(x, s)
+            c, e = self.coefficient(i, j, r2)
+            out[0] += 0.5 * e.sum()
+            for k, (a, b) in enumerate(((0, 0), (1, 1), (2, 2), (0, 1), (0, 2), (1, 2))):
+                out[2 + k] += 0.5 * (c * d[:, a] * d[:, b]).sum()
+        return out
+
+
+def _trajectory(case, d):
+    e = _Exact(case, d)
+    x, v = _dev(d["x"]), _dev(d["v"])
+    slack = 0.1 * d["rc"] if d["x"].shape[0] < 600000 else 0.0
+    acc, dt = d["ftm2v"] / d["mass"], d["dt"]
+    e.list_for(x, slack)
+    f = e.forces(x)
+    for _ in range(case["steps"]):
+        v = v + 0.5 * dt * acc * f
+        x = x + dt * v
+        e.list_for(x, slack)
+        f = e.forces(x)
+        v = v + 0.5 * dt * acc * f
+    return torch.remainder(x, d["L"]), v, f
+
+
+def exact(case, seed):
+    w = work(case)
+    if w["flops"] > 8.0e10:  # tens of seconds in plain torch
+        return None
+    if case["kind"] == "batch":
+        if case["n_rep"] * case["steps"] > 5200:
+            return None
+        got = [_trajectory(case, {"x": r["x"], "v": r["v"], "L": float(r["box"][0]),
+                                  "types": np.zeros(len(r["x"]), np.int32), "mass": 1.0, "rc": case["rc"], "skin": SKIN,
+                                  "dt": DT, "ftm2v": 1.0, "eps": np.ones((1, 1)), "sig": np.ones((1, 1))})
+               for r in _replicas(case, seed)]
+        return {k: torch.cat([g[q] for g in got]) for q, k in enumerate(("x", "v", "f"))}
+    d = _inputs(case, seed)
+    if case["kind"] == "nve":
+        x, v, f = _trajectory(case, d)
+        return {"x": x, "v": v, "f": f}
+    e = _Exact(case, d)
+    x = _dev(d["x"])
+    e.list_for(x, 0)
+    if case["kind"] == "eval":
+        if case["pot"] == "eam":
+            return {"f": e.forces(x), "ev": None}
+        return {"f": e.forces(x), "ev": e.energy_virial(x, _dev(d["v"]), d["mass"])[None]}
+    theta = [_dev(p).requires_grad_() for p in _start_params(case, d, seed)]
+    x.requires_grad_()
+    if case["pot"] == "eam":
+        e.p = theta[0]
+    else:
+        nt = case["types"]
+        where = torch.zeros((nt, nt), dtype=torch.long, device="cuda")
+        a, b = np.triu_indices(nt)
+        where[a, b] = where[b, a] = torch.arange(a.size, device="cuda")
+        e.eps, e.sig = theta[0][where], theta[1][where]
+    f = e.forces(x)
+    loss = ((f - _dev(_reference_forces(case, seed))) ** 2).sum()
+    grads = list(torch.autograd.grad(loss, [x, *theta]))
+    return {"f": f.detach(), "gx": grads[0], "gp": grads[1:]}
