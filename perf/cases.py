@@ -392,7 +392,7 @@ def exact(case, seed):
     if w["flops"] > 8.0e10:  # tens of seconds in plain torch
         return None
     if case["kind"] == "batch":
-        if case["n_rep"] * case["steps"] > 5200:
+        if case["n_rep"] * case["steps"] > 640:
             return None
         got = [_trajectory(case, {"x": r["x"], "v": r["v"], "L": float(r["box"][0]),
                                   "types": np.zeros(len(r["x"]), np.int32), "mass": 1.0, "rc": case["rc"], "skin": SKIN,
