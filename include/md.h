@@ -418,7 +418,7 @@ md_status md_probe_ceilings(void *stream, md_ceilings *out);
 
 /*
  * The library's FP64 reciprocal (op 0) and reciprocal square root (op 1) --
- * Newton-Raphson steps from the FP32 hardware approximations, used by the
+ * a third-order step each from the FP32 hardware approximations, used by the
  * FP64 force passes -- applied to x[n] (device), results in y[n] (device), on
  * `stream`.  For tests that hold them to an error bound against the
  * correctly rounded operations; valid for FLT_MIN < x < FLT_MAX.

@@ -1,6 +1,7 @@
-// k_force.cu -- pair-force kernels over the Verlet list (LJ full and half
-// list, EAM density and force passes), the drift and kick kernels of
-// velocity Verlet, and the md_step loop control.
+// k_force.cu -- mixed-precision pair-force kernels over the Verlet list (LJ
+// full and half list, EAM density and force passes; the FP64 ones are in
+// k_fp64.cu), the drift and kick kernels of velocity Verlet, and the md_step
+// loop control.
 //
 // Force loop (paper Sec. III.B): a group of T threads owns atom i
 // (T = 1 is the paper's thread-per-atom, T = 32 a warp-per-atom form of its
@@ -16,57 +17,23 @@
 // arithmetic in FP32, sums each round's (at most Q) pair terms plainly and
 // adds the round sum with Kahan compensation (forces, energy and virial
 // alike), and folds the compensated sums into FP64 for the group reduction,
-// kick and store.  FP64 does everything in double.
+// kick and store.
 #include "md_common.cuh"
 #include "md_kernels.h"
 
 namespace md {
 
-// ------------------------------------------------------ precision policy --
+// ------------------------------------------------------ FP32 pair helpers --
 
-template <int PREC>
-struct Pol;
-
-template <>
-struct Pol<MD_PREC_MIXED> {
-    using real = float;
-    using Acc = KahanF;
-    __device__ static __forceinline__ void load(const View &V, int j, float &x, float &y, float &z, int &t) {
-        const float4 r = __ldg(&V.rec[j]);
-        x = r.x; y = r.y; z = r.z; t = __float_as_int(r.w);
-    }
-    __device__ static __forceinline__ float h(const Rep &R, int c) { return R.hf[c]; }
-    __device__ static __forceinline__ float rcp(float x) {
-        float y;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-        return y;
-    }
-    __device__ static __forceinline__ float rsqrt(float x) { return rsqrtf(x); }
-    __device__ static __forceinline__ float fp(const View &V, int j) { return __ldg(&V.fp32[j]); }
-};
-
-struct AccD {
-    double s;
-    __device__ __forceinline__ void zero() { s = 0.0; }
-    __device__ __forceinline__ void add(double y) { s += y; }
-    __device__ __forceinline__ double value() const { return s; }
-};
-
-template <>
-struct Pol<MD_PREC_FP64> {
-    using real = double;
-    using Acc = AccD;
-    __device__ static __forceinline__ void load(const View &V, int j, double &x, double &y, double &z, int &t) {
-        const double4_32a q = V.pos4[j];
-        x = q.x; y = q.y; z = q.z; t = (int)__double_as_longlong(q.w);
-    }
-    __device__ static __forceinline__ double h(const Rep &R, int c) { return R.h[c]; }
-    // FP64 throughput is low on this GPU: Newton iterations from the FP32
-    // approximations instead of a full-precision divide / square root
-    __device__ static __forceinline__ double rcp(double x) { return rcp_newton(x); }
-    __device__ static __forceinline__ double rsqrt(double x) { return rsqrt_newton(x); }
-    __device__ static __forceinline__ double fp(const View &V, int j) { return V.fp64[j]; }
-};
+__device__ __forceinline__ void load_rec(const View &V, int j, float &x, float &y, float &z, int &t) {
+    const float4 r = __ldg(&V.rec[j]);
+    x = r.x; y = r.y; z = r.z; t = __float_as_int(r.w);
+}
+__device__ __forceinline__ float rcp32(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 
 __device__ __forceinline__ uint32_t ld_stream(const uint32_t *p) {
     uint32_t v;
@@ -111,9 +78,8 @@ __device__ __forceinline__ double group_sum(double x) {
 
 // |d|^2 with its operations spelled out (no contraction left to the compiler),
 // so that a pair's FP32 r^2 recomputed after the walk is the walk's own
-template <class real>
-__device__ __forceinline__ real pair_r2(real dx, real dy, real dz) {
-    return fma(dz, dz, fma(dy, dy, dx * dx));
+__device__ __forceinline__ float pair_r2(float dx, float dy, float dz) {
+    return fmaf(dz, dz, fmaf(dy, dy, dx * dx));
 }
 
 // Walk this thread's share of atom i's list: rounds of T*Q entries, the
@@ -126,24 +92,19 @@ __device__ __forceinline__ real pair_r2(real dx, real dy, real dz) {
 // added to the running total with compensation (blocked Kahan summation:
 // error ~ (Q + 2) u sum |terms| instead of ~n u for n plain additions).
 // LOCAL: the entries are block-local and the records come from the block's
-// staging in shared memory (srec; mixed precision only).
-template <int PREC, int T, int Q, bool LOCAL, class Pair>
-__device__ __forceinline__ void walk_list(const View &V, const uint32_t *lp, int sub, int cnt,
-                                          typename Pol<PREC>::real xi, typename Pol<PREC>::real yi,
-                                          typename Pol<PREC>::real zi, typename Pol<PREC>::real hx,
-                                          typename Pol<PREC>::real hy, typename Pol<PREC>::real hz,
-                                          const float4 *srec, Pair &pair) {
-    using P = Pol<PREC>;
-    using real = typename P::real;
+// staging in shared memory (srec).
+template <int T, int Q, bool LOCAL, class Pair>
+__device__ __forceinline__ void walk_list(const View &V, const uint32_t *lp, int sub, int cnt, float xi, float yi,
+                                          float zi, float hx, float hy, float hz, const float4 *srec, Pair &pair) {
     constexpr int PER = T * Q;
     const int nr = (cnt + PER - 1) / PER;
-    const real hy4 = hy * (real)0.25, hz16 = hz * (real)0.0625;  // exact: powers of two
+    const float hy4 = hy * 0.25f, hz16 = hz * 0.0625f;  // exact: powers of two
     uint32_t cur[Q], nxt[Q];
     if (nr > 0) load_entries<Q>(lp, cur);
     for (int r = 0; r < nr; ++r) {
         if (r + 1 < nr) load_entries<Q>(lp + (size_t)(r + 1) * 32 * Q, nxt);
         const int left = cnt - (r * PER + sub * Q);
-        real xj[Q], yj[Q], zj[Q];
+        float xj[Q], yj[Q], zj[Q];
         int tj[Q];
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
@@ -152,7 +113,7 @@ __device__ __forceinline__ void walk_list(const View &V, const uint32_t *lp, int
                     const float4 r4 = srec[entry_j(cur[q]) & (kTileCap - 1)];
                     xj[q] = r4.x; yj[q] = r4.y; zj[q] = r4.z; tj[q] = __float_as_int(r4.w);
                 } else {
-                    P::load(V, entry_j(cur[q]), xj[q], yj[q], zj[q], tj[q]);
+                    load_rec(V, entry_j(cur[q]), xj[q], yj[q], zj[q], tj[q]);
                 }
             }
         }
@@ -161,10 +122,10 @@ __device__ __forceinline__ void walk_list(const View &V, const uint32_t *lp, int
         for (int q = 0; q < Q; ++q) {
             if (q < left) {
                 const uint32_t e = cur[q];
-                const real dx = fma(-(real)code_x(e), hx, xi - xj[q]);
-                const real dy = fma(-(real)code_y4(e), hy4, yi - yj[q]);
-                const real dz = fma(-(real)code_z16(e), hz16, zi - zj[q]);
-                const real r2 = pair_r2(dx, dy, dz);
+                const float dx = fmaf(-code_x(e), hx, xi - xj[q]);
+                const float dy = fmaf(-code_y4(e), hy4, yi - yj[q]);
+                const float dz = fmaf(-code_z16(e), hz16, zi - zj[q]);
+                const float r2 = pair_r2(dx, dy, dz);
                 pair(e, dx, dy, dz, r2, tj[q]);
             }
         }
@@ -175,26 +136,18 @@ __device__ __forceinline__ void walk_list(const View &V, const uint32_t *lp, int
 }
 
 // the list walk in this block's tile mode (records staged or gathered)
-template <int PREC, int T, int Q, class Pair>
-__device__ __forceinline__ void walk_mode(const View &V, int mode, const uint32_t *lp, int sub, int cnt,
-                                          typename Pol<PREC>::real xi, typename Pol<PREC>::real yi,
-                                          typename Pol<PREC>::real zi, const Rep &R, const float4 *srec,
-                                          Pair &pair) {
-    using P = Pol<PREC>;
-    if constexpr (PREC == MD_PREC_MIXED) {
-        if (mode == 1) {
-            walk_list<PREC, T, Q, true>(V, lp, sub, cnt, xi, yi, zi, P::h(R, 0), P::h(R, 1), P::h(R, 2), srec, pair);
-            return;
-        }
-    }
-    walk_list<PREC, T, Q, false>(V, lp, sub, cnt, xi, yi, zi, P::h(R, 0), P::h(R, 1), P::h(R, 2), srec, pair);
+template <int T, int Q, class Pair>
+__device__ __forceinline__ void walk_mode(const View &V, int mode, const uint32_t *lp, int sub, int cnt, float xi,
+                                          float yi, float zi, const Rep &R, const float4 *srec, Pair &pair) {
+    if (mode == 1)
+        walk_list<T, Q, true>(V, lp, sub, cnt, xi, yi, zi, R.hf[0], R.hf[1], R.hf[2], srec, pair);
+    else
+        walk_list<T, Q, false>(V, lp, sub, cnt, xi, yi, zi, R.hf[0], R.hf[1], R.hf[2], srec, pair);
 }
 
 // stage the block's tile when its entries are block-local (before the
 // kernel's first block barrier)
-template <int PREC>
 __device__ __forceinline__ int begin_tile(const View &V, int T, float4 *srec) {
-    if constexpr (PREC != MD_PREC_MIXED) return 0;
     const int mode = tile_mode(V, T);
     if (mode == 1) stage_tile(V, blockIdx.x, srec);
     return mode;
@@ -247,91 +200,81 @@ __device__ __forceinline__ bool in_cut_fp64(const View &V, int p, uint32_t e) {
 // FULL: every neighbour in i's list, F_i only, no atomics.
 // HALF: each pair once; F_j -= f_ij by FP64 atomics, F_i += sum by one atomic
 //       per component at the end (F zeroed beforehand; kick in k_kick).
-template <int PREC, int MT, int HALF, int EV>
+template <int MT, int HALF, int EV>
 struct LJPair {
-    using real = typename Pol<PREC>::real;
-    using Acc = typename Pol<PREC>::Acc;
     const View *V;
-    const real *lj1, *lj2, *lj3, *lj4, *off;
-    real c3, c4, c0;  // one atom type: the energy coefficients and shift, likewise
-    real c1, c2;  // one atom type (MT = 0): the coefficients in registers, not
-                  // re-read from shared memory for every pair
-    real rc2;
+    const float *lj1, *lj2, *lj3, *lj4, *off;
+    float c3, c4, c0;  // one atom type: the energy coefficients and shift, likewise
+    float c1, c2;  // one atom type (MT = 0): the coefficients in registers, not
+                   // re-read from shared memory for every pair
+    float rc2;
     int ti, nt, n;
-    real near_min;  // mixed: the smallest |r^2 - rc^2| of this thread's pairs
-    Acc ax, ay, az, e;
-    Acc w[6];
-    real rx, ry, rz;  // this round's plain partial sums
-    real re, rw[6];   // and of the energy and virial terms (EV)
-    __device__ __forceinline__ bool in_cut(real r2) {
-        if constexpr (PREC == MD_PREC_MIXED) {
-            const real t = r2 - rc2;  // t < 0 exactly when r2 < rc2
-            near_min = fminf(near_min, fabsf(t));
-            return t < (real)0;
-        }
-        return r2 < rc2;
+    float near_min;  // the smallest |r^2 - rc^2| of this thread's pairs
+    KahanF ax, ay, az, e;
+    KahanF w[6];
+    float rx, ry, rz;  // this round's plain partial sums
+    float re, rw[6];   // and of the energy and virial terms (EV)
+    __device__ __forceinline__ bool in_cut(float r2) {
+        const float t = r2 - rc2;  // t < 0 exactly when r2 < rc2
+        near_min = fminf(near_min, fabsf(t));
+        return t < 0.f;
     }
     __device__ __forceinline__ void round_begin() {
         rx = 0; ry = 0; rz = 0;
-        if (EV && PREC == MD_PREC_MIXED) {
+        if (EV) {
             re = 0;
             for (int k = 0; k < 6; ++k) rw[k] = 0;
         }
     }
     __device__ __forceinline__ void round_end() {
         ax.add(rx); ay.add(ry); az.add(rz);
-        if (EV && PREC == MD_PREC_MIXED) {
+        if (EV) {
             e.add(re);
             for (int k = 0; k < 6; ++k) w[k].add(rw[k]);
         }
     }
     // energy and virial terms of one pair: summed plainly over the round and
-    // added with compensation per round (mixed), or added directly (FP64)
-    __device__ __forceinline__ void add_ev(real ee, real w0, real w1, real w2, real w3, real w4, real w5) {
-        if constexpr (PREC == MD_PREC_MIXED) {
-            re += ee;
-            rw[0] += w0; rw[1] += w1; rw[2] += w2; rw[3] += w3; rw[4] += w4; rw[5] += w5;
-        } else {
-            e.add(ee);
-            w[0].add(w0); w[1].add(w1); w[2].add(w2); w[3].add(w3); w[4].add(w4); w[5].add(w5);
-        }
+    // added with compensation per round
+    __device__ __forceinline__ void add_ev(float ee, float w0, float w1, float w2, float w3, float w4, float w5) {
+        re += ee;
+        rw[0] += w0; rw[1] += w1; rw[2] += w2; rw[3] += w3; rw[4] += w4; rw[5] += w5;
     }
-    __device__ __forceinline__ void operator()(uint32_t ent, real dx, real dy, real dz, real r2, int tj) {
-        // mixed full list, forces only: branch-free (the skin entries' terms are
+    __device__ __forceinline__ void operator()(uint32_t ent, float dx, float dy, float dz, float r2, int tj) {
+        // full list, forces only: branch-free (the skin entries' terms are
         // computed, finite since r2 >= rc^2 there, and zeroed) -- measured faster
         // than skipping them under a per-lane branch
-        if constexpr (!HALF && !EV && PREC == MD_PREC_MIXED) {
+        if constexpr (!HALF && !EV) {
             const int tp = MT ? ti * nt + tj : 0;
-            const real r2i = Pol<PREC>::rcp(r2);
-            const real r6i = r2i * r2i * r2i;
-            const real a1 = MT ? lj1[tp] : c1, a2 = MT ? lj2[tp] : c2;
-            real fpair = r6i * (a1 * r6i - a2) * r2i;
-            fpair = in_cut(r2) ? fpair : (real)0;
+            const float r2i = rcp32(r2);
+            const float r6i = r2i * r2i * r2i;
+            const float a1 = MT ? lj1[tp] : c1, a2 = MT ? lj2[tp] : c2;
+            float fpair = r6i * (a1 * r6i - a2) * r2i;
+            fpair = in_cut(r2) ? fpair : 0.f;
             rx += dx * fpair; ry += dy * fpair; rz += dz * fpair;
             return;
         }
-        // mixed full list, one atom type, with energy and virial: branch-free
+        // full list, one atom type, with energy and virial: branch-free
         // as well (a zero force term zeroes the virial terms; the energy term
         // is selected)
-        if constexpr (!HALF && EV && !MT && PREC == MD_PREC_MIXED) {
-            const real r2i = Pol<PREC>::rcp(r2);
-            const real r6i = r2i * r2i * r2i;
+        if constexpr (!HALF && EV && !MT) {
+            const float r2i = rcp32(r2);
+            const float r6i = r2i * r2i * r2i;
             const bool in = in_cut(r2);
-            const real fpair = in ? r6i * (c1 * r6i - c2) * r2i : (real)0;
-            const real fxp = dx * fpair, fyp = dy * fpair, fzp = dz * fpair;
+            const float fpair = in ? r6i * (c1 * r6i - c2) * r2i : 0.f;
+            const float fxp = dx * fpair, fyp = dy * fpair, fzp = dz * fpair;
             rx += fxp; ry += fyp; rz += fzp;
-            const real h = (real)0.5;
-            add_ev(in ? h * (r6i * (c3 * r6i - c4) - c0) : (real)0, h * dx * fxp, h * dy * fyp, h * dz * fzp,
+            const float h = 0.5f;
+            add_ev(in ? h * (r6i * (c3 * r6i - c4) - c0) : 0.f, h * dx * fxp, h * dy * fyp, h * dz * fzp,
                    h * dx * fyp, h * dx * fzp, h * dy * fzp);
             return;
         }
         if (in_cut(r2)) {
             const int tp = MT ? ti * nt + tj : 0;
-            const real r2i = Pol<PREC>::rcp(r2);
-            const real r6i = r2i * r2i * r2i;
-            const real a1 = MT ? lj1[tp] : c1, a2 = MT ? lj2[tp] : c2;
-            const real fpair = r6i * (a1 * r6i - a2) * r2i;
-            const real fxp = dx * fpair, fyp = dy * fpair, fzp = dz * fpair;
+            const float r2i = rcp32(r2);
+            const float r6i = r2i * r2i * r2i;
+            const float a1 = MT ? lj1[tp] : c1, a2 = MT ? lj2[tp] : c2;
+            const float fpair = r6i * (a1 * r6i - a2) * r2i;
+            const float fxp = dx * fpair, fyp = dy * fpair, fzp = dz * fpair;
             rx += fxp; ry += fyp; rz += fzp;
             if (HALF) {
                 const int j = entry_j(ent);
@@ -340,8 +283,8 @@ struct LJPair {
                 atomicAdd(&V->f[2 * n + j], -(double)fzp);
             }
             if (EV) {
-                const real wgt = HALF ? (real)1 : (real)0.5;
-                const real a3 = MT ? lj3[tp] : c3, a4 = MT ? lj4[tp] : c4, a0 = MT ? off[tp] : c0;
+                const float wgt = HALF ? 1.f : 0.5f;
+                const float a3 = MT ? lj3[tp] : c3, a4 = MT ? lj4[tp] : c4, a0 = MT ? off[tp] : c0;
                 add_ev(wgt * (r6i * (a3 * r6i - a4) - a0), wgt * dx * fxp, wgt * dy * fyp,
                        wgt * dz * fzp, wgt * dx * fyp, wgt * dx * fzp, wgt * dy * fzp);
             }
@@ -358,7 +301,7 @@ struct LJPair {
 // partner, energy and virial alike.  The terms are summed over the warp into
 // the atom's first thread.  All 32 lanes call this together.
 template <int T, int Q, int MT, int HALF, int EV>
-__device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MD_PREC_MIXED, MT, HALF, EV> &pr, bool flagged,
+__device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV> &pr, bool flagged,
                                               int gw, int lane, int tmode, const float4 *srec) {
     constexpr int A = 32 / T;
     unsigned m = __ballot_sync(0xffffffffu, flagged);
@@ -370,7 +313,7 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MD_PREC_MIXE
         const int cnt = V.ncount[p];
         float xi, yi, zi;
         int ti;
-        Pol<MD_PREC_MIXED>::load(V, p, xi, yi, zi, ti);
+        load_rec(V, p, xi, yi, zi, ti);
         const float hx = R.hf[0], hy4 = R.hf[1] * 0.25f, hz16 = R.hf[2] * 0.0625f;
         const uint32_t *base = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + a * T * Q;
         float cx = 0.f, cy = 0.f, cz = 0.f, ce = 0.f, cw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -382,7 +325,7 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MD_PREC_MIXE
                 const float4 r4 = srec[entry_j(e) & (kTileCap - 1)];
                 xj = r4.x; yj = r4.y; zj = r4.z; tj = __float_as_int(r4.w);
             } else {
-                Pol<MD_PREC_MIXED>::load(V, entry_j(e), xj, yj, zj, tj);
+                load_rec(V, entry_j(e), xj, yj, zj, tj);
             }
             const float dx = fmaf(-code_x(e), hx, xi - xj);
             const float dy = fmaf(-code_y4(e), hy4, yi - yj);
@@ -394,7 +337,7 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MD_PREC_MIXE
             if (exact == (t < 0.f)) continue;
             const float sgn = exact ? 1.f : -1.f;
             const int tp = MT ? ti * pr.nt + tj : 0;
-            const float r2i = Pol<MD_PREC_MIXED>::rcp(r2);
+            const float r2i = rcp32(r2);
             const float r6i = r2i * r2i * r2i;
             const float a1 = MT ? pr.lj1[tp] : pr.c1, a2 = MT ? pr.lj2[tp] : pr.c2;
             const float fpair = sgn * r6i * (a1 * r6i - a2) * r2i;
@@ -436,22 +379,18 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MD_PREC_MIXE
 // registers per thread allowed to the mixed force-only pass: 56 keeps nine
 // 128-thread blocks (36 warps) resident per SM to hide the gather latency;
 // groups of 8+ threads and half lists with 4-entry loads take 64 (no spills);
-// the mixed full-list energy/virial pass 80 (six blocks instead of five, no
+// the full-list energy/virial pass 80 (six blocks instead of five, no
 // spills: 0.39 -> 0.37 ms per md_energy_virial on the 864,000-atom liquid);
-// FP64 and the half-list energy pass what they need
-template <int PREC, int T, int Q, int HALF, int EV>
+// the half-list energy pass what it needs
+template <int T, int Q, int HALF, int EV>
 struct LjRegs {
-    static constexpr int value =
-        (PREC == MD_PREC_MIXED && !EV) ? (Q == 4 && (T > 4 || HALF) ? 64 : 56)
-                                       : ((PREC == MD_PREC_MIXED && !HALF) ? 80 : 255);
+    static constexpr int value = !EV ? (Q == 4 && (T > 4 || HALF) ? 64 : 56) : (!HALF ? 80 : 255);
 };
 
-template <int PREC, int T, int Q, int HALF, int EV, int MT>
-__global__ void __maxnreg__((LjRegs<PREC, T, Q, HALF, EV>::value)) k_lj(View V, KArgs a) {
-    using P = Pol<PREC>;
-    using real = typename P::real;
-    __shared__ real s_lj1[kMaxTypes * kMaxTypes], s_lj2[kMaxTypes * kMaxTypes];
-    __shared__ real s_lj3[kMaxTypes * kMaxTypes], s_lj4[kMaxTypes * kMaxTypes], s_off[kMaxTypes * kMaxTypes];
+template <int T, int Q, int HALF, int EV, int MT>
+__global__ void __maxnreg__((LjRegs<T, Q, HALF, EV>::value)) k_lj(View V, KArgs a) {
+    __shared__ float s_lj1[kMaxTypes * kMaxTypes], s_lj2[kMaxTypes * kMaxTypes];
+    __shared__ float s_lj3[kMaxTypes * kMaxTypes], s_lj4[kMaxTypes * kMaxTypes], s_off[kMaxTypes * kMaxTypes];
     __shared__ double s_ftm_sh[kMaxTypes];
     // one atom type: no table to stage, so no block barrier either (unless
     // the block stages records); the coefficients and ftm2v/m are read into
@@ -461,17 +400,12 @@ __global__ void __maxnreg__((LjRegs<PREC, T, Q, HALF, EV>::value)) k_lj(View V, 
     const double *s_ftm = kRegOnly ? V.tab->ftm_m : s_ftm_sh;
     const int np = kRegOnly ? 0 : V.ntypes * V.ntypes;
     for (int k = threadIdx.x; k < np; k += blockDim.x) {
-        if (PREC == MD_PREC_FP64) {
-            s_lj1[k] = V.tab->lj1[k]; s_lj2[k] = V.tab->lj2[k];
-            s_lj3[k] = V.tab->lj3[k]; s_lj4[k] = V.tab->lj4[k]; s_off[k] = V.tab->off[k];
-        } else {
-            s_lj1[k] = V.tab->lj1f[k]; s_lj2[k] = V.tab->lj2f[k];
-            s_lj3[k] = V.tab->lj3f[k]; s_lj4[k] = V.tab->lj4f[k]; s_off[k] = V.tab->offf[k];
-        }
+        s_lj1[k] = V.tab->lj1f[k]; s_lj2[k] = V.tab->lj2f[k];
+        s_lj3[k] = V.tab->lj3f[k]; s_lj4[k] = V.tab->lj4f[k]; s_off[k] = V.tab->offf[k];
     }
     if (!kRegOnly && threadIdx.x < kMaxTypes) s_ftm_sh[threadIdx.x] = V.tab->ftm_m[threadIdx.x];
     extern __shared__ float4 s_rec[];
-    const int tmode = HALF ? 0 : begin_tile<PREC>(V, T, s_rec);
+    const int tmode = HALF ? 0 : begin_tile(V, T, s_rec);
     if (!kRegOnly || V.tile_atoms != 0) __syncthreads();
 
     const unsigned err = V.ctl->err;
@@ -483,25 +417,25 @@ __global__ void __maxnreg__((LjRegs<PREC, T, Q, HALF, EV>::value)) k_lj(View V, 
     const int sub = lane & (T - 1);
     const bool warp_in = (gw * A < V.n_pad) && err == 0 && tmode >= 0;
 
-    LJPair<PREC, MT, HALF, EV> pr;
+    LJPair<MT, HALF, EV> pr;
     pr.V = &V;
     pr.lj1 = s_lj1; pr.lj2 = s_lj2; pr.lj3 = s_lj3; pr.lj4 = s_lj4; pr.off = s_off;
     if (kRegOnly) {
-        pr.c1 = (PREC == MD_PREC_FP64) ? (real)V.tab->lj1[0] : (real)V.tab->lj1f[0];
-        pr.c2 = (PREC == MD_PREC_FP64) ? (real)V.tab->lj2[0] : (real)V.tab->lj2f[0];
+        pr.c1 = V.tab->lj1f[0];
+        pr.c2 = V.tab->lj2f[0];
         if (EV) {
-            pr.c3 = (PREC == MD_PREC_FP64) ? (real)V.tab->lj3[0] : (real)V.tab->lj3f[0];
-            pr.c4 = (PREC == MD_PREC_FP64) ? (real)V.tab->lj4[0] : (real)V.tab->lj4f[0];
-            pr.c0 = (PREC == MD_PREC_FP64) ? (real)V.tab->off[0] : (real)V.tab->offf[0];
+            pr.c3 = V.tab->lj3f[0];
+            pr.c4 = V.tab->lj4f[0];
+            pr.c0 = V.tab->offf[0];
         }
     } else {
         pr.c1 = s_lj1[0]; pr.c2 = s_lj2[0];
     }
-    pr.rc2 = (PREC == MD_PREC_FP64) ? (real)V.rc2 : (real)V.rc2f;
+    pr.rc2 = V.rc2f;
     pr.nt = V.ntypes;
     pr.n = V.n_pad;
     pr.ti = 0;
-    pr.near_min = (real)3.0e38;
+    pr.near_min = 3.0e38f;
     pr.ax.zero(); pr.ay.zero(); pr.az.zero(); pr.e.zero();
     for (int k = 0; k < 6; ++k) pr.w[k].zero();
     bool valid = false;
@@ -510,12 +444,12 @@ __global__ void __maxnreg__((LjRegs<PREC, T, Q, HALF, EV>::value)) k_lj(View V, 
         valid = (p - R.atom0) < R.natoms;
         if (valid) {
             const int cnt = V.ncount[p];
-            real xi, yi, zi;
-            P::load(V, p, xi, yi, zi, pr.ti);
+            float xi, yi, zi;
+            load_rec(V, p, xi, yi, zi, pr.ti);
             const uint32_t *lp = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + lane * Q;
-            walk_mode<PREC, T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
+            walk_mode<T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
         }
-        if constexpr (PREC == MD_PREC_MIXED) fix_near_warp<T, Q>(V, pr, pr.near_min < V.rc2f_band, gw, lane, tmode, s_rec);
+        fix_near_warp<T, Q>(V, pr, pr.near_min < V.rc2f_band, gw, lane, tmode, s_rec);
     }
     const double fx = group_sum<T>(pr.ax.value());
     const double fy = group_sum<T>(pr.ay.value());
@@ -553,20 +487,19 @@ __global__ void __maxnreg__((LjRegs<PREC, T, Q, HALF, EV>::value)) k_lj(View V, 
 // cells' records from global memory.  Forces only (no energy/virial).
 template <int MT>
 __global__ void __launch_bounds__(128) k_lj_cells(View V, KArgs a) {
-    using P = Pol<MD_PREC_MIXED>;
     __shared__ float s_lj1[kMaxTypes * kMaxTypes], s_lj2[kMaxTypes * kMaxTypes];
     __shared__ double s_ftm[kMaxTypes];
     const int np = V.ntypes * V.ntypes;
     for (int k = threadIdx.x; k < np; k += blockDim.x) { s_lj1[k] = V.tab->lj1f[k]; s_lj2[k] = V.tab->lj2f[k]; }
     if (threadIdx.x < kMaxTypes) s_ftm[threadIdx.x] = V.tab->ftm_m[threadIdx.x];
     extern __shared__ float4 s_rec[];
-    const int tmode = begin_tile<MD_PREC_MIXED>(V, 1, s_rec);
+    const int tmode = begin_tile(V, 1, s_rec);
     __syncthreads();
     const unsigned err = V.ctl->err;
     const int rem = (a.mode == kModeStep) ? V.ctl->remaining : 0;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     const int t = blockIdx.x;
-    LJPair<MD_PREC_MIXED, MT, 0, 0> pr;
+    LJPair<MT, 0, 0> pr;
     pr.V = &V;
     pr.lj1 = s_lj1; pr.lj2 = s_lj2;
     pr.c1 = s_lj1[0]; pr.c2 = s_lj2[0];
@@ -582,7 +515,7 @@ __global__ void __launch_bounds__(128) k_lj_cells(View V, KArgs a) {
         valid = (p - R.atom0) < R.natoms;
         if (valid) {
             float xi, yi, zi;
-            P::load(V, p, xi, yi, zi, pr.ti);
+            load_rec(V, p, xi, yi, zi, pr.ti);
             const int bk = V.bpk[p];
             const int bx = unpack_bx(bk), by = unpack_by(bk), bz = unpack_bz(bk);
             const int nbx = R.nb[0], nby = R.nb[1], nbz = R.nb[2];
@@ -653,9 +586,8 @@ struct GatherPair {
 
 template <int T, int Q>
 __global__ void __launch_bounds__(256, 4) k_gather_probe(View V, KArgs a) {
-    using P = Pol<MD_PREC_MIXED>;
     extern __shared__ float4 s_rec[];
-    const int tmode = begin_tile<MD_PREC_MIXED>(V, T, s_rec);
+    const int tmode = begin_tile(V, T, s_rec);
     __syncthreads();
     constexpr int A = 32 / T;
     const int lane = threadIdx.x & 31;
@@ -672,9 +604,9 @@ __global__ void __launch_bounds__(256, 4) k_gather_probe(View V, KArgs a) {
             const int cnt = V.ncount[p];
             float xi, yi, zi;
             int ti;
-            P::load(V, p, xi, yi, zi, ti);
+            load_rec(V, p, xi, yi, zi, ti);
             const uint32_t *lp = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + lane * Q;
-            walk_mode<MD_PREC_MIXED, T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
+            walk_mode<T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
         }
     }
     const double sum = group_sum<T>((double)pr.acc);
@@ -748,34 +680,22 @@ __global__ void k_kick(View V, KArgs a) {
 
 // pass 1: host density rho_i = sum_j (rc - r)^2 and the embedding derivative
 // F'(rho_i) = -A / (2 sqrt(rho_i)) (0 at rho = 0), FP64 per atom
-template <int PREC>
 struct RhoPair {
-    using real = typename Pol<PREC>::real;
-    typename Pol<PREC>::Acc acc;
-    real rc, rc2, part;
+    KahanF acc;
+    float rc, rc2, part;
     __device__ __forceinline__ void round_begin() { part = 0; }
     __device__ __forceinline__ void round_end() { acc.add(part); }
-    __device__ __forceinline__ void operator()(uint32_t, real, real, real, real r2, int) {
-        if constexpr (PREC == MD_PREC_MIXED) {  // branch-free: t = 0 beyond rc
-            const real r = r2 * Pol<PREC>::rsqrt(r2);
-            const real t = (r2 < rc2) ? rc - r : (real)0;
-            part += t * t;
-            return;
-        }
-        if (r2 < rc2) {
-            const real r = r2 * Pol<PREC>::rsqrt(r2);
-            const real t = rc - r;
-            part += t * t;
-        }
+    __device__ __forceinline__ void operator()(uint32_t, float, float, float, float r2, int) {
+        const float r = r2 * rsqrtf(r2);  // branch-free: t = 0 beyond rc
+        const float t = (r2 < rc2) ? rc - r : 0.f;
+        part += t * t;
     }
 };
 
-template <int PREC, int T, int Q>
+template <int T, int Q>
 __global__ void __launch_bounds__(256) k_eam_rho(View V, KArgs a) {
-    using P = Pol<PREC>;
-    using real = typename P::real;
     extern __shared__ float4 s_rec[];
-    const int tmode = begin_tile<PREC>(V, T, s_rec);
+    const int tmode = begin_tile(V, T, s_rec);
     if (V.tile_atoms != 0) __syncthreads();  // only a staging block has shared state
     const unsigned err = V.ctl->err;
     constexpr int A = 32 / T;
@@ -783,121 +703,101 @@ __global__ void __launch_bounds__(256) k_eam_rho(View V, KArgs a) {
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int p = gw * A + lane / T;
     const int sub = lane & (T - 1);
-    RhoPair<PREC> pr;
+    RhoPair pr;
     pr.acc.zero();
-    pr.rc = (PREC == MD_PREC_FP64) ? (real)V.tab->eam[0] : (real)V.tab->eamf[0];
-    pr.rc2 = (PREC == MD_PREC_FP64) ? (real)V.rc2 : (real)V.rc2f;
+    pr.rc = V.tab->eamf[0];
+    pr.rc2 = V.rc2f;
     bool valid = false;
     if (gw * A < V.n_pad && err == 0 && tmode >= 0) {
         const Rep &R = V.rep[V.tile_rep[p >> 5]];
         valid = (p - R.atom0) < R.natoms;
         if (valid) {
             const int cnt = V.ncount[p];
-            real xi, yi, zi;
+            float xi, yi, zi;
             int ti;
-            P::load(V, p, xi, yi, zi, ti);
+            load_rec(V, p, xi, yi, zi, ti);
             const uint32_t *lp = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + lane * Q;
-            walk_mode<PREC, T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
+            walk_mode<T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
         }
     }
     const double rho = group_sum<T>(pr.acc.value());
     if (valid && sub == 0) {
         const double Aemb = V.tab->eam[1];
-        if (PREC == MD_PREC_FP64) {
-            const double sr = sqrt(rho);
-            V.fp64[p] = rho > 0.0 ? -0.5 * Aemb / sr : 0.0;
-        } else {
-            // single element: the record's type slot is free until the next drift
-            // rewrites it, so F'(rho) rides in rec.w and the force pass gathers
-            // one 16-byte record per pair instead of two separate loads.  It is
-            // stored as FP32, so it is formed in FP32 (one reciprocal square
-            // root, a few FP32 ulps) rather than by an FP64 square root and
-            // divide on the FP64 pipe for every atom
-            const float rf = (float)rho;
-            V.rec[p].w = rf > 0.f ? -0.5f * (float)Aemb * rsqrtf(rf) : 0.f;
-        }
+        // single element: the record's type slot is free until the next drift
+        // rewrites it, so F'(rho) rides in rec.w and the force pass gathers
+        // one 16-byte record per pair instead of two separate loads.  It is
+        // stored as FP32, so it is formed in FP32 (one reciprocal square
+        // root, a few FP32 ulps) rather than by an FP64 square root and
+        // divide on the FP64 pipe for every atom
+        const float rf = (float)rho;
+        V.rec[p].w = rf > 0.f ? -0.5f * (float)Aemb * rsqrtf(rf) : 0.f;
         if (a.mode == kModeEV) V.emb[p] = rho > 0.0 ? -Aemb * sqrt(rho) : 0.0;
     }
 }
 
 // pass 2: F_i = -sum_j [phi'(r) + (F'_i + F'_j) rho'(r)] d / r
-template <int PREC, int EV>
+template <int EV>
 struct EamPair {
-    using real = typename Pol<PREC>::real;
-    using Acc = typename Pol<PREC>::Acc;
-    const View *V;
-    real rc, rc2, c0, c1, c2, fpi;
-    Acc ax, ay, az, e;
-    Acc w[6];
-    real rx, ry, rz;  // this round's plain partial sums
-    real re, rw[6];   // and of the energy and virial terms (EV)
+    float rc, rc2, c0, c1, c2, fpi;
+    KahanF ax, ay, az, e;
+    KahanF w[6];
+    float rx, ry, rz;  // this round's plain partial sums
+    float re, rw[6];   // and of the energy and virial terms (EV)
     __device__ __forceinline__ void round_begin() {
         rx = 0; ry = 0; rz = 0;
-        if (EV && PREC == MD_PREC_MIXED) {
+        if (EV) {
             re = 0;
             for (int k = 0; k < 6; ++k) rw[k] = 0;
         }
     }
     __device__ __forceinline__ void round_end() {
         ax.add(rx); ay.add(ry); az.add(rz);
-        if (EV && PREC == MD_PREC_MIXED) {
+        if (EV) {
             e.add(re);
             for (int k = 0; k < 6; ++k) w[k].add(rw[k]);
         }
     }
-    // energy and virial terms of one pair: summed plainly over the round and
-    // added with compensation per round (mixed), or added directly (FP64)
-    __device__ __forceinline__ void add_ev(real ee, real w0, real w1, real w2, real w3, real w4, real w5) {
-        if constexpr (PREC == MD_PREC_MIXED) {
-            re += ee;
-            rw[0] += w0; rw[1] += w1; rw[2] += w2; rw[3] += w3; rw[4] += w4; rw[5] += w5;
-        } else {
-            e.add(ee);
-            w[0].add(w0); w[1].add(w1); w[2].add(w2); w[3].add(w3); w[4].add(w4); w[5].add(w5);
-        }
-    }
-    __device__ __forceinline__ void operator()(uint32_t ent, real dx, real dy, real dz, real r2, int wj) {
-        if constexpr (PREC == MD_PREC_MIXED && !EV) {  // branch-free: t = 0 beyond rc zeroes the term
-            const real fpj = (real)__int_as_float(wj);
-            const real rinv = Pol<PREC>::rsqrt(r2);
-            const real r = r2 * rinv;
-            const real t = (r2 < rc2) ? rc - r : (real)0;
-            const real poly = c0 + r * (c1 + r * c2);
-            const real dpoly = c1 + (real)2 * c2 * r;
-            const real coef = -t * ((real)-2 * poly + t * dpoly - (real)2 * (fpi + fpj)) * rinv;
+    // wj: F'_j, which came with the record (rec.w, set by the density pass)
+    __device__ __forceinline__ void operator()(uint32_t, float dx, float dy, float dz, float r2, int wj) {
+        if constexpr (!EV) {  // branch-free: t = 0 beyond rc zeroes the term
+            const float fpj = __int_as_float(wj);
+            const float rinv = rsqrtf(r2);
+            const float r = r2 * rinv;
+            const float t = (r2 < rc2) ? rc - r : 0.f;
+            const float poly = c0 + r * (c1 + r * c2);
+            const float dpoly = c1 + 2.f * c2 * r;
+            const float coef = -t * (-2.f * poly + t * dpoly - 2.f * (fpi + fpj)) * rinv;
             rx += dx * coef; ry += dy * coef; rz += dz * coef;
             return;
         }
         if (r2 < rc2) {
-            // mixed: F'_j came with the record (rec.w, set by the density pass)
-            const real fpj = (PREC == MD_PREC_FP64) ? Pol<PREC>::fp(*V, entry_j(ent)) : (real)__int_as_float(wj);
-            const real rinv = Pol<PREC>::rsqrt(r2);
-            const real r = r2 * rinv;
-            const real t = rc - r;
-            const real poly = c0 + r * (c1 + r * c2);
-            const real dpoly = c1 + (real)2 * c2 * r;
+            const float fpj = __int_as_float(wj);
+            const float rinv = rsqrtf(r2);
+            const float r = r2 * rinv;
+            const float t = rc - r;
+            const float poly = c0 + r * (c1 + r * c2);
+            const float dpoly = c1 + 2.f * c2 * r;
             // -(phi' + (F'_i + F'_j) rho') / r with phi' = -2t poly + t^2 dpoly, rho' = -2t
-            const real coef = -t * ((real)-2 * poly + t * dpoly - (real)2 * (fpi + fpj)) * rinv;
-            const real fxp = dx * coef, fyp = dy * coef, fzp = dz * coef;
+            const float coef = -t * (-2.f * poly + t * dpoly - 2.f * (fpi + fpj)) * rinv;
+            const float fxp = dx * coef, fyp = dy * coef, fzp = dz * coef;
             rx += fxp; ry += fyp; rz += fzp;
             if (EV) {
-                const real h = (real)0.5;
-                add_ev(h * t * t * poly, h * dx * fxp, h * dy * fyp, h * dz * fzp, h * dx * fyp, h * dx * fzp,
-                       h * dy * fzp);
+                const float h = 0.5f;
+                re += h * t * t * poly;
+                rw[0] += h * dx * fxp; rw[1] += h * dy * fyp; rw[2] += h * dz * fzp;
+                rw[3] += h * dx * fyp; rw[4] += h * dx * fzp; rw[5] += h * dy * fzp;
             }
         }
     }
 };
 
-template <int PREC, int T, int Q, int EV>
+template <int T, int Q, int EV>
 __global__ void __launch_bounds__(256) k_eam_force(View V, KArgs a) {
-    using P = Pol<PREC>;
-    using real = typename P::real;
     // single element: ftm2v/m is read where it is used, no table to stage, so
     // no block barrier either unless the block stages records
     const double *s_ftm = V.tab->ftm_m;
     extern __shared__ float4 s_rec[];
-    const int tmode = begin_tile<PREC>(V, T, s_rec);
+    const int tmode = begin_tile(V, T, s_rec);
     if (V.tile_atoms != 0) __syncthreads();
     const unsigned err = V.ctl->err;
     const int rem = (a.mode == kModeStep) ? V.ctl->remaining : 0;
@@ -906,14 +806,9 @@ __global__ void __launch_bounds__(256) k_eam_force(View V, KArgs a) {
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int p = gw * A + lane / T;
     const int sub = lane & (T - 1);
-    EamPair<PREC, EV> pr;
-    pr.V = &V;
-    if (PREC == MD_PREC_FP64) {
-        pr.rc = V.tab->eam[0]; pr.c0 = V.tab->eam[2]; pr.c1 = V.tab->eam[3]; pr.c2 = V.tab->eam[4];
-    } else {
-        pr.rc = V.tab->eamf[0]; pr.c0 = V.tab->eamf[2]; pr.c1 = V.tab->eamf[3]; pr.c2 = V.tab->eamf[4];
-    }
-    pr.rc2 = (PREC == MD_PREC_FP64) ? (real)V.rc2 : (real)V.rc2f;
+    EamPair<EV> pr;
+    pr.rc = V.tab->eamf[0]; pr.c0 = V.tab->eamf[2]; pr.c1 = V.tab->eamf[3]; pr.c2 = V.tab->eamf[4];
+    pr.rc2 = V.rc2f;
     pr.fpi = 0;
     pr.ax.zero(); pr.ay.zero(); pr.az.zero(); pr.e.zero();
     for (int k = 0; k < 6; ++k) pr.w[k].zero();
@@ -924,11 +819,11 @@ __global__ void __launch_bounds__(256) k_eam_force(View V, KArgs a) {
         valid = (p - R.atom0) < R.natoms;
         if (valid) {
             const int cnt = V.ncount[p];
-            real xi, yi, zi;
-            P::load(V, p, xi, yi, zi, ti);
-            pr.fpi = (PREC == MD_PREC_FP64) ? P::fp(V, p) : (real)__int_as_float(ti);
+            float xi, yi, zi;
+            load_rec(V, p, xi, yi, zi, ti);
+            pr.fpi = __int_as_float(ti);
             const uint32_t *lp = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + lane * Q;
-            walk_mode<PREC, T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
+            walk_mode<T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
         }
     }
     const double fx = group_sum<T>(pr.ax.value());
@@ -940,8 +835,8 @@ __global__ void __launch_bounds__(256) k_eam_force(View V, KArgs a) {
         for (int k = 0; k < 6; ++k) w_acc[k] = group_sum<T>(pr.w[k].value());
     }
     if (valid && sub == 0) {
-        // single element (checked at creation): type 0 for the mass; in the mixed
-        // path the loaded record's .w holds F'(rho), not a type
+        // single element (checked at creation): type 0 for the mass; the loaded
+        // record's .w holds F'(rho), not a type
         epilogue(V, a.mode, rem, p, 0, fx, fy, fz, s_ftm);
         if (EV) write_ev(V, p, 0, e_acc + V.emb[p], w_acc, s_ftm);
     }
@@ -988,8 +883,8 @@ __device__ __forceinline__ float drift_one(const View &V, int p, int first, int 
         V.pos4[p] = make_double4_32a(x[0], x[1], x[2], __longlong_as_double((long long)t));
     } else {
         for (int c = 0; c < 3; ++c) V.xr[c * n + p] = x[c];
-        V.rec[p] = nr;
     }
+    V.rec[p] = nr;  // FP64: the records that the force passes test first
     const float ex = nr.x - b.x, ey = nr.y - b.y, ez = nr.z - b.z;
     float d2 = ex * ex + ey * ey + ez * ez;
     if (!(d2 <= 3.0e38f)) d2 = __int_as_float(0x7f800000);  // NaN/Inf -> +Inf
@@ -1142,105 +1037,100 @@ __global__ void k_loop_init(View V, KArgs a) {
 
 // ------------------------------------------------------------- dispatch ----
 
-template <int PREC, int Q, int HALF, int EV, int MT>
+template <int Q, int HALF, int EV, int MT>
 static const void *pick_lj_t(int T) {
     switch (T) {
-        case 1: return (const void *)k_lj<PREC, 1, Q, HALF, EV, MT>;
-        case 2: return (const void *)k_lj<PREC, 2, Q, HALF, EV, MT>;
-        case 4: return (const void *)k_lj<PREC, 4, Q, HALF, EV, MT>;
-        case 8: return (const void *)k_lj<PREC, 8, Q, HALF, EV, MT>;
-        case 16: return (const void *)k_lj<PREC, 16, Q, HALF, EV, MT>;
-        default: return (const void *)k_lj<PREC, 32, Q, HALF, EV, MT>;
+        case 1: return (const void *)k_lj<1, Q, HALF, EV, MT>;
+        case 2: return (const void *)k_lj<2, Q, HALF, EV, MT>;
+        case 4: return (const void *)k_lj<4, Q, HALF, EV, MT>;
+        case 8: return (const void *)k_lj<8, Q, HALF, EV, MT>;
+        case 16: return (const void *)k_lj<16, Q, HALF, EV, MT>;
+        default: return (const void *)k_lj<32, Q, HALF, EV, MT>;
     }
 }
 
-template <int PREC, int Q>
+template <int Q>
 static const void *pick_lj_q(int T, int half, int ev, int mt) {
     if (half) {
-        if (ev) return mt ? pick_lj_t<PREC, Q, 1, 1, 1>(T) : pick_lj_t<PREC, Q, 1, 1, 0>(T);
-        return mt ? pick_lj_t<PREC, Q, 1, 0, 1>(T) : pick_lj_t<PREC, Q, 1, 0, 0>(T);
+        if (ev) return mt ? pick_lj_t<Q, 1, 1, 1>(T) : pick_lj_t<Q, 1, 1, 0>(T);
+        return mt ? pick_lj_t<Q, 1, 0, 1>(T) : pick_lj_t<Q, 1, 0, 0>(T);
     }
-    if (ev) return mt ? pick_lj_t<PREC, Q, 0, 1, 1>(T) : pick_lj_t<PREC, Q, 0, 1, 0>(T);
-    return mt ? pick_lj_t<PREC, Q, 0, 0, 1>(T) : pick_lj_t<PREC, Q, 0, 0, 0>(T);
+    if (ev) return mt ? pick_lj_t<Q, 0, 1, 1>(T) : pick_lj_t<Q, 0, 1, 0>(T);
+    return mt ? pick_lj_t<Q, 0, 0, 1>(T) : pick_lj_t<Q, 0, 0, 0>(T);
 }
 
-template <int PREC>
-static const void *pick_lj_prec(int T, int Q, int half, int ev, int mt) {
-    if (Q == 4) return pick_lj_q<PREC, 4>(T, half, ev, mt);
-    if (Q == 2) return pick_lj_q<PREC, 2>(T, half, ev, mt);
-    return pick_lj_q<PREC, 1>(T, half, ev, mt);
+static const void *pick_lj(int T, int Q, int half, int ev, int mt) {
+    if (Q == 4) return pick_lj_q<4>(T, half, ev, mt);
+    if (Q == 2) return pick_lj_q<2>(T, half, ev, mt);
+    return pick_lj_q<1>(T, half, ev, mt);
 }
 
-template <int PREC, int Q>
+template <int Q>
 static const void *pick_rho_q(int T) {
     switch (T) {
-        case 1: return (const void *)k_eam_rho<PREC, 1, Q>;
-        case 2: return (const void *)k_eam_rho<PREC, 2, Q>;
-        case 4: return (const void *)k_eam_rho<PREC, 4, Q>;
-        case 8: return (const void *)k_eam_rho<PREC, 8, Q>;
-        case 16: return (const void *)k_eam_rho<PREC, 16, Q>;
-        default: return (const void *)k_eam_rho<PREC, 32, Q>;
+        case 1: return (const void *)k_eam_rho<1, Q>;
+        case 2: return (const void *)k_eam_rho<2, Q>;
+        case 4: return (const void *)k_eam_rho<4, Q>;
+        case 8: return (const void *)k_eam_rho<8, Q>;
+        case 16: return (const void *)k_eam_rho<16, Q>;
+        default: return (const void *)k_eam_rho<32, Q>;
     }
 }
 
-template <int PREC>
 static const void *pick_rho(int T, int Q) {
-    if (Q == 4) return pick_rho_q<PREC, 4>(T);
-    if (Q == 2) return pick_rho_q<PREC, 2>(T);
-    return pick_rho_q<PREC, 1>(T);
+    if (Q == 4) return pick_rho_q<4>(T);
+    if (Q == 2) return pick_rho_q<2>(T);
+    return pick_rho_q<1>(T);
 }
 
-template <int PREC, int Q, int EV>
+template <int Q, int EV>
 static const void *pick_eamf_q(int T) {
     switch (T) {
-        case 1: return (const void *)k_eam_force<PREC, 1, Q, EV>;
-        case 2: return (const void *)k_eam_force<PREC, 2, Q, EV>;
-        case 4: return (const void *)k_eam_force<PREC, 4, Q, EV>;
-        case 8: return (const void *)k_eam_force<PREC, 8, Q, EV>;
-        case 16: return (const void *)k_eam_force<PREC, 16, Q, EV>;
-        default: return (const void *)k_eam_force<PREC, 32, Q, EV>;
+        case 1: return (const void *)k_eam_force<1, Q, EV>;
+        case 2: return (const void *)k_eam_force<2, Q, EV>;
+        case 4: return (const void *)k_eam_force<4, Q, EV>;
+        case 8: return (const void *)k_eam_force<8, Q, EV>;
+        case 16: return (const void *)k_eam_force<16, Q, EV>;
+        default: return (const void *)k_eam_force<32, Q, EV>;
     }
 }
 
-template <int PREC>
 static const void *pick_eamf(int T, int Q, int ev) {
-    if (Q == 4) return ev ? pick_eamf_q<PREC, 4, 1>(T) : pick_eamf_q<PREC, 4, 0>(T);
-    if (Q == 2) return ev ? pick_eamf_q<PREC, 2, 1>(T) : pick_eamf_q<PREC, 2, 0>(T);
-    return ev ? pick_eamf_q<PREC, 1, 1>(T) : pick_eamf_q<PREC, 1, 0>(T);
+    if (Q == 4) return ev ? pick_eamf_q<4, 1>(T) : pick_eamf_q<4, 0>(T);
+    if (Q == 2) return ev ? pick_eamf_q<2, 1>(T) : pick_eamf_q<2, 0>(T);
+    return ev ? pick_eamf_q<1, 1>(T) : pick_eamf_q<1, 0>(T);
+}
+
+// the pair passes of one precision: [LJ pass], or [density, force] for EAM
+static void mixed_force_sequence(const View &V, int mode, int block, KArgs a, std::vector<KCall> &seq) {
+    const int T = V.tpa;
+    const int ev = (mode == kModeEV) ? 1 : 0;
+    const long long threads = (long long)V.n_pad * T;
+    const dim3 grid((unsigned)((threads + block - 1) / block));
+    const size_t sm = V.tile_atoms > 0 ? kTileSmem : 0;
+    if (V.pot == MD_POT_LJ) {
+        seq.push_back(KCall{pick_lj(T, V.vec, V.half, ev, V.ntypes > 1 ? 1 : 0), grid, dim3(block), sm, a});
+    } else {
+        KArgs ar = a;
+        ar.in_graph = 0;
+        seq.push_back(KCall{pick_rho(T, V.vec), grid, dim3(block), sm, ar});
+        seq.push_back(KCall{pick_eamf(T, V.vec, ev), grid, dim3(block), sm, a});
+    }
 }
 
 void force_sequence(const View &V, int mode, int block, bool in_graph, std::vector<KCall> &seq) {
     KArgs a{};
     a.mode = mode;
     a.in_graph = in_graph ? 1 : 0;
-    const int T = V.tpa;
-    const int ev = (mode == kModeEV) ? 1 : 0;
-    const long long threads = (long long)V.n_pad * T;
-    const dim3 grid((unsigned)((threads + block - 1) / block));
-    const int fp64 = (V.prec == MD_PREC_FP64);
-    const size_t sm = V.tile_atoms > 0 ? kTileSmem : 0;
-    if (V.pot == MD_POT_LJ) {
-        const int mt = V.ntypes > 1 ? 1 : 0;
-        const void *fn = fp64 ? pick_lj_prec<MD_PREC_FP64>(T, V.vec, V.half, ev, mt)
-                              : pick_lj_prec<MD_PREC_MIXED>(T, V.vec, V.half, ev, mt);
-        if (V.half) {
-            seq.push_back(KCall{(const void *)k_zero_f, dim3((3 * V.n_pad + 255) / 256), dim3(256), 0, a});
-            KArgs af = a;
-            af.mode = kModeStoreF;
-            af.in_graph = 0;
-            seq.push_back(KCall{fn, grid, dim3(block), 0, af});
-            seq.push_back(KCall{(const void *)k_kick, dim3((V.n_pad + 255) / 256), dim3(256), 0, a});
-        } else {
-            seq.push_back(KCall{fn, grid, dim3(block), sm, a});
-        }
-    } else {
-        KArgs ar = a;
-        ar.in_graph = 0;
-        const void *fr = fp64 ? pick_rho<MD_PREC_FP64>(T, V.vec) : pick_rho<MD_PREC_MIXED>(T, V.vec);
-        seq.push_back(KCall{fr, grid, dim3(block), sm, ar});
-        const void *fn = fp64 ? pick_eamf<MD_PREC_FP64>(T, V.vec, ev) : pick_eamf<MD_PREC_MIXED>(T, V.vec, ev);
-        seq.push_back(KCall{fn, grid, dim3(block), sm, a});
+    KArgs af = a;
+    if (V.half) {  // the kick and the closing store follow in k_kick, once F is complete
+        seq.push_back(KCall{(const void *)k_zero_f, dim3((3 * V.n_pad + 255) / 256), dim3(256), 0, a});
+        af.mode = kModeStoreF;
+        af.in_graph = 0;
     }
+    if (V.prec == MD_PREC_FP64) fp64_force_sequence(V, mode, af, seq);
+    else mixed_force_sequence(V, mode, block, af, seq);
+    if (V.half) seq.push_back(KCall{(const void *)k_kick, dim3((V.n_pad + 255) / 256), dim3(256), 0, a});
 }
 
 void drift_sequence(const View &V, bool in_graph, std::vector<KCall> &seq) {

@@ -145,7 +145,7 @@ struct View {
     double *ev;
     double *ev_tile;      // [n_tiles][8] per-tile partial sums
     // backward
-    double *gs, *gx;      // [3][n_pad] gradient in / out (sorted)
+    double4_32a *bpack;   // [n_pad][2] x, y, z, type | dL/dF, 0
     double *bw;           // [2][n_pad] EAM backward: F'(rho_i), mu_i = lambda_i F''(rho_i)
     double *gp_part;      // per block partial parameter gradients
     // block-local lists (tile_atoms = 0: every list entry holds a slot)
@@ -232,33 +232,43 @@ __device__ __forceinline__ float code_z16(uint32_t e) {
     return __int_as_float(0x4B400000u | (e & 0x30u)) - 12582928.0f;
 }
 
-// FP64 reciprocal by Newton-Raphson (y <- y (2 - x y), quadratic convergence)
-// from the FP32 hardware approximation (relative error < 2^-22, plus 2^-24
-// from rounding x to FP32): one step reaches ~2^-44, and the final step in
-// residual form, y + y (1 - x y) with fused multiply-adds, ~2^-88 before the
-// last rounding, i.e. double precision.  For 0 < x < FLT_MAX (squared
-// distances here).
-__device__ __forceinline__ double rcp_newton(double x) {
-    float xf = (float)x, yf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(xf));
-    double y = (double)yf;
-    y = y * fma(-x, y, 2.0);
-    const double e = fma(-x, y, 1.0);
-    return fma(y, e, y);
+// A positive double as float, truncated, and a float as double, by moving the
+// exponent and mantissa bits: integer instructions, where a conversion holds
+// the FP64 pipe for as long as an FP64 multiply.  For FLT_MIN <= x < FLT_MAX.
+__device__ __forceinline__ float narrow_bits(double x) {
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(x), (unsigned)__double2hiint(x) - 0x38000000u, 3));
+}
+__device__ __forceinline__ double widen_bits(float y) {
+    const unsigned b = __float_as_uint(y);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
-// FP64 reciprocal square root by Newton-Raphson (y <- y (3 - x y^2) / 2)
-// from the FP32 hardware approximation (relative error ~2^-22): the error
-// roughly squares per step (times 3/2), so two steps reach double precision
-// up to the last roundings.  For FLT_MIN < x < FLT_MAX.
-__device__ __forceinline__ double rsqrt_newton(double x) {
-    float xf = (float)x, yf;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(xf));
-    double y = (double)yf;
-    const double hx = 0.5 * x;
-    y = y * fma(-hx, y * y, 1.5);
-    y = y * fma(-hx, y * y, 1.5);
-    return y;
+// FP64 reciprocal and reciprocal square root from the FP32 hardware
+// approximations y0 (relative error < 2^-21, the truncation of x included) by
+// one third-order step each (the series of 1/(1 - e) and (1 - e)^-1/2 to e^2):
+//   1/x:       e = 1 - x y0,   y = y0 (1 + e + e^2)              error e^3
+//   x^-1/2:    e = 1 - x y0^2, y = y0 (1 + e/2 + 3 e^2 / 8)      error 5 e^3 / 16
+// both below 2^-62, so that only the last roundings are left; the residuals
+// are single fused multiply-adds of exact products (y0 has 24 bits).  3 and 5
+// FP64 instructions; the two-step Newton forms with conversions took 6 and 9.
+// For FLT_MIN <= x < FLT_MAX; below (x = 0 included) the result is NaN.
+__device__ __forceinline__ double seed64(float y0, double x) {
+    const double y = widen_bits(y0);
+    return __double2hiint(x) < 0x38100000 ? __hiloint2double(0x7ff80000, 0) : y;
+}
+__device__ __forceinline__ double rcp64(double x) {
+    float yf;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(narrow_bits(x)));
+    const double y = seed64(yf, x);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsqrt64(double x) {
+    float yf;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(narrow_bits(x)));
+    const double y = seed64(yf, x);
+    const double e = fma(-x, y * y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
 __device__ __forceinline__ float warp_max(float x) {

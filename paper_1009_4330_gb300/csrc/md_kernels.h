@@ -30,6 +30,10 @@ void drift_sequence(const View &V, bool in_graph, std::vector<KCall> &seq);
 // kModeEV).  `block` = threads per block.
 void force_sequence(const View &V, int mode, int block, bool in_graph, std::vector<KCall> &seq);
 
+// its FP64 pair passes ([LJ pass], or [density, force] for EAM); mode: as above,
+// a: the arguments of the launches (half lists: the mode of a pass that only stores)
+void fp64_force_sequence(const View &V, int mode, KArgs a, std::vector<KCall> &seq);
+
 // memory-only twin of the mixed full-list LJ force pass (see md_time_gather)
 void gather_probe_sequence(const View &V, int block, std::vector<KCall> &seq);
 // cell-list LJ force pass (no Verlet list) over the tiles of the last build
@@ -44,12 +48,13 @@ cudaError_t launch_stage_in(const View &V, int r, int natoms, const double *x, c
 cudaError_t launch_restage(const View &V, const double *x, const double *v, cudaStream_t s);
 cudaError_t launch_state_out(const View &V, double *x, double *v, double *f, cudaStream_t s);
 cudaError_t launch_ev_reduce(const View &V, double *out, cudaStream_t s);
-cudaError_t launch_backward(const View &V, const double *grad_f, double *grad_x, double *grad_params,
-                            int nblocks_part, cudaStream_t s);
+cudaError_t launch_backward(const View &V, const double *grad_f, double *grad_x, double *grad_params, cudaStream_t s);
 cudaError_t launch_eam_backward(const View &V, const double *grad_f, double *grad_x, double *grad_params,
-                                int nblocks_part, cudaStream_t s);
+                                cudaStream_t s);
 cudaError_t launch_neighbors_out(const View &V, int *counts, int *nbr, int cap, cudaStream_t s);
+// partial parameter gradients of a backward pass: blocks, and doubles per block
 int backward_partial_blocks(const View &V);
+int backward_partials_per_block(const View &V);
 // halo buffers of a spatial decomposition (md_halo_pack / md_halo_unpack)
 cudaError_t launch_halo_pack(const View &V, const int *idx, long long m, int what, int width, const double shift[3],
                              long long n_real, double *buf, cudaStream_t s);

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256) k_copy_peak(const float4 *a, float4 *b, l
 // ------------------------------------------------------------- FP64 math --
 __global__ void k_fp64_math(int op, long long n, const double *x, double *y) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        y[i] = op == 0 ? rcp_newton(x[i]) : rsqrt_newton(x[i]);
+        y[i] = op == 0 ? rcp64(x[i]) : rsqrt64(x[i]);
 }
 
 // time `reps` runs of `launch` (after one untimed run) with CUDA events on s
