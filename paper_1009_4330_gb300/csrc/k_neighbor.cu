@@ -463,6 +463,29 @@ __device__ __forceinline__ float fmin3(float a, float b, float c) {
     return d;
 }
 
+// Two FP32 operations in one instruction (sm_100 and later), each rounded as
+// the scalar one: half the issue slots of a pair of operations.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long d) {
+    float2 v;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(d));
+    return v;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // 32 x 32 bit-matrix transpose across a warp: on entry lane r holds row r
 // (bit c = M[r][c]); on return lane c holds column c (bit r = M[r][c]).
 // Five butterfly stages of recursive 2x2 block swaps.
@@ -478,51 +501,89 @@ __device__ __forceinline__ unsigned warp_transpose32(unsigned x, int lane) {
     return x;
 }
 
+// Append entry e to this lane's column of the append buffer if `bit` of the
+// lane's mask is set: store at shared address sa, then sa += one row.  Spelled out
+// with predicates: as C++ the compiler branches around the two statements.
+__device__ __forceinline__ void append_if(unsigned mask, unsigned bit, uint32_t e, unsigned &sa) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
+        "and.b32 t, %1, %3;\n\t"
+        "setp.ne.u32 p, t, 0;\n\t"
+        "@p st.shared.u32 [%0], %2;\n\t"
+        "@p add.u32 %0, %0, 128;\n\t}"
+        : "+r"(sa)
+        : "r"(mask), "r"(e), "r"(bit));
+}
+// the buffer is only accessed through these (volatile: in program order among themselves,
+// while the queue's ordinary loads move freely)
+__device__ __forceinline__ uint32_t buf_load(unsigned sa) {
+    uint32_t e;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(e) : "r"(sa));
+    return e;
+}
+__device__ __forceinline__ void buf_store(unsigned sa, uint32_t e) {
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(sa), "r"(e));
+}
+
 // Verlet list of every atom of a rebuilding replica: all j in the 27 cells
 // around i's cell with |x_i - x_j| < rl.  One warp per home cell (home atoms
-// in chunks of 32; a cell with more than 32 atoms is shared out over several
-// warps).  The 27 neighbour cells form 9 rows of 3 x-adjacent cells; lanes
-// 0..26 fetch the 27 cell bounds at once.  Each row is read as one flat
-// candidate range, 32 candidates at a time, one per lane, shifted into the
-// home cell's frame.  A candidate farther than rl from the bounding box of
-// the home atoms cannot be accepted by any of them (about 38 % of the 27-cell
+// in chunks of 32, one per lane; a cell with more than 32 atoms is shared out
+// over several warps).  The 27 neighbour cells form 9 rows of 3 x-adjacent cells.
+// Each row is read as one flat candidate range, 32 candidates at a time, one per
+// lane, the next 32 on their way meanwhile, shifted into the home cell's
+// frame.  A candidate farther than rl from the bounding box of
+// the home atoms cannot be accepted by any of them (about 30 % of the 27-cell
 // candidates); the others go to a per-warp queue in shared memory, in
-// candidate order, and are tested in full rounds of 32.  In a round each lane
+// candidate order, and are tested in full rounds of 32: each lane
 // tests its candidate against every home atom (records broadcast from shared
-// memory) into a 32-bit acceptance mask; a warp bit-matrix transpose turns the
-// candidates' masks into each home atom's mask of accepted candidates.  The
-// masks and entries of up to kBatch rounds are kept in shared memory, and
-// each home-atom lane then appends its accepted candidates in candidate order,
-// moving from round to round through a bitmask of its non-empty rounds (warp
-// ballot/prefix compaction in transposed form: deterministic lists; the loop
-// runs as long as the longest share of the batch, not the sum of each round's
-// longest share).  The test is FP32 with a margin far above its rounding
+// memory) into a 32-bit acceptance mask, and a warp bit-matrix transpose turns the
+// candidates' masks into each home atom's mask of accepted candidates.  Then the
+// candidates' entries are read one after another, and a home-atom lane that accepts
+// one appends it to its column of an append buffer in shared memory (test, store and
+// address in three predicated instructions, no bank conflicts), which is
+// written out four entries (16 bytes) at a time.  So the lists are in candidate
+// order (deterministic).
+// The home atoms' tests are two to an instruction (FP32x2).  What bounds it: instruction issue (73 %) and
+// the L1 data pipe (75 %) at rc 2.5, both at ~65 % at rc 5.0.  Against scanning each home
+// atom's masks bit by bit and storing 4-byte entries straight to the list, whose
+// scattered sectors bound the build at rc 5.0 (one launch, 500,000 atoms): rc 2.5 225 ->
+// 220 us (209.6 M -> 187.8 M warp instructions), rc 5.0 1.51 -> 1.09 ms; measured and not kept:
+// one lane per home atom testing the candidates one after another (219 M, 235 us at rc 2.5,
+// 1.14 ms at rc 5.0), storing straight to the list with predicates (234 M, 245 us, 1.53 ms),
+// larger and smaller append buffers (24 .. 52 rows: 219 .. 241 us).
+// The test is FP32 with a margin far above its rounding
 // error; pairs inside the margin band are decided in FP64, so the list equals
 // the FP64 definition exactly.  HALF keeps j > i only.
 constexpr int kQueue = 64;  // queued candidates per warp (< 32 left + 32 new)
-constexpr int kBatch = 14;  // rounds whose list entries are appended together
+constexpr int kApp = 16;    // candidates appended between two looks at the buffer's room
+constexpr int kBuf = 36;    // rows of the append buffer: a multiple of 4, >= 3 left over + kApp
+
 // The list build runs NW warps (cells or cell parts) per block.  One warp
 // per block when every cell has one warp: no block barrier, a block's
 // registers come free as soon as its cell is done, and the warp's
-// shared-memory addresses are constants, so that 64 registers (32 warps per
-// SM) hold the loops without spills.  Four when the warps of a cell share it
-// out, so that they share its candidates in L1; compiled for 28 warps per
-// SM (72 registers: at 64 this form spilled inside the loops).
-template <int NW>
-struct BuildOcc {
-    static constexpr int warps_per_sm = NW == 1 ? 32 : 28;
-};
+// shared-memory addresses are constants.  Four when the warps of a cell share it
+// out, so that they share its candidates in L1.  28 warps per SM (72 registers): by shared
+// memory there is no room for more, and at 64 registers the loops spill (work-list build: 735
+// against 702 us per step of 512 replicas).
+constexpr int kBuildWarps = 28;
+// blocks of the work-list build per resident one: a finer deal (702 -> 696 us)
+constexpr int kBuildWlDeal = 4;
 
 template <int PREC, int HALF, int NW>
 __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int hsplit, int lane, int w,
                                            int &my_max, long long &my_sum) {
-    __shared__ float4 s_h[NW][32];
-    __shared__ float4 s_q[NW][kQueue];  // shifted candidate position, .w = list entry bits
+    // home atoms 2k, 2k + 1: {x, x, y, y}, {z, z, |x|^2, |x|^2}
+    __shared__ __align__(16) float s_h[NW][16][8];
+    __shared__ float4 s_q[NW][kQueue];  // queued candidates: position in the home frame, .w = list entry bits
+    __shared__ __align__(16) uint32_t s_e[NW][32];  // the round's list entries
+    __shared__ uint32_t s_buf[NW][kBuf][32];            // append buffer: a column per home atom
     __shared__ float4 s_box[NW][2];     // bounding box of the home chunk: lo, hi
-    __shared__ int2 s_cell[NW][27];     // neighbour cells: first slot, count
-    __shared__ int s_delta[NW][2][64];     // per tile of the chunk, per stencil code: entry shift
-    __shared__ uint32_t s_t[NW][kBatch][32];  // per round: home atom's mask of accepted candidates
-    __shared__ uint32_t s_e[NW][kBatch][32];  // per round: candidate's list entry
+    // per row of 3 cells: candidate f's entry is f << 6 plus that of its cell
+    // ({cell 0, 1, 2}.x/y/z); candidates of the row; first candidate of cells 1 and
+    // 2, and the row's shift in y and z as float bits
+    __shared__ uint4 s_row[NW][9];
+    __shared__ int4 s_row2[NW][9];
+    __shared__ int s_delta[NW][2][64];  // per tile of the chunk, per stencil code: entry shift
     const int r = V.bin_rep[gb];
     const Rep &R = V.rep[r];
     const int maxn = V.maxneigh, lt = V.ltpa, lq = V.lvec;
@@ -532,15 +593,25 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
     const int bx = unpack_bx(xyz), by = unpack_by(xyz), bz = unpack_bz(xyz);
     const float hx = R.hf[0], hy = R.hf[1], hz = R.hf[2];
     // neighbour cell (row = lane / 3, dx = lane % 3 - 1) bounds, one lane each
-    if (lane < 27) {
-        const int row = lane / 3;
-        const int dx = lane - 3 * row - 1, dy = row % 3 - 1, dz = row / 3 - 1;
+    int cell_first = 0;
+    {
+        const int l = min(lane, 26), row = l / 3;
+        const int dx = l - 3 * row - 1, dy = row % 3 - 1, dz = row / 3 - 1;
         int cx = bx + dx, cy = by + dy, cz = bz + dz;
         cx += (cx < 0) ? nbx : ((cx >= nbx) ? -nbx : 0);
         cy += (cy < 0) ? nby : ((cy >= nby) ? -nby : 0);
         cz += (cz < 0) ? nbz : ((cz >= nbz) ? -nbz : 0);
         const int nbin = V.lin2bin[R.bin0 + (cz * nby + cy) * nbx + cx];
-        s_cell[w][lane] = make_int2(V.bin_start[nbin], V.bin_count[nbin]);
+        cell_first = V.bin_start[nbin];
+        const int cnt = V.bin_count[nbin];
+        const int c1 = __shfl_down_sync(0xffffffffu, cnt, 1), c2 = __shfl_down_sync(0xffffffffu, cnt, 2);
+        const int f1 = __shfl_down_sync(0xffffffffu, cell_first, 1), f2 = __shfl_down_sync(0xffffffffu, cell_first, 2);
+        if (lane < 27 && dx == -1) {
+            const uint32_t code = (uint32_t)((dz + 1) << 4 | (dy + 1) << 2);
+            s_row[w][row] = make_uint4(((uint32_t)cell_first << 6) + code, ((uint32_t)(f1 - cnt) << 6) + code + 1u,
+                                       ((uint32_t)(f2 - cnt - c1) << 6) + code + 2u, (uint32_t)(cnt + c1 + c2));
+            s_row2[w][row] = make_int4(cnt, cnt + c1, __float_as_int(dy * hy), __float_as_int(dz * hz));
+        }
     }
     const int hs = V.bin_start[gb], hn = V.bin_count[gb];
     const float rl2f = 0.5f * (V.rl2f_lo + V.rl2f_hi), margin = 0.5f * (V.rl2f_hi - V.rl2f_lo);
@@ -555,7 +626,8 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
             float4 hr = make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.f);
             if (lane < nh) hr = V.rec[hbase + lane];
             hr.w = hr.x * hr.x + hr.y * hr.y + hr.z * hr.z;
-            s_h[w][lane] = hr;
+            float *h = s_h[w][lane >> 1] + (lane & 1);
+            h[0] = hr.x; h[2] = hr.y; h[4] = hr.z; h[6] = hr.w;
             // bounding box of the chunk's home atoms
             const bool in = lane < nh;
             float lox = in ? hr.x : 3.0e38f, hix = in ? hr.x : -3.0e38f;
@@ -598,68 +670,63 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
                     const unsigned wd = V.tile_bits[(size_t)t * 32 + (idx >> 5)];
                     int k = V.tile_wpre[(size_t)t * 32 + (idx >> 5)] + __popc(wd & ((1u << (idx & 31)) - 1u));
                     k = min(k, kTileCells - 1);
-                    delta = (V.tile_off[(size_t)t * kTileCells + k] - s_cell[w][lane].x) * 64;
+                    delta = (V.tile_off[(size_t)t * kTileCells + k] - cell_first) * 64;
                 }
                 s_delta[w][X][code] = delta;
             }
         }
         __syncwarp();
-        // this lane as a home atom: its list
+        // this lane as a home atom: its list and its column of the append buffer
         const int p = hbase + lane;
         const int tsel = (tpa_atoms && p / tpa_atoms != tA) ? 1 : 0;
         uint32_t *const lbase = V.nlist + (size_t)(p >> la) * (size_t)((1 << la) * maxn) + (size_t)((p & ((1 << la) - 1)) << ltq);
-        unsigned slot = 0u;  // offset from lbase
-        const int jump = (32 << lq) - (tq - 1);
-        int mycnt = 0;
-        int qn = 0;  // queued candidates (warp-uniform)
-        // append the batch's accepted candidates to the home atoms' lists,
-        // round by round in candidate order: each home-atom lane walks its
-        // own masks, so the loop runs as long as the longest share of the
-        // batch rather than the sum of each round's longest share
-        int rb = 0;      // rounds in the pending batch (warp-uniform)
-        unsigned nz = 0u;  // this home atom: rounds of the batch in which it accepts a candidate
-        auto append = [&]() {
-            __syncwarp();
-            // written without branches: every lane runs every iteration, a
-            // lane whose share is done with all its predicates false
-            int r = nz ? __ffs(nz) - 1 : 0;     // round being appended
-            unsigned t = nz ? s_t[w][r][lane] : 0u;  // its candidates not yet appended
-            unsigned rest = nz & (nz - 1u);      // later rounds with entries
-            while (__any_sync(0xffffffffu, t != 0u)) {
-                // up to two entries of round r
-                const unsigned t1 = t & (t - 1u), t2 = t1 & (t1 - 1u);
-                const int c1 = (__ffs(t) - 1) & 31, c2 = (__ffs(t1) - 1) & 31;
-                uint32_t e1 = s_e[w][r][c1], e2 = s_e[w][r][c2];
-                if (tpa_atoms) {
-                    e1 += (uint32_t)s_delta[w][tsel][e1 & 63u];
-                    e2 += (uint32_t)s_delta[w][tsel][e2 & 63u];
+        const unsigned sa0 = (unsigned)__cvta_generic_to_shared(&s_buf[w][0][lane]);
+        unsigned sa = sa0;
+        int done = 0;  // entries written out: a multiple of 4 until the last flush
+        // write the buffer out, four entries at a time; all: the last, partly filled four too
+        // (entries past the list's end are never read)
+        auto flush = [&](bool all) {
+            const int pend = (int)((sa - sa0) >> 7);
+            const int out = all ? pend : pend & ~3;
+            const int most = min(out, maxn - done);  // (the capacity is a multiple of 4)
+            const int rounds = (__reduce_max_sync(0xffffffffu, out) + 3) >> 2;
+            unsigned at = sa0;
+            int kk = done;
+#pragma unroll 1
+            for (int k = 0; k < rounds; ++k, kk += 4, at += 4 * 128) {
+                if (kk < done + most) {
+                    uint32_t e[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) e[i] = buf_load(at + (unsigned)i * 128u);
+                    if (tpa_atoms) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) e[i] += (uint32_t)s_delta[w][tsel][e[i] & 63u];
+                    }
+                    if (lq == 2) {
+                        *reinterpret_cast<uint4 *>(lbase + (((unsigned)(kk >> ltq) << 7) + (unsigned)(kk & (tq - 1)))) =
+                            make_uint4(e[0], e[1], e[2], e[3]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            lbase[((unsigned)((kk + i) >> ltq) << (5 + lq)) + (unsigned)((kk + i) & (tq - 1))] = e[i];
+                    }
                 }
-                const bool s1 = t != 0u, s2 = t1 != 0u;
-                const int m1 = mycnt + 1, m2 = mycnt + 2;
-                const unsigned slot1 = slot + ((m1 & (tq - 1)) ? 1u : (unsigned)jump);
-                const unsigned slot2 = slot1 + ((m2 & (tq - 1)) ? 1u : (unsigned)jump);
-                if (s1 && mycnt < maxn) lbase[slot] = e1;
-                if (s2 && m1 < maxn) lbase[slot1] = e2;
-                mycnt = s2 ? m2 : (s1 ? m1 : mycnt);
-                slot = s2 ? slot2 : (s1 ? slot1 : slot);
-                // round r used up: on to the next round with entries
-                const int rn = rest ? __ffs(rest) - 1 : 0;
-                const unsigned tn = s_t[w][rn][lane];
-                const bool more = t2 != 0u;
-                t = more ? t2 : (rest ? tn : 0u);
-                r = more ? r : rn;
-                rest = more ? rest : (rest & (rest - 1u));
             }
-            __syncwarp();
-            rb = 0;
-            nz = 0u;
+            done += out;
+            if (all) return;
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                if (i < pend - out) buf_store(sa0 + (unsigned)i * 128u, buf_load(sa0 + (unsigned)(out + i) * 128u));
+            sa = sa0 + ((unsigned)(pend - out) << 7);
         };
+        int qn = 0;  // queued candidates (warp-uniform)
         // one round: queue entries 0..cnt-1 (cnt <= 32), one per lane
         auto round = [&](int cnt) {
             const float4 cq = s_q[w][lane];
             const bool qin = lane < cnt;
             const float qx = qin ? cq.x : -1.0e18f, qy = qin ? cq.y : -1.0e18f, qz = qin ? cq.z : -1.0e18f;
             const uint32_t e = qin ? __float_as_uint(cq.w) : 0u;
+            s_e[w][lane] = e;
             // acceptance bits over the home atoms, 8 at a time with
             // compile-time bit positions.  t = |x_i - q|^2 - rl^2 in the
             // dot-product form |x_i|^2 + |q|^2 - 2 x_i.q (FP32 error
@@ -669,87 +736,104 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
             const float q2m = qx * qx + qy * qy + qz * qz - rl2f;
             unsigned acc = 0u;
             float tmin = 3.0e38f;
-            // home atoms from the top down, 8 at a time: each test shifts its
-            // sign bit in at bit 0, so that home atom h ends at bit h
+            // home atoms from the top down, 8 at a time, two to an instruction: each
+            // test shifts its sign bit in at bit 0, so that home atom h ends at bit h
+            const unsigned long long qxx = pack2(qx2, qx2), qyy = pack2(qy2, qy2), qzz = pack2(qz2, qz2),
+                                     qww = pack2(q2m, q2m);
 #pragma unroll 1
             for (int hb = (nh - 1) & ~7; hb >= 0; hb -= 8) {
-                float t8[8];
 #pragma unroll
-                for (int k = 7; k >= 0; --k) {
-                    const float4 ri = s_h[w][hb + k];
-                    t8[k] = fmaf(qx2, ri.x, fmaf(qy2, ri.y, fmaf(qz2, ri.z, ri.w + q2m)));
-                    acc = __funnelshift_l(__float_as_uint(t8[k]), acc, 1);
+                for (int k = 6; k >= 0; k -= 2) {
+                    const ulonglong2 *h = reinterpret_cast<const ulonglong2 *>(s_h[w][(hb + k) >> 1]);
+                    const ulonglong2 xy = h[0], zw = h[1];
+                    const float2 t = unpack2(fma2(qxx, xy.x, fma2(qyy, xy.y, fma2(qzz, zw.x, add2(zw.y, qww)))));
+                    acc = __funnelshift_l(__float_as_uint(t.y), acc, 1);
+                    acc = __funnelshift_l(__float_as_uint(t.x), acc, 1);
+                    tmin = fmin3(tmin, fabsf(t.x), fabsf(t.y));
                 }
-#pragma unroll
-                for (int k = 0; k < 8; k += 2) tmin = fmin3(tmin, fabsf(t8[k]), fabsf(t8[k + 1]));
             }
             const int j = (int)(e >> 6);
             if (tmin < margin) {  // margin band: decide those pairs in FP64 (rare)
-                for (int h = 0; h < nh; ++h) {
-                    const float4 ri = s_h[w][h];
-                    const float t = fmaf(qx2, ri.x, fmaf(qy2, ri.y, fmaf(qz2, ri.z, ri.w + q2m)));
+                for (int k = 0; k < nh; ++k) {
+                    const float *h = s_h[w][k >> 1] + (k & 1);
+                    const float t = fmaf(qx2, h[0], fmaf(qy2, h[2], fmaf(qz2, h[4], h[6] + q2m)));
                     if (fabsf(t) < margin) {
-                        const bool in = in_list_fp64<PREC>(V, R, hbase + h, j, entry_dx(e), entry_dy(e),
+                        const bool in = in_list_fp64<PREC>(V, R, hbase + k, j, entry_dx(e), entry_dy(e),
                                                             entry_dz(e));
-                        acc = in ? (acc | (1u << h)) : (acc & ~(1u << h));
+                        acc = in ? (acc | (1u << k)) : (acc & ~(1u << k));
                     }
                 }
             }
             // exclusions: the atom itself; for HALF every home atom with slot >= j
             const int jh = j - hbase;  // j as a home-atom index, if it is one
-            if ((e & 63u) == 21u && jh >= 0 && jh < 32) acc &= ~(1u << jh);
+            if ((e & 63u) == kSelfCode && jh >= 0 && jh < 32) acc &= ~(1u << jh);
             if (HALF) acc &= jh <= 0 ? 0u : (jh >= 32 ? 0xffffffffu : ((1u << jh) - 1u));
-            // lane = home atom: bit c set if candidate lane c is accepted;
-            // kept with the round's entries until the batch is appended
+            // lane = home atom: bit c set if candidate lane c is accepted
             const unsigned tr = warp_transpose32(acc, lane);
-            s_t[w][rb][lane] = tr;
-            s_e[w][rb][lane] = e;
-            nz |= (tr != 0u ? 1u : 0u) << rb;
-            if (++rb == kBatch) append();
+            __syncwarp();
+            const uint4 *qe = reinterpret_cast<const uint4 *>(s_e[w]);
+#pragma unroll
+            for (int c0 = 0; c0 < 32; c0 += kApp) {
+                if (__any_sync(0xffffffffu, sa > sa0 + (kBuf - kApp) * 128)) flush(false);
+#pragma unroll
+                for (int c = c0; c < c0 + kApp; c += 4) {
+                    const uint4 u = qe[c / 4];
+                    append_if(tr, 1u << c, u.x, sa);
+                    append_if(tr, 2u << c, u.y, sa);
+                    append_if(tr, 4u << c, u.z, sa);
+                    append_if(tr, 8u << c, u.w, sa);
+                }
+            }
         };
+        // the row's next 32 candidates, one per lane: entry, record, shift (lanes past
+        // the row's end read the chunk's first home atom's record, and are dropped: no branch)
+        int row = 0, c0 = 0;
+        uint32_t ne = 0u;
+        float4 nr;
+        float nx = 0.f, ny = 0.f, nz = 0.f;
+        bool nin = false;
+        auto fetch = [&]() {
+            const uint4 ra = s_row[w][row];
+            const int4 rb = s_row2[w][row];
+            const int f = c0 + lane;
+            const bool s1 = f >= rb.x, s2 = f >= rb.y;
+            nin = f < (int)ra.w;
+            ne = ((uint32_t)f << 6) + (s2 ? ra.z : s1 ? ra.y : ra.x);
+            nx = s2 ? hx : s1 ? 0.f : -hx;
+            nr = V.rec[nin ? (int)(ne >> 6) : hbase];
+            ny = __int_as_float(rb.z);
+            nz = __int_as_float(rb.w);
+            c0 += 32;
+            if (c0 >= (int)ra.w) {
+                c0 = 0;
+                ++row;
+            }
+        };
+        fetch();
+        bool last = false;  // nothing more to fetch
         // fill the queue from the rows in order until it holds a full
         // round (or the rows are done), then run the round
-        int row = 0, c0 = 0;
-        int m = s_cell[w][0].y + s_cell[w][1].y + s_cell[w][2].y;
 #pragma unroll 1
         while (true) {
 #pragma unroll 1
-            while (qn < 32 && row < 9) {
-                // this lane as a candidate, shifted into the home frame,
+            while (qn < 32 && !last) {
                 // kept if within rl (plus the band) of the home bounding box
-                // (lanes past the row's end read a valid record, the chunk's
-                // first home atom's, and are dropped: no branch)
-                const int f = c0 + lane;
-                const int2 ca = s_cell[w][3 * row], cb = s_cell[w][3 * row + 1];
-                const int cxs = s_cell[w][3 * row + 2].x;
-                const int nab = ca.y + cb.y;
-                const int seg = (f >= ca.y) + (f >= nab);
-                const int j0 = seg == 0 ? ca.x + f : (seg == 1 ? cb.x + f - ca.y : cxs + f - nab);
-                const bool in = f < m;
-                const int j = in ? j0 : hbase;
-                const float4 rj = V.rec[j];
-                const int dy = row % 3 - 1, dz = row / 3 - 1;
-                float4 c;
-                c.x = rj.x + (seg == 0 ? -hx : (seg == 1 ? 0.f : hx));
-                c.y = rj.y + dy * hy;
-                c.z = rj.z + dz * hz;
-                c.w = __uint_as_float(((uint32_t)j << 6) | (uint32_t)seg | ((uint32_t)(dz + 1) << 4) |
-                                      ((uint32_t)(dy + 1) << 2));
+                const uint32_t e = ne;
+                const bool in = nin;
+                const float cx = nr.x + nx, cy = nr.y + ny, cz = nr.z + nz;
+                last = row >= 9;
+                if (!last) fetch();
                 const float4 lo = s_box[w][0], hi = s_box[w][1];
-                const float bx_ = fmaxf(fmaxf(lo.x - c.x, c.x - hi.x), 0.f);
-                const float by_ = fmaxf(fmaxf(lo.y - c.y, c.y - hi.y), 0.f);
-                const float bz_ = fmaxf(fmaxf(lo.z - c.z, c.z - hi.z), 0.f);
+                const float bx_ = fmaxf(fmaxf(lo.x - cx, cx - hi.x), 0.f);
+                const float by_ = fmaxf(fmaxf(lo.y - cy, cy - hi.y), 0.f);
+                const float bz_ = fmaxf(fmaxf(lo.z - cz, cz - hi.z), 0.f);
                 const bool keep = in && (bx_ * bx_ + by_ * by_ + bz_ * bz_ < keep2);
                 const unsigned kb = __ballot_sync(0xffffffffu, keep);
-                if (keep) s_q[w][qn + __popc(kb & ((1u << lane) - 1u))] = c;
-                qn += __popc(kb);
-                c0 += 32;
-                if (c0 >= m) {
-                    c0 = 0;
-                    ++row;
-                    if (row < 9)
-                        m = s_cell[w][3 * row].y + s_cell[w][3 * row + 1].y + s_cell[w][3 * row + 2].y;
+                if (keep) {
+                    const int at = qn + __popc(kb & ((1u << lane) - 1u));
+                    s_q[w][at] = make_float4(cx, cy, cz, __uint_as_float(e));
                 }
+                qn += __popc(kb);
             }
             if (qn == 0) break;
             const int cnt = min(qn, 32);
@@ -762,8 +846,9 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
             if (lane < qn) s_q[w][lane] = rest;
             __syncwarp();
         }
-        if (rb > 0) append();
+        flush(true);
         if (lane < nh) {
+            const int mycnt = done;
             V.ncount[p] = min(mycnt, maxn);
             if (mycnt > maxn) {
                 atomicMax(&V.ctl->need_maxneigh, mycnt);
@@ -776,7 +861,7 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
 }
 
 template <int PREC, int HALF, int NW>
-__global__ void __launch_bounds__(32 * NW, BuildOcc<NW>::warps_per_sm / NW) k_build(View V, KArgs a) {
+__global__ void __launch_bounds__(32 * NW, kBuildWarps / NW) k_build(View V, KArgs a) {
     const int lane = threadIdx.x & 31, w = NW == 1 ? 0 : threadIdx.x >> 5;
     // warp -> (cell, part): part q of a cell takes its home chunks q, q + hsplit, ...
     const int gw = blockIdx.x * NW + w;
@@ -846,7 +931,7 @@ __global__ void __launch_bounds__(1024) k_worklist(View V, KArgs a) {
 // Batched rebuild: a fixed grid walks the work list's units (k_worklist), so
 // that the bins of replicas keeping their lists cost no block launches.
 template <int PREC, int HALF>
-__global__ void __launch_bounds__(32, BuildOcc<1>::warps_per_sm) k_build_wl(View V, KArgs a) {
+__global__ void __launch_bounds__(32, kBuildWarps) k_build_wl(View V, KArgs a) {
     const int lane = threadIdx.x & 31, w = 0;
     const int nf = *V.wl_n;
     const int total = V.wl_u0[nf];
@@ -906,7 +991,7 @@ void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &
     if (wl) {
         const void *kb = fp64 ? (V.half ? (const void *)k_build_wl<MD_PREC_FP64, 1> : (const void *)k_build_wl<MD_PREC_FP64, 0>)
                               : (V.half ? (const void *)k_build_wl<MD_PREC_MIXED, 1> : (const void *)k_build_wl<MD_PREC_MIXED, 0>);
-        seq.push_back(KCall{kb, dim3(V.n_sm * BuildOcc<1>::warps_per_sm), dim3(32), 0, a});
+        seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * kBuildWlDeal), dim3(32), 0, a});
         return;
     }
     const int nw = V.hsplit > 1 ? 4 : 1;
