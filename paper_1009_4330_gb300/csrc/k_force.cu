@@ -76,6 +76,8 @@ __device__ __forceinline__ double group_sum(double x) {
     return x;
 }
 
+__device__ __forceinline__ float lane_value(float x, int src) { return __shfl_sync(0xffffffffu, x, src); }
+
 // |d|^2 with its operations spelled out (no contraction left to the compiler),
 // so that a pair's FP32 r^2 recomputed after the walk is the walk's own
 __device__ __forceinline__ float pair_r2(float dx, float dy, float dz) {
@@ -143,6 +145,77 @@ __device__ __forceinline__ void walk_mode(const View &V, int mode, const uint32_
         walk_list<T, Q, true>(V, lp, sub, cnt, xi, yi, zi, R.hf[0], R.hf[1], R.hf[2], srec, pair);
     else
         walk_list<T, Q, false>(V, lp, sub, cnt, xi, yi, zi, R.hf[0], R.hf[1], R.hf[2], srec, pair);
+}
+
+// The same walk for a system too small to fill the GPU with T threads per
+// atom, whose rounds would follow one another at the latency of a gather:
+// G lanes stand in for each of the T threads, lane g taking rounds g, g + G, ...,
+// and the rounds' sums are then added in the thread's own order, by all G
+// lanes alike (shuffles): bit for bit the sums of walk_list.  Bound by latency still: a gather
+// and G dependent compensated additions per G rounds instead of G gathers.
+struct Wide {
+    int lt, lg;   // log2 of T and G
+    int p;        // this lane's atom
+    int sub, g;   // its thread of the atom's T, its lane of that thread's G
+    bool lead;    // the lane that writes the atom
+};
+
+__device__ __forceinline__ Wide wide_lane(const View &V, int lg) {
+    Wide w;
+    w.lt = V.ltpa;
+    w.lg = lg;
+    const int ll = w.lt + lg, lane = threadIdx.x & 31;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    w.p = (gw << (5 - ll)) + (lane >> ll);
+    const int i = lane & ((1 << ll) - 1);
+    w.sub = i >> lg;
+    w.g = i & ((1 << lg) - 1);
+    w.lead = i == 0;
+    return w;
+}
+
+// sum over the T threads of the atom, in group_sum's order
+__device__ __forceinline__ double wide_sum(const Wide &w, double x) {
+    for (int o = (1 << w.lt) >> 1; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o << w.lg);
+    return x;
+}
+
+template <int Q, class Pair>
+__device__ __forceinline__ void walk_wide(const View &V, const Wide &w, const Rep &R, int cnt, float xi, float yi,
+                                          float zi, Pair &pair) {
+    const float hx = R.hf[0], hy4 = R.hf[1] * 0.25f, hz16 = R.hf[2] * 0.0625f;
+    const int per = Q << w.lt, G = 1 << w.lg, la = 5 - w.lt;
+    const int nr = (cnt + per - 1) >> (w.lt + (Q == 4 ? 2 : Q == 2 ? 1 : 0));
+    const int most = __reduce_max_sync(0xffffffffu, nr);
+    const uint32_t *lp = V.nlist + (size_t)(w.p >> la) * ((size_t)V.maxneigh << la) +
+                         (size_t)(((w.p & ((1 << la) - 1)) << w.lt) + w.sub) * Q;
+    const int first = (threadIdx.x & 31) - w.g;
+    uint32_t cur[Q], nxt[Q];
+    if (w.g < nr) load_entries<Q>(lp + (size_t)w.g * 32 * Q, cur);
+    for (int r0 = 0; r0 < most; r0 += G) {
+        const int r = r0 + w.g;
+        if (r + G < nr) load_entries<Q>(lp + (size_t)(r + G) * 32 * Q, nxt);
+        const int left = r < nr ? cnt - (r * per + w.sub * Q) : 0;
+        float xj[Q], yj[Q], zj[Q];
+        int tj[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            if (q < left) load_rec(V, entry_j(cur[q]), xj[q], yj[q], zj[q], tj[q]);
+        pair.round_begin();
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            if (q < left) {
+                const uint32_t e = cur[q];
+                const float dx = fmaf(-code_x(e), hx, xi - xj[q]);
+                const float dy = fmaf(-code_y4(e), hy4, yi - yj[q]);
+                const float dz = fmaf(-code_z16(e), hz16, zi - zj[q]);
+                pair(e, dx, dy, dz, pair_r2(dx, dy, dz), tj[q]);
+            }
+        }
+        for (int g = 0; g < G; ++g) pair.round_from(first + g, r0 + g < nr);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) cur[q] = nxt[q];
+    }
 }
 
 // stage the block's tile when its entries are block-local (before the
@@ -233,6 +306,19 @@ struct LJPair {
             for (int k = 0; k < 6; ++k) w[k].add(rw[k]);
         }
     }
+    // round_end with lane src's round sums (all lanes call it; use: this round exists)
+    __device__ __forceinline__ void round_from(int src, bool use) {
+        const float x = lane_value(rx, src), y = lane_value(ry, src), z = lane_value(rz, src);
+        if (use) { ax.add(x); ay.add(y); az.add(z); }
+        if (EV) {
+            const float u = lane_value(re, src);
+            if (use) e.add(u);
+            for (int k = 0; k < 6; ++k) {
+                const float q = lane_value(rw[k], src);
+                if (use) w[k].add(q);
+            }
+        }
+    }
     // energy and virial terms of one pair: summed plainly over the round and
     // added with compensation per round
     __device__ __forceinline__ void add_ev(float ee, float w0, float w1, float w2, float w3, float w4, float w5) {
@@ -300,14 +386,17 @@ struct LJPair {
 // out (counted by the walk) or to add (left out by it): force, half-list
 // partner, energy and virial alike.  The terms are summed over the warp into
 // the atom's first thread.  All 32 lanes call this together.
+// (T = 0: the lanes per atom, 2^ll, are a run-time value: the wide kernels.)
 template <int T, int Q, int MT, int HALF, int EV>
 __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV> &pr, bool flagged,
-                                              int gw, int lane, int tmode, const float4 *srec) {
-    constexpr int A = 32 / T;
+                                              int gw, int lane, int tmode, const float4 *srec, int ll = 0) {
+    constexpr bool kWide = T == 0;
+    const int L = kWide ? 1 << ll : T;  // lanes per atom
+    const int A = 32 / L;
     unsigned m = __ballot_sync(0xffffffffu, flagged);
     while (m) {
-        const int a = (__ffs(m) - 1) / T;  // the atom's index in the warp
-        m &= (T == 32) ? 0u : ~((((1u << (T & 31)) - 1u)) << (a * T));
+        const int a = (__ffs(m) - 1) / L;  // the atom's index in the warp
+        m &= (L == 32) ? 0u : ~((((1u << (L & 31)) - 1u)) << (a * L));
         const int p = gw * A + a;
         const Rep &R = V.rep[V.tile_rep[p >> 5]];
         const int cnt = V.ncount[p];
@@ -315,10 +404,11 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV
         int ti;
         load_rec(V, p, xi, yi, zi, ti);
         const float hx = R.hf[0], hy4 = R.hf[1] * 0.25f, hz16 = R.hf[2] * 0.0625f;
-        const uint32_t *base = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + a * T * Q;
+        const uint32_t *base = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + a * L * Q;
         float cx = 0.f, cy = 0.f, cz = 0.f, ce = 0.f, cw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         for (int k = lane; k < cnt; k += 32) {
-            const uint32_t e = base[(size_t)(k / (T * Q)) * 32 * Q + (k % (T * Q))];
+            const uint32_t e = kWide ? V.nlist[list_index(p, k, V.ltpa, V.lvec, V.maxneigh)]
+                                     : base[(size_t)(k / (L * Q)) * 32 * Q + (k % (L * Q))];
             float xj, yj, zj;
             int tj;
             if (tmode == 1) {
@@ -366,7 +456,7 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV
                 for (int c = 0; c < 6; ++c) cw[c] += __shfl_xor_sync(0xffffffffu, cw[c], o);
             }
         }
-        if (lane == a * T) {
+        if (lane == a * L) {
             pr.ax.add(cx); pr.ay.add(cy); pr.az.add(cz);
             if (EV) {
                 pr.e.add(ce);
@@ -375,6 +465,8 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV
         }
     }
 }
+
+constexpr int kWideBlock = 64;
 
 // registers per thread allowed to the mixed force-only pass: 56 keeps nine
 // 128-thread blocks (36 warps) resident per SM to hide the gather latency;
@@ -473,6 +565,55 @@ __global__ void __maxnreg__((LjRegs<T, Q, HALF, EV>::value)) k_lj(View V, KArgs 
             epilogue(V, a.mode, rem, p, pr.ti, fx, fy, fz, s_ftm);
             if (EV) write_ev(V, p, pr.ti, e_acc, w_acc, s_ftm);
         }
+    }
+}
+
+// the full-list pass of a small system (see walk_wide); a.aux = log2 of G
+template <int Q, int EV, int MT>
+__global__ void __launch_bounds__(kWideBlock) k_lj_wide(View V, KArgs a) {
+    __shared__ float s_tab[5][kMaxTypes * kMaxTypes];
+    if (MT) {
+        for (int k = threadIdx.x; k < V.ntypes * V.ntypes; k += blockDim.x) {
+            s_tab[0][k] = V.tab->lj1f[k]; s_tab[1][k] = V.tab->lj2f[k];
+            s_tab[2][k] = V.tab->lj3f[k]; s_tab[3][k] = V.tab->lj4f[k]; s_tab[4][k] = V.tab->offf[k];
+        }
+        __syncthreads();
+    }
+    const unsigned err = V.ctl->err;
+    const int rem = (a.mode == kModeStep) ? V.ctl->remaining : 0;
+    const Wide w = wide_lane(V, a.aux);
+    if (err || w.p >= V.n_pad) return;  // whole warps: n_pad is a multiple of 32
+    LJPair<MT, 0, EV> pr;
+    pr.V = &V;
+    pr.lj1 = s_tab[0]; pr.lj2 = s_tab[1]; pr.lj3 = s_tab[2]; pr.lj4 = s_tab[3]; pr.off = s_tab[4];
+    if (!MT) {
+        pr.c1 = V.tab->lj1f[0]; pr.c2 = V.tab->lj2f[0];
+        pr.c3 = V.tab->lj3f[0]; pr.c4 = V.tab->lj4f[0]; pr.c0 = V.tab->offf[0];
+    }
+    pr.rc2 = V.rc2f;
+    pr.nt = V.ntypes;
+    pr.n = V.n_pad;
+    pr.ti = 0;
+    pr.near_min = 3.0e38f;
+    pr.ax.zero(); pr.ay.zero(); pr.az.zero(); pr.e.zero();
+    for (int k = 0; k < 6; ++k) pr.w[k].zero();
+    const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
+    const bool valid = (w.p - R.atom0) < R.natoms;
+    const int cnt = valid ? V.ncount[w.p] : 0;
+    float xi, yi, zi;
+    load_rec(V, w.p, xi, yi, zi, pr.ti);
+    walk_wide<Q>(V, w, R, cnt, xi, yi, zi, pr);
+    fix_near_warp<0, Q>(V, pr, pr.near_min < V.rc2f_band, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                        threadIdx.x & 31, 0, nullptr, w.lt + w.lg);
+    const double fx = wide_sum(w, pr.ax.value()), fy = wide_sum(w, pr.ay.value()), fz = wide_sum(w, pr.az.value());
+    double e_acc = 0.0, w_acc[6] = {0, 0, 0, 0, 0, 0};
+    if (EV) {
+        e_acc = wide_sum(w, pr.e.value());
+        for (int k = 0; k < 6; ++k) w_acc[k] = wide_sum(w, pr.w[k].value());
+    }
+    if (valid && w.lead) {
+        epilogue(V, a.mode, rem, w.p, pr.ti, fx, fy, fz, V.tab->ftm_m);
+        if (EV) write_ev(V, w.p, pr.ti, e_acc, w_acc, V.tab->ftm_m);
     }
 }
 
@@ -685,12 +826,30 @@ struct RhoPair {
     float rc, rc2, part;
     __device__ __forceinline__ void round_begin() { part = 0; }
     __device__ __forceinline__ void round_end() { acc.add(part); }
+    __device__ __forceinline__ void round_from(int src, bool use) {
+        const float x = lane_value(part, src);
+        if (use) acc.add(x);
+    }
     __device__ __forceinline__ void operator()(uint32_t, float, float, float, float r2, int) {
         const float r = r2 * rsqrtf(r2);  // branch-free: t = 0 beyond rc
         const float t = (r2 < rc2) ? rc - r : 0.f;
         part += t * t;
     }
 };
+
+// F'(rho_i) of atom p, and its embedding energy for an energy pass
+__device__ __forceinline__ void finish_rho(const View &V, int mode, int p, double rho) {
+    const double Aemb = V.tab->eam[1];
+    // single element: the record's type slot is free until the next drift
+    // rewrites it, so F'(rho) rides in rec.w and the force pass gathers
+    // one 16-byte record per pair instead of two separate loads.  It is
+    // stored as FP32, so it is formed in FP32 (one reciprocal square
+    // root, a few FP32 ulps) rather than by an FP64 square root and
+    // divide on the FP64 pipe for every atom
+    const float rf = (float)rho;
+    V.rec[p].w = rf > 0.f ? -0.5f * (float)Aemb * rsqrtf(rf) : 0.f;
+    if (mode == kModeEV) V.emb[p] = rho > 0.0 ? -Aemb * sqrt(rho) : 0.0;
+}
 
 template <int T, int Q>
 __global__ void __launch_bounds__(256) k_eam_rho(View V, KArgs a) {
@@ -721,18 +880,27 @@ __global__ void __launch_bounds__(256) k_eam_rho(View V, KArgs a) {
         }
     }
     const double rho = group_sum<T>(pr.acc.value());
-    if (valid && sub == 0) {
-        const double Aemb = V.tab->eam[1];
-        // single element: the record's type slot is free until the next drift
-        // rewrites it, so F'(rho) rides in rec.w and the force pass gathers
-        // one 16-byte record per pair instead of two separate loads.  It is
-        // stored as FP32, so it is formed in FP32 (one reciprocal square
-        // root, a few FP32 ulps) rather than by an FP64 square root and
-        // divide on the FP64 pipe for every atom
-        const float rf = (float)rho;
-        V.rec[p].w = rf > 0.f ? -0.5f * (float)Aemb * rsqrtf(rf) : 0.f;
-        if (a.mode == kModeEV) V.emb[p] = rho > 0.0 ? -Aemb * sqrt(rho) : 0.0;
-    }
+    if (valid && sub == 0) finish_rho(V, a.mode, p, rho);
+}
+
+// the density pass of a small system (see walk_wide)
+template <int Q>
+__global__ void __launch_bounds__(kWideBlock) k_eam_rho_wide(View V, KArgs a) {
+    const unsigned err = V.ctl->err;
+    const Wide w = wide_lane(V, a.aux);
+    if (err || w.p >= V.n_pad) return;
+    RhoPair pr;
+    pr.acc.zero();
+    pr.rc = V.tab->eamf[0];
+    pr.rc2 = V.rc2f;
+    const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
+    const bool valid = (w.p - R.atom0) < R.natoms;
+    float xi, yi, zi;
+    int ti;
+    load_rec(V, w.p, xi, yi, zi, ti);
+    walk_wide<Q>(V, w, R, valid ? V.ncount[w.p] : 0, xi, yi, zi, pr);
+    const double rho = wide_sum(w, pr.acc.value());
+    if (valid && w.lead) finish_rho(V, a.mode, w.p, rho);
 }
 
 // pass 2: F_i = -sum_j [phi'(r) + (F'_i + F'_j) rho'(r)] d / r
@@ -755,6 +923,19 @@ struct EamPair {
         if (EV) {
             e.add(re);
             for (int k = 0; k < 6; ++k) w[k].add(rw[k]);
+        }
+    }
+    // round_end with lane src's round sums (all lanes call it; use: this round exists)
+    __device__ __forceinline__ void round_from(int src, bool use) {
+        const float x = lane_value(rx, src), y = lane_value(ry, src), z = lane_value(rz, src);
+        if (use) { ax.add(x); ay.add(y); az.add(z); }
+        if (EV) {
+            const float u = lane_value(re, src);
+            if (use) e.add(u);
+            for (int k = 0; k < 6; ++k) {
+                const float q = lane_value(rw[k], src);
+                if (use) w[k].add(q);
+            }
         }
     }
     // wj: F'_j, which came with the record (rec.w, set by the density pass)
@@ -839,6 +1020,37 @@ __global__ void __launch_bounds__(256) k_eam_force(View V, KArgs a) {
         // record's .w holds F'(rho), not a type
         epilogue(V, a.mode, rem, p, 0, fx, fy, fz, s_ftm);
         if (EV) write_ev(V, p, 0, e_acc + V.emb[p], w_acc, s_ftm);
+    }
+}
+
+// the force pass of a small system (see walk_wide)
+template <int Q, int EV>
+__global__ void __launch_bounds__(kWideBlock) k_eam_force_wide(View V, KArgs a) {
+    const unsigned err = V.ctl->err;
+    const int rem = (a.mode == kModeStep) ? V.ctl->remaining : 0;
+    const Wide w = wide_lane(V, a.aux);
+    if (err || w.p >= V.n_pad) return;
+    EamPair<EV> pr;
+    pr.rc = V.tab->eamf[0]; pr.c0 = V.tab->eamf[2]; pr.c1 = V.tab->eamf[3]; pr.c2 = V.tab->eamf[4];
+    pr.rc2 = V.rc2f;
+    pr.ax.zero(); pr.ay.zero(); pr.az.zero(); pr.e.zero();
+    for (int k = 0; k < 6; ++k) pr.w[k].zero();
+    const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
+    const bool valid = (w.p - R.atom0) < R.natoms;
+    float xi, yi, zi;
+    int ti;
+    load_rec(V, w.p, xi, yi, zi, ti);
+    pr.fpi = __int_as_float(ti);
+    walk_wide<Q>(V, w, R, valid ? V.ncount[w.p] : 0, xi, yi, zi, pr);
+    const double fx = wide_sum(w, pr.ax.value()), fy = wide_sum(w, pr.ay.value()), fz = wide_sum(w, pr.az.value());
+    double e_acc = 0.0, w_acc[6] = {0, 0, 0, 0, 0, 0};
+    if (EV) {
+        e_acc = wide_sum(w, pr.e.value());
+        for (int k = 0; k < 6; ++k) w_acc[k] = wide_sum(w, pr.w[k].value());
+    }
+    if (valid && w.lead) {
+        epilogue(V, a.mode, rem, w.p, 0, fx, fy, fz, V.tab->ftm_m);
+        if (EV) write_ev(V, w.p, 0, e_acc + V.emb[w.p], w_acc, V.tab->ftm_m);
     }
 }
 
@@ -1101,10 +1313,45 @@ static const void *pick_eamf(int T, int Q, int ev) {
     return ev ? pick_eamf_q<1, 1>(T) : pick_eamf_q<1, 0>(T);
 }
 
-// the pair passes of one precision: [LJ pass], or [density, force] for EAM
+// log2 of the lanes that stand in for one thread of the list layout (walk_wide): as
+// many as keep the whole system within kWideThreads threads per SM, at most
+// eight.  us per step with one lane, and with 512 / 1024 / 2048 threads per SM: 4,000
+// atoms 30.6, 24.4 (8 lanes); 16,000 atoms 30.9, 26.4 (4) / 27.7 (8); 32,771 atoms 32.7, 30.9 (2) / 30.4
+// (4) / 36.0 (8); 65,536 atoms 36.7, 37.5 (2); 8,000 atoms at four threads per atom 27.0, 26.8 (2) /
+// 29.1 (4).  16 and 32 lanes for the smallest systems: 4,000 atoms 24.8 and 26.6.
+constexpr int kWideThreads = 640, kWideMost = 3;
+
+static int wide_log(const View &V) {
+    int lg = 0;
+    while (lg < kWideMost && V.ltpa + lg < 5 && ((long long)V.n_pad << (V.ltpa + lg + 1)) <= (long long)V.n_sm * kWideThreads)
+        ++lg;
+    return lg;
+}
+
+#define PICK_WIDE(K, ...) \
+    (V.vec == 4 ? (const void *)K<4, ##__VA_ARGS__> : V.vec == 2 ? (const void *)K<2, ##__VA_ARGS__> : (const void *)K<1, ##__VA_ARGS__>)
+
+// the mixed pair passes: [LJ pass], or [density, force] for EAM
 static void mixed_force_sequence(const View &V, int mode, int block, KArgs a, std::vector<KCall> &seq) {
     const int T = V.tpa;
     const int ev = (mode == kModeEV) ? 1 : 0;
+    const int lg = V.half || V.tile_atoms > 0 ? 0 : wide_log(V);
+    if (lg > 0) {
+        a.aux = lg;
+        const dim3 grid((unsigned)((((long long)V.n_pad << (V.ltpa + lg)) + kWideBlock - 1) / kWideBlock));
+        if (V.pot == MD_POT_LJ) {
+            const void *fn = V.ntypes > 1 ? (ev ? PICK_WIDE(k_lj_wide, 1, 1) : PICK_WIDE(k_lj_wide, 0, 1))
+                                          : (ev ? PICK_WIDE(k_lj_wide, 1, 0) : PICK_WIDE(k_lj_wide, 0, 0));
+            seq.push_back(KCall{fn, grid, dim3(kWideBlock), 0, a});
+        } else {
+            KArgs ar = a;
+            ar.in_graph = 0;
+            seq.push_back(KCall{PICK_WIDE(k_eam_rho_wide), grid, dim3(kWideBlock), 0, ar});
+            seq.push_back(KCall{ev ? PICK_WIDE(k_eam_force_wide, 1) : PICK_WIDE(k_eam_force_wide, 0), grid,
+                                dim3(kWideBlock), 0, a});
+        }
+        return;
+    }
     const long long threads = (long long)V.n_pad * T;
     const dim3 grid((unsigned)((threads + block - 1) / block));
     const size_t sm = V.tile_atoms > 0 ? kTileSmem : 0;
