@@ -37,7 +37,7 @@ __device__ __forceinline__ void abs_pos(const View &V, const Rep &R, int p, doub
     } else {
         for (int c = 0; c < 3; ++c) x[c] = V.xr[c * V.n_pad + p];
     }
-    for (int c = 0; c < 3; ++c) x[c] += ((double)bc[c] + 0.5) * R.h[c];
+    for (int c = 0; c < 3; ++c) x[c] = fma(bin_centre(bc[c]), R.h[c], x[c]);
 }
 
 // Stage new positions and/or velocities (original order; NULL keeps the
@@ -74,11 +74,7 @@ __global__ void k_state_out(View V, double *x, double *v, double *f) {
         double xa[3];
         abs_pos<PREC>(V, R, p, xa);
         for (int c = 0; c < 3; ++c) {
-            const double L = R.L[c];
-            double w = xa[c] - floor(xa[c] * R.Linv[c]) * L;
-            if (w >= L) w -= L;
-            if (w < 0.0) w += L;
-            x[3 * o + c] = w;
+            x[3 * o + c] = wrap_box(xa[c], R.L[c], R.Linv[c]);
         }
     }
     if (v) for (int c = 0; c < 3; ++c) v[3 * o + c] = V.v[c * n + p];
@@ -87,11 +83,18 @@ __global__ void k_state_out(View V, double *x, double *v, double *f) {
 
 // ------------------------------------------------------ energy / virial ----
 
-// Two fixed-order stages: per 32-atom tile (one warp each), then per
-// replica over its tiles (one block each, each thread a fixed stride of
-// tiles, then the block's fixed-order sum).  The tile stage loads its eight
-// terms before the eight shuffle trees, the replica stage reads each tile's
-// eight sums together: both are bound by memory, not by chains of waits.
+// Fixed-order stages: per 32-atom tile (one warp each), per segment of a
+// replica's tiles (one block each), and, where a replica has several
+// segments, over these in the last block.  The FP64 adds bound it (2 lanes per clock
+// and SM): a warp's eight sums are reduced by halves (lanes exchange the half they do
+// not keep: 9 adds instead of 8 trees of 5), and the tiles of a few
+// large systems are spread over several blocks each.
+constexpr int kEvSegment = 256;  // tiles per block
+
+__device__ __forceinline__ double ev_fold(double keep, double send, int o) {
+    return keep + __shfl_xor_sync(0xffffffffu, send, o);
+}
+
 __global__ void k_ev_tiles(View V) {
     const int lane = threadIdx.x & 31;
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -101,40 +104,55 @@ __global__ void k_ev_tiles(View V) {
     const bool ok = (p - R.atom0) < R.natoms;
     double x[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) x[k] = ok ? V.ev[k * V.n_pad + p] : 0.0;
+    for (int k = 0; k < 8; ++k) x[k] = ok ? V.ev[(size_t)k * V.n_pad + p] : 0.0;
+    // lane bit 4 keeps terms 0..3 or 4..7, bit 3 two of these, bit 2 one
+    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+    double y[4], z[2];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
+    for (int k = 0; k < 4; ++k) y[k] = ev_fold(h4 ? x[k + 4] : x[k], h4 ? x[k] : x[k + 4], 16);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) x[k] += __shfl_xor_sync(0xffffffffu, x[k], o);
-    if (lane < 8) {
-        double y = x[0];
-#pragma unroll
-        for (int k = 1; k < 8; ++k) y = lane == k ? x[k] : y;
-        V.ev_tile[(size_t)t * 8 + lane] = y;
-    }
+    for (int k = 0; k < 2; ++k) z[k] = ev_fold(h3 ? y[k + 2] : y[k], h3 ? y[k] : y[k + 2], 8);
+    double u = ev_fold(h2 ? z[1] : z[0], h2 ? z[0] : z[1], 4);
+    u = ev_fold(u, u, 2);
+    u = ev_fold(u, u, 1);
+    if ((lane & 3) == 0) V.ev_tile[(size_t)t * 8 + (lane >> 2)] = u;
 }
 
-__global__ void __launch_bounds__(1024) k_ev_reduce(View V, double *out) {
-    __shared__ double s_w[32];
-    const int r = blockIdx.x;
+// nseg blocks per replica, 256 threads: thread = (slot, term)
+__global__ void __launch_bounds__(256) k_ev_reduce(View V, int nseg, double *out) {
+    __shared__ double s_w[8][8];
+    const int r = blockIdx.x / nseg, seg = blockIdx.x - r * nseg;
     const Rep &R = V.rep[r];
-    double acc[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll 2
-    for (int t = R.tile0 + threadIdx.x; t < R.tile0 + R.ntiles; t += blockDim.x) {
-        const double2 *q = reinterpret_cast<const double2 *>(&V.ev_tile[(size_t)t * 8]);
-        double2 u[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) u[k] = q[k];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            acc[2 * k] += u[k].x;
-            acc[2 * k + 1] += u[k].y;
-        }
+    const int term = threadIdx.x & 7, slot = threadIdx.x >> 3, w = threadIdx.x >> 5;
+    auto sum = [&](const double *rows, int n) {  // sum of n rows of eight terms; thread < 8 gets its term
+        double acc = 0.0;
+#pragma unroll 4
+        for (int t = slot; t < n; t += 32) acc += __ldcg(&rows[(size_t)t * 8 + term]);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+        __syncthreads();
+        if ((threadIdx.x & 31) < 8) s_w[w][term] = acc;
+        __syncthreads();
+        double tot = 0.0;
+        if (threadIdx.x < 8)
+            for (int k = 0; k < 8; ++k) tot += s_w[k][term];
+        return tot;
+    };
+    const int t0 = R.tile0 + (int)((long long)R.ntiles * seg / nseg);
+    const int t1 = R.tile0 + (int)((long long)R.ntiles * (seg + 1) / nseg);
+    const double part = sum(V.ev_tile + (size_t)t0 * 8, t1 - t0);
+    if (nseg == 1) {
+        if (threadIdx.x < 8) out[8 * r + term] = part;
+        return;
     }
-    for (int k = 0; k < 8; ++k) {
-        const double tot = block_sum(acc[k], s_w);
-        if (threadIdx.x == 0) out[8 * r + k] = tot;
+    if (threadIdx.x < 8) V.ev_seg[(size_t)blockIdx.x * 8 + term] = part;
+    if (!last_block(&V.ctl->ticket_ev)) return;
+    __threadfence();
+    for (int q = 0; q < V.n_rep; ++q) {
+        const double tot = sum(V.ev_seg + (size_t)q * nseg * 8, nseg);
+        if (threadIdx.x < 8) out[8 * q + term] = tot;
     }
+    if (threadIdx.x == 0) V.ctl->ticket_ev = 0;
 }
 
 // ------------------------------------------------------------ list out ----
@@ -189,11 +207,7 @@ __global__ void k_halo_pack(View V, const int *idx, long long m, int what, int w
             abs_pos<PREC>(V, R, p, xa);
             const double sh[3] = {sx, sy, sz};
             for (int a = 0; a < 3; ++a) {
-                const double L = R.L[a];
-                double w = xa[a] - floor(xa[a] * R.Linv[a]) * L;
-                if (w >= L) w -= L;
-                if (w < 0.0) w += L;
-                row[c++] = w + sh[a];
+                row[c++] = wrap_box(xa[a], R.L[a], R.Linv[a]) + sh[a];
             }
         }
         if (what & kHaloV) for (int a = 0; a < 3; ++a) row[c++] = V.v[a * n + p];
@@ -220,7 +234,7 @@ __global__ void k_halo_unpack(View V, const int *idx, long long m, int what, int
             const int bc[3] = {unpack_bx(b), unpack_by(b), unpack_bz(b)};
             double d[3];
             for (int a = 0; a < 3; ++a) {
-                double t = row[c++] - ((double)bc[a] + 0.5) * R.h[a];
+                double t = fma(-bin_centre(bc[a]), R.h[a], row[c++]);
                 t -= R.L[a] * rint(t * R.Linv[a]);
                 d[a] = t;
             }
@@ -295,7 +309,10 @@ cudaError_t launch_state_out(const View &V, double *x, double *v, double *f, cud
 
 cudaError_t launch_ev_reduce(const View &V, double *out, cudaStream_t s) {
     k_ev_tiles<<<grid_of(V.n_tiles * 32, 256), 256, 0, s>>>(V);
-    k_ev_reduce<<<V.n_rep, 1024, 0, s>>>(V, out);
+    // segments of about kEvSegment tiles, at most kEvSegments in all
+    const int per = (V.n_tiles / V.n_rep + kEvSegment - 1) / kEvSegment;
+    const int nseg = std::max(1, std::min(per, kEvSegments / V.n_rep));
+    k_ev_reduce<<<V.n_rep * nseg, 256, 0, s>>>(V, nseg, out);
     return cudaGetLastError();
 }
 

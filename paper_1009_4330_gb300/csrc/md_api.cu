@@ -525,6 +525,7 @@ static md_status create_impl(int n_rep, const md_config *cfgs, const double *con
     V.lin2bin = d_lin2bin;
     V.bin2xyz = d_bin2xyz;
     AL(V.ev_tile, (size_t)V.n_tiles * 8);
+    AL(V.ev_seg, (size_t)kEvSegments * 8);
     if (V.prec == MD_PREC_FP64) AL(V.pos4, n);
     else AL(V.xr, 3 * n);
     AL(V.v, 3 * n);

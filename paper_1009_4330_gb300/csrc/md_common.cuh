@@ -75,6 +75,7 @@ struct Ctl {                // device control block of a handle
     long long steps;        // completed time steps
     long long rebuilds;     // completed replica builds
     unsigned disp_max;      // md_vv MD_VV_DISP: max squared displacement since the build, float bits
+    unsigned ticket_ev;     // last-block ticket of the energy reduction (reset by the last block)
     unsigned ticket_scan;   // last-block ticket of the bin-count scan's first pass (reset by the last block)
 };
 
@@ -144,6 +145,7 @@ struct View {
     // per-atom energy / virial for deterministic reductions: [8][n_pad]
     double *ev;
     double *ev_tile;      // [n_tiles][8] per-tile partial sums
+    double *ev_seg;       // [kEvSegments][8] partial sums of segments of a replica's tiles
     // backward
     double4_32a *bpack;   // [n_pad][2] x, y, z, type | dL/dF, 0
     double *bw;           // [2][n_pad] EAM backward: F'(rho_i), mu_i = lambda_i F''(rho_i)
@@ -387,6 +389,28 @@ __device__ __forceinline__ int tile_mode(const View &V, int T) {
         return -1;
     }
     return V.tile_cnt[blockIdx.x] >= 0 ? 1 : 0;
+}
+
+// blocks an energy reduction is spread over at most (where a replica takes several)
+constexpr int kEvSegments = 152;
+
+// b + 1/2 in FP64 from the exact FP32 sum (b < 2^22) by moving bits: the
+// conversion of an integer holds the FP64 pipe for as long as an FP64 add
+__device__ __forceinline__ double bin_centre(int b) { return widen_bits((float)b + 0.5f); }
+
+// 0 <= x < L (NaN: false) by the order of the bits: integer compares
+__device__ __forceinline__ bool in_box(double x, double L) {
+    return (unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(L);
+}
+
+// x wrapped into [0, L); nearly every coordinate is there already, and the
+// FP64 product, floor and compares are then left out
+__device__ __forceinline__ double wrap_box(double x, double L, double Linv) {
+    if (in_box(x, L)) return x;
+    double w = x - floor(x * Linv) * L;
+    if (w >= L) w -= L;
+    if (w < 0.0) w += L;
+    return w;
 }
 
 // last-block-done ticket: returns true in every thread of the last block to
