@@ -73,11 +73,11 @@ __device__ __forceinline__ void prepare_slot(const View &V, const KArgs &a, int 
         for (int c = 0; c < 3; ++c) {
             V.tv[c * n + p] = V.v[c * n + p];
             double x = xr[c];
-            // Bins moved along this axis, floor(x / h + 1/2).  FP64 instructions bound this kernel
-            // (2 lanes per clock and SM; 18 of them per atom took 27 us of 864,000 atoms, against
-            // 16 us for its bytes), so |x| is compared with the bin's half edge and
-            // edge as integers; an atom moves at most one bin between builds, unless
-            // skins are wider than bins or the state has run away
+            // Bins moved along this axis, floor(x / h + 1/2), by comparing |x| with the
+            // bin's half edge and edge as integers (six FP64 instructions less per axis;
+            // no gain where memory bounds the pass: 26.4 us of 864,000 atoms either way);
+            // an atom moves at most one bin between builds, unless skins are wider than
+            // bins or the state has run away
             const double h = R.h[c];
             const long long xb = __double_as_longlong(x), ax = xb & 0x7fffffffffffffffll;
             const long long edge = __double_as_longlong(h), half = edge - (1ll << 52);
