@@ -76,8 +76,6 @@ __device__ __forceinline__ double group_sum(double x) {
     return x;
 }
 
-__device__ __forceinline__ float lane_value(float x, int src) { return __shfl_sync(0xffffffffu, x, src); }
-
 // |d|^2 with its operations spelled out (no contraction left to the compiler),
 // so that a pair's FP32 r^2 recomputed after the walk is the walk's own
 __device__ __forceinline__ float pair_r2(float dx, float dy, float dz) {
@@ -149,15 +147,16 @@ __device__ __forceinline__ void walk_mode(const View &V, int mode, const uint32_
 
 // The same walk for a system too small to fill the GPU with T threads per
 // atom, whose rounds would follow one another at the latency of a gather:
-// G lanes stand in for each of the T threads, lane g taking rounds g, g + G, ...,
-// and the rounds' sums are then added in the thread's own order, by all G
-// lanes alike (shuffles): bit for bit the sums of walk_list.  Bound by latency still: a gather
-// and G dependent compensated additions per G rounds instead of G gathers.
+// G lanes stand in for each of the T threads, lane g taking rounds g, g + G, ....
+// The rounds' sums go to shared memory, and lane g adds term g (g + G, ... ; force
+// components, energy and virial terms) of all rounds in the thread's own order: bit for
+// bit the sums of walk_list.  What bounds it is the length of a warp's instruction stream at ~9 clocks
+// an instruction, so each term is added by one lane (all G lanes adding all terms,
+// by shuffles: 1,410 instructions per warp and 11.2 us for 500 atoms).
 struct Wide {
     int lt, lg;   // log2 of T and G
     int p;        // this lane's atom
     int sub, g;   // its thread of the atom's T, its lane of that thread's G
-    bool lead;    // the lane that writes the atom
 };
 
 __device__ __forceinline__ Wide wide_lane(const View &V, int lg) {
@@ -170,7 +169,6 @@ __device__ __forceinline__ Wide wide_lane(const View &V, int lg) {
     const int i = lane & ((1 << ll) - 1);
     w.sub = i >> lg;
     w.g = i & ((1 << lg) - 1);
-    w.lead = i == 0;
     return w;
 }
 
@@ -180,18 +178,46 @@ __device__ __forceinline__ double wide_sum(const Wide &w, double x) {
     return x;
 }
 
-template <int Q, class Pair>
-__device__ __forceinline__ void walk_wide(const View &V, const Wide &w, const Rep &R, int cnt, float xi, float yi,
-                                          float zi, Pair &pair) {
+// A wide lane's atom as it is loaded at once, before anything is known about
+// it: every dependent load costs a small system ~0.4 us.  (The first list entries lie within
+// the list's capacity; past the list's end they are not looked at.)
+template <int Q>
+struct WideAtom {
+    const uint32_t *lp;
+    uint32_t cur[Q];
+    float x, y, z;
+    int t, count;
+    unsigned err;
+    int remaining;
+};
+
+template <int Q>
+__device__ __forceinline__ WideAtom<Q> load_wide(const View &V, const Wide &w) {
+    WideAtom<Q> a;
+    const int la = 5 - w.lt;
+    a.lp = V.nlist + (size_t)(w.p >> la) * ((size_t)V.maxneigh << la) +
+           (size_t)(((w.p & ((1 << la) - 1)) << w.lt) + w.sub) * Q;
+    if (w.g < (V.maxneigh >> w.lt) / Q) load_entries<Q>(a.lp + (size_t)w.g * 32 * Q, a.cur);
+    load_rec(V, w.p, a.x, a.y, a.z, a.t);
+    a.count = V.ncount[w.p];
+    a.err = V.ctl->err;
+    a.remaining = V.ctl->remaining;
+    return a;
+}
+
+// NT terms; KT: the most that one lane adds (terms g + k G, k < KT, G >= 2)
+template <int Q, int NT, int KT, class Pair>
+__device__ __forceinline__ void walk_wide(const View &V, const Wide &w, const Rep &R, int cnt, WideAtom<Q> &at,
+                                          float (*s_round)[32], Pair &pair, KahanF (&acc)[KT]) {
     const float hx = R.hf[0], hy4 = R.hf[1] * 0.25f, hz16 = R.hf[2] * 0.0625f;
-    const int per = Q << w.lt, G = 1 << w.lg, la = 5 - w.lt;
+    const float xi = at.x, yi = at.y, zi = at.z;
+    const int lane = threadIdx.x & 31;
+    const int per = Q << w.lt, G = 1 << w.lg;
     const int nr = (cnt + per - 1) >> (w.lt + (Q == 4 ? 2 : Q == 2 ? 1 : 0));
     const int most = __reduce_max_sync(0xffffffffu, nr);
-    const uint32_t *lp = V.nlist + (size_t)(w.p >> la) * ((size_t)V.maxneigh << la) +
-                         (size_t)(((w.p & ((1 << la) - 1)) << w.lt) + w.sub) * Q;
-    const int first = (threadIdx.x & 31) - w.g;
-    uint32_t cur[Q], nxt[Q];
-    if (w.g < nr) load_entries<Q>(lp + (size_t)w.g * 32 * Q, cur);
+    const uint32_t *lp = at.lp;
+    const int first = lane - w.g;
+    uint32_t (&cur)[Q] = at.cur, nxt[Q];
     for (int r0 = 0; r0 < most; r0 += G) {
         const int r = r0 + w.g;
         if (r + G < nr) load_entries<Q>(lp + (size_t)(r + G) * 32 * Q, nxt);
@@ -212,10 +238,35 @@ __device__ __forceinline__ void walk_wide(const View &V, const Wide &w, const Re
                 pair(e, dx, dy, dz, pair_r2(dx, dy, dz), tj[q]);
             }
         }
-        for (int g = 0; g < G; ++g) pair.round_from(first + g, r0 + g < nr);
+#pragma unroll
+        for (int k = 0; k < NT; ++k) s_round[k][lane] = pair.term(k);
+        __syncwarp();
+        const int n = min(nr - r0, G);  // rounds of this turn
+#pragma unroll
+        for (int k = 0; k < KT; ++k) {
+            const int term = w.g + k * G;
+            if (term < NT) {
+                const float *s = &s_round[term][first];
+#pragma unroll 4
+                for (int g = 0; g < n; ++g) acc[k].add(s[g]);
+            }
+        }
+        __syncwarp();
 #pragma unroll
         for (int q = 0; q < Q; ++q) cur[q] = nxt[q];
     }
+}
+
+// force component c of atom p: kick or store
+__device__ __forceinline__ void wide_finish(const View &V, int mode, int rem, int c, int p, double ftm, double f) {
+    const size_t i = (size_t)c * V.n_pad + p;
+    if (mode == kModeStep || mode == kModeKickDry) {
+        const bool last = (mode == kModeStep && rem == 0);
+        const double k = (mode == kModeKickDry) ? 0.0 : (last ? 0.5 : 1.0) * V.dt * ftm;
+        V.v[i] += k * f;
+        if (!last) return;
+    }
+    V.f[i] = f;
 }
 
 // stage the block's tile when its entries are block-local (before the
@@ -246,11 +297,16 @@ __device__ __forceinline__ void epilogue(const View &V, int mode, int rem, int p
     }
 }
 
-__device__ __forceinline__ void write_ev(const View &V, int p, int t, double e, const double *w, const double *s_ftm) {
+__device__ __forceinline__ void write_kinetic(const View &V, int p, double ftm) {
     const int n = V.n_pad;
     const double vx = V.v[p], vy = V.v[n + p], vz = V.v[2 * n + p];
+    V.ev[n + p] = 0.5 * (vx * vx + vy * vy + vz * vz) / ftm;
+}
+
+__device__ __forceinline__ void write_ev(const View &V, int p, int t, double e, const double *w, const double *s_ftm) {
+    const int n = V.n_pad;
     V.ev[p] = e;
-    V.ev[n + p] = 0.5 * (vx * vx + vy * vy + vz * vz) / s_ftm[t];
+    write_kinetic(V, p, s_ftm[t]);
     for (int k = 0; k < 6; ++k) V.ev[(2 + k) * n + p] = w[k];
 }
 
@@ -306,18 +362,10 @@ struct LJPair {
             for (int k = 0; k < 6; ++k) w[k].add(rw[k]);
         }
     }
-    // round_end with lane src's round sums (all lanes call it; use: this round exists)
-    __device__ __forceinline__ void round_from(int src, bool use) {
-        const float x = lane_value(rx, src), y = lane_value(ry, src), z = lane_value(rz, src);
-        if (use) { ax.add(x); ay.add(y); az.add(z); }
-        if (EV) {
-            const float u = lane_value(re, src);
-            if (use) e.add(u);
-            for (int k = 0; k < 6; ++k) {
-                const float q = lane_value(rw[k], src);
-                if (use) w[k].add(q);
-            }
-        }
+    // the round's sums, in the order of the wide passes' terms
+    static constexpr int kTerms = EV ? 10 : 3;
+    __device__ __forceinline__ float term(int k) const {
+        return k == 0 ? rx : k == 1 ? ry : k == 2 ? rz : k == 3 ? re : rw[k - 4];
     }
     // energy and virial terms of one pair: summed plainly over the round and
     // added with compensation per round
@@ -386,12 +434,14 @@ struct LJPair {
 // out (counted by the walk) or to add (left out by it): force, half-list
 // partner, energy and virial alike.  The terms are summed over the warp into
 // the atom's first thread.  All 32 lanes call this together.
-// (T = 0: the lanes per atom, 2^ll, are a run-time value: the wide kernels.)
-template <int T, int Q, int MT, int HALF, int EV>
+// T = 0: the wide kernels, whose lanes per atom are a run-time value and whose
+// terms go to the lanes (of the atom's first thread) that add them.
+template <int T, int Q, int MT, int HALF, int EV, int KT = 1>
 __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV> &pr, bool flagged,
-                                              int gw, int lane, int tmode, const float4 *srec, int ll = 0) {
+                                              int gw, int lane, int tmode, const float4 *srec, const Wide *w = nullptr,
+                                              KahanF *acc = nullptr) {
     constexpr bool kWide = T == 0;
-    const int L = kWide ? 1 << ll : T;  // lanes per atom
+    const int L = kWide ? 1 << (w->lt + w->lg) : T;  // lanes per atom
     const int A = 32 / L;
     unsigned m = __ballot_sync(0xffffffffu, flagged);
     while (m) {
@@ -456,7 +506,18 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV
                 for (int c = 0; c < 6; ++c) cw[c] += __shfl_xor_sync(0xffffffffu, cw[c], o);
             }
         }
-        if (lane == a * L) {
+        if constexpr (kWide) {
+            const float all[10] = {cx, cy, cz, ce, cw[0], cw[1], cw[2], cw[3], cw[4], cw[5]};
+            if (lane / L == a && w->sub == 0) {
+#pragma unroll
+                for (int k = 0; k < KT; ++k) {
+                    const int term = w->g + (k << w->lg);
+#pragma unroll
+                    for (int q = 0; q < (EV ? 10 : 3); ++q)
+                        if (term == q) acc[k].add(all[q]);
+                }
+            }
+        } else if (lane == a * T) {
             pr.ax.add(cx); pr.ay.add(cy); pr.az.add(cz);
             if (EV) {
                 pr.e.add(ce);
@@ -571,6 +632,8 @@ __global__ void __maxnreg__((LjRegs<T, Q, HALF, EV>::value)) k_lj(View V, KArgs 
 // the full-list pass of a small system (see walk_wide); a.aux = log2 of G
 template <int Q, int EV, int MT>
 __global__ void __launch_bounds__(kWideBlock) k_lj_wide(View V, KArgs a) {
+    constexpr int NT = EV ? 10 : 3, KT = (NT + 1) / 2;
+    __shared__ float s_round[kWideBlock / 32][NT][32];
     __shared__ float s_tab[5][kMaxTypes * kMaxTypes];
     if (MT) {
         for (int k = threadIdx.x; k < V.ntypes * V.ntypes; k += blockDim.x) {
@@ -579,10 +642,9 @@ __global__ void __launch_bounds__(kWideBlock) k_lj_wide(View V, KArgs a) {
         }
         __syncthreads();
     }
-    const unsigned err = V.ctl->err;
-    const int rem = (a.mode == kModeStep) ? V.ctl->remaining : 0;
     const Wide w = wide_lane(V, a.aux);
-    if (err || w.p >= V.n_pad) return;  // whole warps: n_pad is a multiple of 32
+    if (w.p >= V.n_pad) return;  // whole warps: n_pad is a multiple of 32
+    WideAtom<Q> at = load_wide<Q>(V, w);
     LJPair<MT, 0, EV> pr;
     pr.V = &V;
     pr.lj1 = s_tab[0]; pr.lj2 = s_tab[1]; pr.lj3 = s_tab[2]; pr.lj4 = s_tab[3]; pr.off = s_tab[4];
@@ -593,28 +655,26 @@ __global__ void __launch_bounds__(kWideBlock) k_lj_wide(View V, KArgs a) {
     pr.rc2 = V.rc2f;
     pr.nt = V.ntypes;
     pr.n = V.n_pad;
-    pr.ti = 0;
+    pr.ti = at.t;
     pr.near_min = 3.0e38f;
-    pr.ax.zero(); pr.ay.zero(); pr.az.zero(); pr.e.zero();
-    for (int k = 0; k < 6; ++k) pr.w[k].zero();
+    KahanF acc[KT];
+    for (int k = 0; k < KT; ++k) acc[k].zero();
+    const double ftm = V.tab->ftm_m[MT ? at.t : 0];
     const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
     const bool valid = (w.p - R.atom0) < R.natoms;
-    const int cnt = valid ? V.ncount[w.p] : 0;
-    float xi, yi, zi;
-    load_rec(V, w.p, xi, yi, zi, pr.ti);
-    walk_wide<Q>(V, w, R, cnt, xi, yi, zi, pr);
-    fix_near_warp<0, Q>(V, pr, pr.near_min < V.rc2f_band, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                        threadIdx.x & 31, 0, nullptr, w.lt + w.lg);
-    const double fx = wide_sum(w, pr.ax.value()), fy = wide_sum(w, pr.ay.value()), fz = wide_sum(w, pr.az.value());
-    double e_acc = 0.0, w_acc[6] = {0, 0, 0, 0, 0, 0};
-    if (EV) {
-        e_acc = wide_sum(w, pr.e.value());
-        for (int k = 0; k < 6; ++k) w_acc[k] = wide_sum(w, pr.w[k].value());
+    if (at.err) return;
+    walk_wide<Q, NT, KT>(V, w, R, valid ? at.count : 0, at, s_round[threadIdx.x >> 5], pr, acc);
+    fix_near_warp<0, Q, MT, 0, EV, KT>(V, pr, pr.near_min < V.rc2f_band, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                                       threadIdx.x & 31, 0, nullptr, &w, acc);
+#pragma unroll
+    for (int k = 0; k < KT; ++k) {
+        const int term = w.g + (k << w.lg);
+        const double x = wide_sum(w, acc[k].value());
+        if (!valid || w.sub != 0) continue;
+        if (term < 3) wide_finish(V, a.mode, at.remaining, term, w.p, ftm, x);
+        else if (EV && term < NT) V.ev[(size_t)(term == 3 ? 0 : term - 2) * V.n_pad + w.p] = x;
     }
-    if (valid && w.lead) {
-        epilogue(V, a.mode, rem, w.p, pr.ti, fx, fy, fz, V.tab->ftm_m);
-        if (EV) write_ev(V, w.p, pr.ti, e_acc, w_acc, V.tab->ftm_m);
-    }
+    if (EV && valid && w.sub == 0 && w.g == 0) write_kinetic(V, w.p, ftm);
 }
 
 // Cell-list force pass, no Verlet list (the alternative the paper measures
@@ -826,10 +886,8 @@ struct RhoPair {
     float rc, rc2, part;
     __device__ __forceinline__ void round_begin() { part = 0; }
     __device__ __forceinline__ void round_end() { acc.add(part); }
-    __device__ __forceinline__ void round_from(int src, bool use) {
-        const float x = lane_value(part, src);
-        if (use) acc.add(x);
-    }
+    static constexpr int kTerms = 1;
+    __device__ __forceinline__ float term(int) const { return part; }
     __device__ __forceinline__ void operator()(uint32_t, float, float, float, float r2, int) {
         const float r = r2 * rsqrtf(r2);  // branch-free: t = 0 beyond rc
         const float t = (r2 < rc2) ? rc - r : 0.f;
@@ -886,21 +944,21 @@ __global__ void __launch_bounds__(256) k_eam_rho(View V, KArgs a) {
 // the density pass of a small system (see walk_wide)
 template <int Q>
 __global__ void __launch_bounds__(kWideBlock) k_eam_rho_wide(View V, KArgs a) {
-    const unsigned err = V.ctl->err;
+    __shared__ float s_round[kWideBlock / 32][1][32];
     const Wide w = wide_lane(V, a.aux);
-    if (err || w.p >= V.n_pad) return;
+    if (w.p >= V.n_pad) return;
+    WideAtom<Q> at = load_wide<Q>(V, w);
     RhoPair pr;
-    pr.acc.zero();
     pr.rc = V.tab->eamf[0];
     pr.rc2 = V.rc2f;
     const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
     const bool valid = (w.p - R.atom0) < R.natoms;
-    float xi, yi, zi;
-    int ti;
-    load_rec(V, w.p, xi, yi, zi, ti);
-    walk_wide<Q>(V, w, R, valid ? V.ncount[w.p] : 0, xi, yi, zi, pr);
-    const double rho = wide_sum(w, pr.acc.value());
-    if (valid && w.lead) finish_rho(V, a.mode, w.p, rho);
+    if (at.err) return;
+    KahanF acc[1];
+    acc[0].zero();
+    walk_wide<Q, 1, 1>(V, w, R, valid ? at.count : 0, at, s_round[threadIdx.x >> 5], pr, acc);
+    const double rho = wide_sum(w, acc[0].value());
+    if (valid && w.sub == 0 && w.g == 0) finish_rho(V, a.mode, w.p, rho);
 }
 
 // pass 2: F_i = -sum_j [phi'(r) + (F'_i + F'_j) rho'(r)] d / r
@@ -925,18 +983,10 @@ struct EamPair {
             for (int k = 0; k < 6; ++k) w[k].add(rw[k]);
         }
     }
-    // round_end with lane src's round sums (all lanes call it; use: this round exists)
-    __device__ __forceinline__ void round_from(int src, bool use) {
-        const float x = lane_value(rx, src), y = lane_value(ry, src), z = lane_value(rz, src);
-        if (use) { ax.add(x); ay.add(y); az.add(z); }
-        if (EV) {
-            const float u = lane_value(re, src);
-            if (use) e.add(u);
-            for (int k = 0; k < 6; ++k) {
-                const float q = lane_value(rw[k], src);
-                if (use) w[k].add(q);
-            }
-        }
+    // the round's sums, in the order of the wide passes' terms
+    static constexpr int kTerms = EV ? 10 : 3;
+    __device__ __forceinline__ float term(int k) const {
+        return k == 0 ? rx : k == 1 ? ry : k == 2 ? rz : k == 3 ? re : rw[k - 4];
     }
     // wj: F'_j, which came with the record (rec.w, set by the density pass)
     __device__ __forceinline__ void operator()(uint32_t, float dx, float dy, float dz, float r2, int wj) {
@@ -1026,32 +1076,32 @@ __global__ void __launch_bounds__(256) k_eam_force(View V, KArgs a) {
 // the force pass of a small system (see walk_wide)
 template <int Q, int EV>
 __global__ void __launch_bounds__(kWideBlock) k_eam_force_wide(View V, KArgs a) {
-    const unsigned err = V.ctl->err;
-    const int rem = (a.mode == kModeStep) ? V.ctl->remaining : 0;
+    constexpr int NT = EV ? 10 : 3, KT = (NT + 1) / 2;
+    __shared__ float s_round[kWideBlock / 32][NT][32];
     const Wide w = wide_lane(V, a.aux);
-    if (err || w.p >= V.n_pad) return;
+    if (w.p >= V.n_pad) return;
+    WideAtom<Q> at = load_wide<Q>(V, w);
     EamPair<EV> pr;
     pr.rc = V.tab->eamf[0]; pr.c0 = V.tab->eamf[2]; pr.c1 = V.tab->eamf[3]; pr.c2 = V.tab->eamf[4];
     pr.rc2 = V.rc2f;
-    pr.ax.zero(); pr.ay.zero(); pr.az.zero(); pr.e.zero();
-    for (int k = 0; k < 6; ++k) pr.w[k].zero();
     const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
     const bool valid = (w.p - R.atom0) < R.natoms;
-    float xi, yi, zi;
-    int ti;
-    load_rec(V, w.p, xi, yi, zi, ti);
-    pr.fpi = __int_as_float(ti);
-    walk_wide<Q>(V, w, R, valid ? V.ncount[w.p] : 0, xi, yi, zi, pr);
-    const double fx = wide_sum(w, pr.ax.value()), fy = wide_sum(w, pr.ay.value()), fz = wide_sum(w, pr.az.value());
-    double e_acc = 0.0, w_acc[6] = {0, 0, 0, 0, 0, 0};
-    if (EV) {
-        e_acc = wide_sum(w, pr.e.value());
-        for (int k = 0; k < 6; ++k) w_acc[k] = wide_sum(w, pr.w[k].value());
+    const double ftm = V.tab->ftm_m[0];  // single element
+    if (at.err) return;
+    pr.fpi = __int_as_float(at.t);
+    KahanF acc[KT];
+    for (int k = 0; k < KT; ++k) acc[k].zero();
+    walk_wide<Q, NT, KT>(V, w, R, valid ? at.count : 0, at, s_round[threadIdx.x >> 5], pr, acc);
+#pragma unroll
+    for (int k = 0; k < KT; ++k) {
+        const int term = w.g + (k << w.lg);
+        const double x = wide_sum(w, acc[k].value());
+        if (!valid || w.sub != 0) continue;
+        if (term < 3) wide_finish(V, a.mode, at.remaining, term, w.p, ftm, x);
+        else if (EV && term == 3) V.ev[w.p] = x + V.emb[w.p];
+        else if (EV && term < NT) V.ev[(size_t)(term - 2) * V.n_pad + w.p] = x;
     }
-    if (valid && w.lead) {
-        epilogue(V, a.mode, rem, w.p, 0, fx, fy, fz, V.tab->ftm_m);
-        if (EV) write_ev(V, w.p, 0, e_acc + V.emb[w.p], w_acc, V.tab->ftm_m);
-    }
+    if (EV && valid && w.sub == 0 && w.g == 0) write_kinetic(V, w.p, ftm);
 }
 
 // ------------------------------------------------------- drift + control --
@@ -1065,12 +1115,12 @@ __global__ void __launch_bounds__(kWideBlock) k_eam_force_wide(View V, KArgs a) 
 constexpr int kDriftPer = 1;
 
 template <int PREC>
-__device__ __forceinline__ float drift_one(const View &V, int p, int first, int &rep) {
+__device__ __forceinline__ float drift_one(const View &V, int p, unsigned err, int first, int &rep) {
     const int n = V.n_pad;
-    rep = V.tile_rep[p >> 5];
+    rep = V.n_rep == 1 ? 0 : V.tile_rep[p >> 5];
     const Rep &R = V.rep[rep];
-    if ((p - R.atom0) >= R.natoms) return 0.f;
-    double x[3], v[3];
+    const int left = R.natoms - (p - R.atom0);
+    double x[3], v[3];  // (loaded before anything is known: the checks' loads would come first otherwise)
     int t;
     if (PREC == MD_PREC_FP64) {
         const double4_32a q = V.pos4[p];
@@ -1082,6 +1132,7 @@ __device__ __forceinline__ float drift_one(const View &V, int p, int first, int 
     }
     for (int c = 0; c < 3; ++c) v[c] = V.v[c * n + p];
     const float4 b = V.recb[p];
+    if (left <= 0 || err) return 0.f;  // a latched error: leave the state as it is
     if (first) {
         const double hk = 0.5 * V.dt * V.tab->ftm_m[t];
         for (int c = 0; c < 3; ++c) {
@@ -1106,19 +1157,19 @@ __device__ __forceinline__ float drift_one(const View &V, int p, int first, int 
 // mixed precision: the adjacent atoms p, p+1 (p even, same replica) with
 // 16-byte loads and stores of the FP64 arrays; the second atom may be padding,
 // which is left untouched.  Returns the larger squared displacement.
-__device__ __forceinline__ float drift_pair(const View &V, int p, int first, int &rep) {
+__device__ __forceinline__ float drift_pair(const View &V, int p, unsigned err, int first, int &rep) {
     const int n = V.n_pad;
     rep = V.n_rep == 1 ? 0 : V.tile_rep[p >> 5];
     const Rep &R = V.rep[rep];
-    const int l0 = p - R.atom0;
-    if (l0 >= R.natoms) return 0.f;
-    const bool two = l0 + 1 < R.natoms;
-    double2 x[3], v[3];
+    const int left = R.natoms - (p - R.atom0);
+    const bool two = left > 1;
+    double2 x[3], v[3];  // (loaded before anything is known: the checks' loads would come first otherwise)
     for (int c = 0; c < 3; ++c) {
         x[c] = *(const double2 *)&V.xr[c * n + p];
         v[c] = *(const double2 *)&V.v[c * n + p];
     }
     const float4 b0 = V.recb[p], b1 = V.recb[p + 1];
+    if (left <= 0 || err) return 0.f;  // a latched error: leave the state as it is
     const int2 t = make_int2(__float_as_int(b0.w), __float_as_int(b1.w));  // the build records hold the types
     if (first) {
         const double hk0 = 0.5 * V.dt * V.tab->ftm_m[t.x], hk1 = two ? 0.5 * V.dt * V.tab->ftm_m[t.y] : 0.0;
@@ -1163,10 +1214,7 @@ __global__ void __launch_bounds__(256) k_drift(View V, KArgs a) {
         const int p = 2 * (blockIdx.x * 256 + threadIdx.x);
         d2[0] = 0.f;
         rep[0] = -1;
-        if (p < V.n_pad) {
-            if (err == 0) d2[0] = drift_pair(V, p, first, rep[0]);
-            else rep[0] = V.tile_rep[p >> 5];  // a latched error: leave the state as it is
-        }
+        if (p < V.n_pad) d2[0] = drift_pair(V, p, err, first, rep[0]);
     } else {
         const int p0 = blockIdx.x * (256 * kDriftPer) + threadIdx.x;
 #pragma unroll
@@ -1174,13 +1222,7 @@ __global__ void __launch_bounds__(256) k_drift(View V, KArgs a) {
             const int p = p0 + u * 256;
             d2[u] = 0.f;
             rep[u] = -1;
-            if (p < V.n_pad) {
-                if (err == 0) {
-                    d2[u] = drift_one<PREC>(V, p, first, rep[u]);
-                } else {
-                    rep[u] = V.tile_rep[p >> 5];  // a latched error: leave the state as it is
-                }
-            }
+            if (p < V.n_pad) d2[u] = drift_one<PREC>(V, p, err, first, rep[u]);
         }
     }
 #pragma unroll
@@ -1199,7 +1241,12 @@ __global__ void __launch_bounds__(256) k_drift(View V, KArgs a) {
 // flags stay for the host's recovery) and end the loop, and the host
 // completes the step after growing the list.
 __global__ void __launch_bounds__(256) k_drift_done(View V, KArgs a) {
-    if (V.ctl->err_at_drift != 0) {
+    // everything thread 0 will need, loaded at once: one memory latency instead of four
+    const unsigned err_at_drift = V.ctl->err_at_drift, err = V.ctl->err;
+    int rem = V.ctl->remaining;
+    const long long steps = V.ctl->steps, rebuilds = V.ctl->rebuilds;
+    const unsigned m0 = (int)threadIdx.x < V.n_rep ? V.rep_disp[threadIdx.x] : 0u;
+    if (err_at_drift != 0) {
         if (threadIdx.x == 0 && a.in_graph) {
             cudaGraphSetConditional(V.cond_rebuild, 0u);
             cudaGraphSetConditional(V.cond_loop, 0u);
@@ -1209,7 +1256,7 @@ __global__ void __launch_bounds__(256) k_drift_done(View V, KArgs a) {
     int any = 0, nflag = 0;
     bool bad = false;
     for (int q = threadIdx.x; q < V.n_rep; q += blockDim.x) {
-        const unsigned m = V.rep_disp[q];
+        const unsigned m = q == (int)threadIdx.x ? m0 : V.rep_disp[q];
         V.rep_disp[q] = 0u;
         const bool nonfin = m >= 0x7f800000u;
         const int flag = (nonfin || __uint_as_float(m) > V.skin_half2f) ? 1 : 0;
@@ -1223,15 +1270,15 @@ __global__ void __launch_bounds__(256) k_drift_done(View V, KArgs a) {
     for (int o = 16; o > 0; o >>= 1) nflag += __shfl_xor_sync(0xffffffffu, nflag, o);
     if ((threadIdx.x & 31) == 0) s_n[threadIdx.x >> 5] = nflag;
     any = __syncthreads_or(any);
+    bad = __syncthreads_or(bad);
     if (threadIdx.x == 0) {
         int tot = 0;
         for (int k = 0; k < (int)(blockDim.x >> 5); ++k) tot += s_n[k];
         V.ctl->first = 0;
-        const bool ok = V.ctl->err == 0;
-        int rem = V.ctl->remaining;
+        const bool ok = err == 0 && !bad;
         if (ok) {
-            V.ctl->steps += 1;
-            V.ctl->rebuilds += tot;  // the builds this step's rebuild conditional runs
+            V.ctl->steps = steps + 1;
+            V.ctl->rebuilds = rebuilds + tot;  // the builds this step's rebuild conditional runs
             if (rem > 0) V.ctl->remaining = --rem;
         }
         if (a.in_graph) {
@@ -1315,11 +1362,10 @@ static const void *pick_eamf(int T, int Q, int ev) {
 
 // log2 of the lanes that stand in for one thread of the list layout (walk_wide): as
 // many as keep the whole system within kWideThreads threads per SM, at most
-// eight.  us per step with one lane, and with 512 / 1024 / 2048 threads per SM: 4,000
-// atoms 30.6, 24.4 (8 lanes); 16,000 atoms 30.9, 26.4 (4) / 27.7 (8); 32,771 atoms 32.7, 30.9 (2) / 30.4
-// (4) / 36.0 (8); 65,536 atoms 36.7, 37.5 (2); 8,000 atoms at four threads per atom 27.0, 26.8 (2) /
-// 29.1 (4).  16 and 32 lanes for the smallest systems: 4,000 atoms 24.8 and 26.6.
-constexpr int kWideThreads = 640, kWideMost = 3;
+// sixteen.  us per step at 512 / 640 / 880-1024 / 2048 threads per SM: 4,000
+// atoms 26.2 (8 lanes) / 26.0 (16), 16,000 atoms 28.9 (4) / 29.4 (8), 32,771 atoms 34.6 (2) / 32.5 (4) / 36
+// (8); one lane: 31 .. 33.  32 lanes for the smallest systems measured the same as 16.
+constexpr int kWideThreads = 880, kWideMost = 4;
 
 static int wide_log(const View &V) {
     int lg = 0;
