@@ -870,6 +870,18 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
     }
 }
 
+// list statistics of a replica from one warp: one atomic pair, no block barrier
+__device__ __forceinline__ void build_stats(const View &V, int rep, int my_max, long long my_sum, int lane) {
+    for (int o = 16; o > 0; o >>= 1) {
+        my_max = max(my_max, __shfl_xor_sync(0xffffffffu, my_max, o));
+        my_sum += __shfl_xor_sync(0xffffffffu, my_sum, o);
+    }
+    if (lane == 0 && rep >= 0 && my_sum > 0) {
+        atomicMax(&V.rep_maxcnt[rep], my_max);
+        atomicAdd(&V.rep_entries[rep], (unsigned long long)my_sum);
+    }
+}
+
 template <int PREC, int HALF, int NW>
 __global__ void __launch_bounds__(32 * NW, kBuildWarps / NW) k_build(View V, KArgs a) {
     const int lane = threadIdx.x & 31, w = NW == 1 ? 0 : threadIdx.x >> 5;
@@ -884,18 +896,174 @@ __global__ void __launch_bounds__(32 * NW, kBuildWarps / NW) k_build(View V, KAr
         my_rep = r;
         if (a.all || V.rep_flag[r]) build_cell<PREC, HALF, NW>(V, gb, part, V.hsplit, lane, w, my_max, my_sum);
     }
-    // statistics per replica: one atomic pair per warp, no block barrier
-    for (int o = 16; o > 0; o >>= 1) {
-        my_max = max(my_max, __shfl_xor_sync(0xffffffffu, my_max, o));
-        my_sum += __shfl_xor_sync(0xffffffffu, my_sum, o);
-    }
-    if (lane == 0 && my_rep >= 0 && my_sum > 0) {
-        atomicMax(&V.rep_maxcnt[my_rep], my_max);
-        atomicAdd(&V.rep_entries[my_rep], (unsigned long long)my_sum);
-    }
+    build_stats(V, my_rep, my_max, my_sum, lane);
     // builds of every replica (creation, md_build_neighbors, md_set_state) are
     // counted here; the step's builds of flagged replicas were counted with the
     // flags (k_drift_done), so that those launches take no ticket
+    if (a.all && last_block(&V.ctl->ticket_build)) {
+        if (threadIdx.x == 0) {
+            V.ctl->ticket_build = 0;
+            V.ctl->rebuilds += V.n_rep;
+        }
+    }
+}
+
+// The list build of a system with too few cells to fill the GPU (kRowBuild): one
+// block of nine warps per (cell, part), one warp per row of three cells.  A
+// warp alone on its scheduler takes ~8 clocks an instruction, so the ~8,000
+// instructions of a whole cell in one warp are 35 us whatever the size; here the
+// rows are tested side by side and counted, the block's warps exchange their counts,
+// and each warp then writes its row's entries behind those of the
+// rows before it: the same lists, entry by entry.  The acceptance masks and
+// entries of a row's first kRowKeep rounds are kept between the two passes, later rounds
+// (rows of more than 32 kRowKeep candidates) are tested again.
+constexpr int kRowKeep = 4;
+
+template <int PREC, int HALF>
+__global__ void __launch_bounds__(288) k_build_rows(View V, KArgs a) {
+    __shared__ __align__(16) float s_h[16][8];  // home atoms 2k, 2k + 1: {x, x, y, y}, {z, z, |x|^2, |x|^2}
+    __shared__ int s_cnt[9][32];                // accepted per row and home atom
+    __shared__ uint32_t s_t[9][kRowKeep][32], s_e[9][kRowKeep][32];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int gb = blockIdx.x / V.hsplit, part = blockIdx.x - gb * V.hsplit;
+    const int r = V.bin_rep[gb];
+    const Rep &R = V.rep[r];
+    int my_max = 0;
+    long long my_sum = 0;
+    const int hs = V.bin_start[gb], hn = (a.all || V.rep_flag[r]) ? V.bin_count[gb] : 0;  // 0: nothing to do
+    const int xyz = V.bin2xyz[gb];
+    const int dy = row % 3 - 1, dz = row / 3 - 1;
+    // the row's three cells, one lane each (the other lanes repeat the last)
+    const int nbx = R.nb[0], nby = R.nb[1], nbz = R.nb[2];
+    int cx = unpack_bx(xyz) + min(lane, 2) - 1, cy = unpack_by(xyz) + dy, cz = unpack_bz(xyz) + dz;
+    cx += (cx < 0) ? nbx : ((cx >= nbx) ? -nbx : 0);
+    cy += (cy < 0) ? nby : ((cy >= nby) ? -nby : 0);
+    cz += (cz < 0) ? nbz : ((cz >= nbz) ? -nbz : 0);
+    const int nbin = V.lin2bin[R.bin0 + (cz * nby + cy) * nbx + cx];
+    const int first = V.bin_start[nbin], count = V.bin_count[nbin];
+    const int n0 = __shfl_sync(0xffffffffu, count, 0), n1 = n0 + __shfl_sync(0xffffffffu, count, 1);
+    const int m = n1 + __shfl_sync(0xffffffffu, count, 2);
+    const uint32_t code = (uint32_t)((dz + 1) << 4 | (dy + 1) << 2);
+    const uint32_t e0 = ((uint32_t)__shfl_sync(0xffffffffu, first, 0) << 6) + code;
+    const uint32_t e1 = ((uint32_t)(__shfl_sync(0xffffffffu, first, 1) - n0) << 6) + code + 1u;
+    const uint32_t e2 = ((uint32_t)(__shfl_sync(0xffffffffu, first, 2) - n1) << 6) + code + 2u;
+    const float hx = R.hf[0], ys = dy * R.hf[1], zs = dz * R.hf[2];
+    const float rl2f = 0.5f * (V.rl2f_lo + V.rl2f_hi), margin = 0.5f * (V.rl2f_hi - V.rl2f_lo);
+    const int maxn = V.maxneigh, lt = V.ltpa, lq = V.lvec;
+    const int la = 5 - lt, ltq = lt + lq, tq = 1 << ltq;
+    for (int h0 = 32 * part; h0 < hn; h0 += 32 * V.hsplit) {
+        const int nh = min(32, hn - h0);
+        const int hbase = hs + h0;  // slot of home atom 0 of this chunk
+        __syncthreads();
+        if (row == 0) {
+            // padding far away (never accepted, never in the band)
+            float4 hr = make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.f);
+            if (lane < nh) hr = V.rec[hbase + lane];
+            float *h = s_h[lane >> 1] + (lane & 1);
+            h[0] = hr.x; h[2] = hr.y; h[4] = hr.z;
+            h[6] = hr.x * hr.x + hr.y * hr.y + hr.z * hr.z;
+        }
+        __syncthreads();
+        // candidates c0 .. c0 + 31 of the row against the home atoms: this lane's entry,
+        // and its home atom's mask of accepted candidates
+        auto round = [&](int c0, uint32_t &e) {
+            const int f = c0 + lane;
+            const bool in = f < m;
+            const bool s1 = f >= n0, s2 = f >= n1;
+            e = in ? ((uint32_t)f << 6) + (s2 ? e2 : s1 ? e1 : e0) : 0u;
+            const int j = (int)(e >> 6);
+            const float4 rj = V.rec[in ? j : hbase];
+            const float qx = in ? rj.x + (s2 ? hx : s1 ? 0.f : -hx) : -1.0e18f, qy = in ? rj.y + ys : -1.0e18f,
+                        qz = in ? rj.z + zs : -1.0e18f;
+            const float qx2 = -2.0f * qx, qy2 = -2.0f * qy, qz2 = -2.0f * qz;
+            const float q2m = qx * qx + qy * qy + qz * qz - rl2f;
+            const unsigned long long qxx = pack2(qx2, qx2), qyy = pack2(qy2, qy2), qzz = pack2(qz2, qz2),
+                                     qww = pack2(q2m, q2m);
+            unsigned acc = 0u;
+            float tmin = 3.0e38f;
+#pragma unroll 1
+            for (int hb = (nh - 1) & ~7; hb >= 0; hb -= 8) {
+#pragma unroll
+                for (int k = 6; k >= 0; k -= 2) {
+                    const ulonglong2 *h = reinterpret_cast<const ulonglong2 *>(s_h[(hb + k) >> 1]);
+                    const ulonglong2 xy = h[0], zw = h[1];
+                    const float2 t = unpack2(fma2(qxx, xy.x, fma2(qyy, xy.y, fma2(qzz, zw.x, add2(zw.y, qww)))));
+                    acc = __funnelshift_l(__float_as_uint(t.y), acc, 1);
+                    acc = __funnelshift_l(__float_as_uint(t.x), acc, 1);
+                    tmin = fmin3(tmin, fabsf(t.x), fabsf(t.y));
+                }
+            }
+            if (tmin < margin) {  // margin band: decide those pairs in FP64 (rare)
+                for (int k = 0; k < nh; ++k) {
+                    const float *h = s_h[k >> 1] + (k & 1);
+                    const float t = fmaf(qx2, h[0], fmaf(qy2, h[2], fmaf(qz2, h[4], h[6] + q2m)));
+                    if (fabsf(t) < margin) {
+                        const bool ok = in_list_fp64<PREC>(V, R, hbase + k, j, entry_dx(e), entry_dy(e), entry_dz(e));
+                        acc = ok ? (acc | (1u << k)) : (acc & ~(1u << k));
+                    }
+                }
+            }
+            const int jh = j - hbase;
+            if ((e & 63u) == kSelfCode && jh >= 0 && jh < 32) acc &= ~(1u << jh);
+            if (HALF) acc &= jh <= 0 ? 0u : (jh >= 32 ? 0xffffffffu : ((1u << jh) - 1u));
+            return warp_transpose32(acc, lane);
+        };
+        int cnt = 0;
+        for (int c0 = 0, k = 0; c0 < m; c0 += 32, ++k) {
+            uint32_t e;
+            const unsigned t = round(c0, e);
+            cnt += __popc(t);
+            if (k < kRowKeep) {
+                s_t[row][k][lane] = t;
+                s_e[row][k][lane] = e;
+            }
+        }
+        s_cnt[row][lane] = cnt;
+        __syncthreads();
+        int k0 = 0, total = 0;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const int c = s_cnt[q][lane];
+            k0 += q < row ? c : 0;
+            total += c;
+        }
+        const int p = hbase + lane;
+        uint32_t *const lbase =
+            V.nlist + (size_t)(p >> la) * (size_t)((1 << la) * maxn) + (size_t)((p & ((1 << la) - 1)) << ltq);
+        for (int c0 = 0, k = 0; c0 < m; c0 += 32, ++k) {
+            unsigned t;
+            const uint32_t *es;
+            __syncwarp();
+            if (k < kRowKeep) {
+                t = s_t[row][k][lane];
+                es = s_e[row][k];
+            } else {  // (the last kept round's entries are used up by now)
+                uint32_t e;
+                t = round(c0, e);
+                s_e[row][kRowKeep - 1][lane] = e;
+                es = s_e[row][kRowKeep - 1];
+                __syncwarp();
+            }
+            while (__any_sync(0xffffffffu, t != 0u)) {
+                if (t) {
+                    const uint32_t e = es[__ffs(t) - 1];
+                    if (k0 < maxn) lbase[((unsigned)(k0 >> ltq) << (5 + lq)) + (unsigned)(k0 & (tq - 1))] = e;
+                    ++k0;
+                    t &= t - 1u;
+                }
+            }
+        }
+        if (row == 0 && lane < nh) {
+            V.ncount[p] = min(total, maxn);
+            if (total > maxn) {
+                atomicMax(&V.ctl->need_maxneigh, total);
+                latch_error(V.ctl, kErrOverflow);
+            }
+            my_max = max(my_max, total);
+            my_sum += total;
+        }
+    }
+    if (row == 0) build_stats(V, r, my_max, my_sum, lane);
     if (a.all && last_block(&V.ctl->ticket_build)) {
         if (threadIdx.x == 0) {
             V.ctl->ticket_build = 0;
@@ -959,19 +1127,16 @@ __global__ void __launch_bounds__(32, kBuildWarps) k_build_wl(View V, KArgs a) {
         int my_max = 0;
         long long my_sum = 0;
         build_cell<PREC, HALF, 1>(V, gb, part, hs, lane, w, my_max, my_sum);
-        for (int o = 16; o > 0; o >>= 1) {
-            my_max = max(my_max, __shfl_xor_sync(0xffffffffu, my_max, o));
-            my_sum += __shfl_xor_sync(0xffffffffu, my_sum, o);
-        }
-        if (lane == 0 && my_sum > 0) {
-            const int r = V.bin_rep[gb];
-            atomicMax(&V.rep_maxcnt[r], my_max);
-            atomicAdd(&V.rep_entries[r], (unsigned long long)my_sum);
-        }
+        build_stats(V, V.bin_rep[gb], my_max, my_sum, lane);
     }
 }
 
 // ------------------------------------------------------------- dispatch ----
+
+// Systems of at most so many (cell, part) units per SM are built by rows.  us per step (a rebuild every
+// ~8): LJ 500 atoms 20.7 -> 18.7, 4,000 22.4 -> 20.1, 4,000 FP64 31.6 -> 29.3, 8,000 at rc 4.0 43.8 -> 36.9;
+// 32,771 atoms (11 units per SM) 29.3 -> 29.9, 65,536 (21) 38.1 -> 41.8.
+constexpr int kRowBuild = 6;
 
 void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &seq) {
     KArgs a{};
@@ -1004,8 +1169,14 @@ void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &
         seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * kBuildWlDeal), dim3(32), 0, a});
         return;
     }
-    const int nw = V.hsplit > 1 ? 4 : 1;
     const void *kb;
+    if (V.tile_atoms == 0 && V.nbins_total * V.hsplit <= V.n_sm * kRowBuild) {
+        kb = fp64 ? (V.half ? (const void *)k_build_rows<MD_PREC_FP64, 1> : (const void *)k_build_rows<MD_PREC_FP64, 0>)
+                  : (V.half ? (const void *)k_build_rows<MD_PREC_MIXED, 1> : (const void *)k_build_rows<MD_PREC_MIXED, 0>);
+        seq.push_back(KCall{kb, dim3(V.nbins_total * V.hsplit), dim3(288), 0, a});
+        return;
+    }
+    const int nw = V.hsplit > 1 ? 4 : 1;
     if (nw == 1)
         kb = fp64 ? (V.half ? (const void *)k_build<MD_PREC_FP64, 1, 1> : (const void *)k_build<MD_PREC_FP64, 0, 1>)
                   : (V.half ? (const void *)k_build<MD_PREC_MIXED, 1, 1> : (const void *)k_build<MD_PREC_MIXED, 0, 1>);

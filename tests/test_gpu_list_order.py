@@ -52,3 +52,20 @@ def test_capacity_grows_from_far_too_small():
     ref = oracle.neighbors(x, box, 4.3)
     with System.lj(x, np.zeros_like(x), box, cutoff=4.0, skin=0.3, dt=0.005, mass=1.0, precision="mixed", tpa=2) as s:
         assert_lists_equal(gpu_lists(*s.neighbors()), ref)
+
+
+@pytest.mark.parametrize("rc,copies", [(2.5, 60), (4.4, 130)])
+def test_row_build_equals_the_cell_build(rc, copies):
+    """A small system's lists are built by rows of cells, those of a batch with many cells by whole cells:
+    the same entries in the same order (rc 4.4: rows of more candidates than are kept between the passes)."""
+    from paper_1009_4330_gb300 import System, lj_params
+    n = 1237
+    x, box = synth.fcc_subset(n, 0.8442, 11)
+    x = synth.displace(x, box, 0.05, 12)
+    r = {"x": x, "v": np.zeros_like(x), "box": box}
+    kw = dict(params=lj_params(1.0, 1.0, 1), cutoff=rc, skin=0.3, dt=0.005, mass=1.0, precision="mixed", tpa=1)
+    for lst in ("full", "half"):
+        with System(x, r["v"], None, box, list=lst, **kw) as s:
+            solo = _neighbors(s)
+        with System.batch([r] * copies, list=lst, **kw) as b:
+            assert all(np.array_equal(a, c) for a, c in zip(_neighbors(b), solo))
