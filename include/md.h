@@ -200,6 +200,19 @@ md_status md_set_state(md_system *h, const double *x, const double *v);
 md_status md_set_params(md_system *h, const double *params);
 
 /*
+ * Forces at new parameters (host, layout of md_config.params; NULL keeps the
+ * current ones) and/or new positions (device [n][3], original order; NULL
+ * keeps them), written to f_out[n][3] (device, original order; may be NULL):
+ * md_set_params, md_set_state(x, NULL) and md_compute_forces in turn, with the
+ * forces evaluated once instead of after each and the stream synchronised
+ * once, and only if x is given (the list's overflow check).  Errors as those
+ * calls'; rejected parameters leave the handle as it was.
+ * Cite: Sec. III.B (the neighbour-list force kernels), App. A (the potentials
+ * and their parameters); one call for force-matching loops is library plumbing.
+ */
+md_status md_eval_forces(md_system *h, const double *params, const double *x, double *f_out);
+
+/*
  * Backward pass of the forces for a force-matching loss (the forces of the
  * pair-force step, App. A potentials, made differentiable): given grad_f =
  * dL/dF ([n][3], original order), write grad_x = dL/dx ([n][3], original

@@ -838,8 +838,7 @@ md_status md_set_state(md_system *h, const double *x, const double *v) {
     return compute_forces(h, kModeStoreF);
 }
 
-md_status md_set_params(md_system *h, const double *params) {
-    if (!h || !params) return fail(h, MD_ERR_INVALID, "null argument");
+static md_status check_params(md_system *h, const double *params) {
     if (h->cfg.pot == MD_POT_EAM_FS && params[0] != h->cfg.cutoff)
         return fail(h, MD_ERR_INVALID, "the EAM cut-off cannot change");
     if (h->cfg.pot == MD_POT_LJ) {
@@ -850,10 +849,47 @@ md_status md_set_params(md_system *h, const double *params) {
                     params[nt * nt + a * nt + b] != params[nt * nt + b * nt + a])
                     return fail(h, MD_ERR_INVALID, "LJ parameters must be symmetric");
     }
+    return MD_OK;
+}
+
+md_status md_set_params(md_system *h, const double *params) {
+    if (!h || !params) return fail(h, MD_ERR_INVALID, "null argument");
+    md_status st = check_params(h, params);
+    if (st) return st;
     h->params.assign(params, params + h->cfg.n_params);
-    md_status st = upload_tab(h);
+    st = upload_tab(h);
     if (st) return st;
     return compute_forces(h, kModeStoreF);
+}
+
+md_status md_eval_forces(md_system *h, const double *params, const double *x, double *f_out) {
+    if (!h) return fail(nullptr, MD_ERR_INVALID, "null handle");
+    if (params) {
+        md_status st = check_params(h, params);
+        if (st) return st;
+        h->params.assign(params, params + h->cfg.n_params);
+        // from pageable memory: the call returns once the table has been read
+        PairTab t;
+        fill_tab(h, t);
+        CK(h, cudaMemcpyAsync(h->d_tab, &t, sizeof(PairTab), cudaMemcpyHostToDevice, h->s));
+    }
+    std::vector<KCall> seq;
+    if (x) {
+        CK(h, launch_restage(h->V, x, nullptr, h->s));
+        rebuild_sequence(h->V, true, true, seq);
+    }
+    force_sequence(h->V, kModeStoreF, h->block, false, seq);
+    CK(h, run_seq(h, seq));
+    if (f_out) CK(h, launch_state_out(h->V, nullptr, nullptr, f_out, h->s));
+    if (!x) return MD_OK;
+    // the force pass skipped itself if the build overflowed the list
+    Ctl c;
+    md_status st = read_ctl(h, &c);
+    if (st) return st;
+    if (!c.err) return MD_OK;
+    st = settle_overflow(h, true);
+    if (st) return st;
+    return md_compute_forces(h, f_out);
 }
 
 md_status md_forces_backward(md_system *h, const double *grad_f, double *grad_x, double *grad_params) {

@@ -232,6 +232,17 @@ class System:
         self._version += 1
         self._call("md_set_params", p.ctypes.data_as(ctypes.POINTER(ctypes.c_double)))
 
+    def eval_forces(self, params=None, x=None, out=None):
+        """Forces (n,3) at new parameters and/or positions, which the system keeps: set_params,
+        set_state(x=x) and compute_forces in one call, the forces evaluated once."""
+        f = out if out is not None else torch.empty((self.n, 3), dtype=torch.float64, device="cuda")
+        p = np.ascontiguousarray(params, dtype=np.float64).ravel() if params is not None else None
+        xd = _dev(x, torch.float64, (-1, 3)) if x is not None else None
+        self._version += 1
+        self._call("md_eval_forces", p.ctypes.data_as(ctypes.POINTER(ctypes.c_double)) if p is not None else None,
+                   _ptr(xd), _ptr(f))
+        return f
+
     def backward(self, grad_f):
         """dL/dx (n,3) and dL/dparams (ABI layout: 2 n_types^2 for LJ; 5 for EAM, the cut-off slot 0)
         for dL/dF = grad_f."""
@@ -390,6 +401,15 @@ def pairs_to_matrix(vals, nt):
     return m
 
 
+def _to_host(a, b):
+    """Two tensors as float64 numpy arrays, by one copy if they are on one GPU."""
+    a, b = a.detach(), b.detach()
+    if a.is_cuda and a.device == b.device:
+        both = torch.cat([a.double().reshape(-1), b.double().reshape(-1)]).cpu().numpy()
+        return both[:a.numel()], both[a.numel():]
+    return a.cpu().double().numpy(), b.cpu().double().numpy()
+
+
 def _check_fresh(ctx):
     """The backward kernels differentiate at the system's CURRENT positions and
     parameters: refuse if they changed after this forward (a step, set_state,
@@ -406,19 +426,16 @@ class LJForces(torch.autograd.Function):
     eps_pairs / sig_pairs: one entry per unordered type pair (upper triangle,
     row-major: AA, AB, BB for two types), any float dtype, learnable.  x (n,3)
     may be None to keep the system's positions (then no gradient for x).
-    Forward sets the parameters (and positions, which rebuilds the list),
-    runs the force kernel; backward runs the library's backward kernel.
+    Forward sets the parameters (and positions, which rebuilds the list) and
+    runs the force kernel in one call; backward runs the library's backward kernel.
     """
 
     @staticmethod
     def forward(ctx, system, x, eps_pairs, sig_pairs):
         nt = system.n_types
-        e = pairs_to_matrix(eps_pairs.detach().cpu().double().numpy(), nt)
-        s = pairs_to_matrix(sig_pairs.detach().cpu().double().numpy(), nt)
-        system.set_params(lj_params(e, s, nt))
-        if x is not None:
-            system.set_state(x=x.detach())
-        f = system.compute_forces()
+        e, s = _to_host(eps_pairs, sig_pairs)
+        params = lj_params(pairs_to_matrix(e, nt), pairs_to_matrix(s, nt), nt)
+        f = system.eval_forces(params, x.detach() if x is not None else None)
         ctx.system = system
         ctx.version = system.version
         ctx.has_x = x is not None
@@ -432,12 +449,15 @@ class LJForces(torch.autograd.Function):
         _check_fresh(ctx)
         nt = system.n_types
         gx, gp = system.backward(grad_f.contiguous())
-        gp = gp.cpu().numpy()
-        ge = np.array([gp[a * nt + b] for a in range(nt) for b in range(a, nt)])
-        gs = np.array([gp[nt * nt + a * nt + b] for a in range(nt) for b in range(a, nt)])
         edt, sdt, edev, sdev = ctx.p_dtype
-        ge_t = torch.as_tensor(ge, dtype=edt, device=edev)
-        gs_t = torch.as_tensor(gs, dtype=sdt, device=sdev)
+        # the unordered pairs' entries (both places hold the derivative), picked where the gradients are
+        upper = torch.triu_indices(nt, nt)
+        at = upper[0] * nt + upper[1]
+        if edev.type == "cpu" and sdev.type == "cpu":
+            gp = gp.cpu()
+        at = at.to(gp.device, non_blocking=True)
+        ge_t = gp[:nt * nt].index_select(0, at).to(dtype=edt, device=edev)
+        gs_t = gp[nt * nt:].index_select(0, at).to(dtype=sdt, device=sdev)
         gxo = gx.to(ctx.x_dtype) if ctx.has_x else None
         return None, gxo, ge_t, gs_t
 
@@ -456,10 +476,7 @@ class EAMForces(torch.autograd.Function):
     def forward(ctx, system, x, params):
         if system.potential != "eam":
             raise MDError(int(L.MD_ERR_INVALID), "EAMForces needs an EAM system")
-        system.set_params(params.detach().cpu().double().numpy())
-        if x is not None:
-            system.set_state(x=x.detach())
-        f = system.compute_forces()
+        f = system.eval_forces(params.detach().cpu().double().numpy(), x.detach() if x is not None else None)
         ctx.system = system
         ctx.version = system.version
         ctx.has_x = x is not None
