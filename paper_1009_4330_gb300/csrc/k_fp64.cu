@@ -407,10 +407,24 @@ __global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsMany) k64_eam_rho(View 
     });
 }
 
+// The pair function about its own cut-off: with t = rc - r, phi = t^2 (p0 + p1 t + p2 t^2),
+//   phi' = -t (2 p0 + 3 p1 t + 4 p2 t^2),  phi'' = 2 (p0 + 3 p1 t + 6 p2 t^2),
+// two FP64 instructions each instead of five for phi' and eight for both from the
+// polynomial in r and its derivative.
+struct EamPoly {
+    double p0, p1, p2;
+    __device__ __forceinline__ explicit EamPoly(const PairTab *tab) {
+        const double rc = tab->eam[0], c0 = tab->eam[2], c1 = tab->eam[3], c2 = tab->eam[4];
+        p0 = fma(rc, fma(rc, c2, c1), c0);
+        p1 = -fma(2.0 * rc, c2, c1);
+        p2 = c2;
+    }
+};
+
 template <int EV>
 struct Eam64 {
     double ax, ay, az, e, w[6];
-    double rc, rc2, c0, c1, c2, c2x2, fpi;
+    double rc, rc2, p0, p1, p2, d0, d1, d2, fpi;  // d: 2 p0, 3 p1, 4 p2
     __device__ __forceinline__ void begin(const View &V, int p) {
         ax = 0.0; ay = 0.0; az = 0.0;
         if (EV) {
@@ -427,10 +441,8 @@ struct Eam64 {
         const double rinv = rsqrt64(r2);
         const double r = r2 * rinv;
         const double t = rc - r;
-        const double poly = fma(r, fma(r, c2, c1), c0);
-        const double dpoly = fma(c2x2, r, c1);
-        // -(phi' + (F'_i + F'_j) rho') / r with phi' = -2t poly + t^2 dpoly, rho' = -2t
-        double coef = -t * fma(-2.0, poly + (fpi + fpj), t * dpoly) * rinv;
+        // -(phi' + (F'_i + F'_j) rho') / r with rho' = -2t
+        double coef = t * fma(2.0, fpi + fpj, fma(t, fma(t, d2, d1), d0)) * rinv;
         coef = in ? coef : 0.0;
         if (!EV) {
             ax = fma(dx, coef, ax); ay = fma(dy, coef, ay); az = fma(dz, coef, az);
@@ -438,7 +450,7 @@ struct Eam64 {
         }
         const double fx = dx * coef, fy = dy * coef, fz = dz * coef;
         ax += fx; ay += fy; az += fz;
-        e += in ? t * t * poly : 0.0;
+        e += in ? t * t * fma(t, fma(t, p2, p1), p0) : 0.0;
         w[0] = fma(dx, fx, w[0]); w[1] = fma(dy, fy, w[1]); w[2] = fma(dz, fz, w[2]);
         w[3] = fma(dx, fy, w[3]); w[4] = fma(dx, fz, w[4]); w[5] = fma(dy, fz, w[5]);
     }
@@ -460,8 +472,9 @@ __global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_eam_force(View
     Eam64<EV> pr{};
     pr.rc = V.tab->eam[0];
     pr.rc2 = V.rc2;
-    pr.c0 = V.tab->eam[2]; pr.c1 = V.tab->eam[3]; pr.c2 = V.tab->eam[4];
-    pr.c2x2 = 2.0 * pr.c2;
+    const EamPoly poly(V.tab);
+    pr.p0 = poly.p0; pr.p1 = poly.p1; pr.p2 = poly.p2;
+    pr.d0 = 2.0 * poly.p0; pr.d1 = 3.0 * poly.p1; pr.d2 = 4.0 * poly.p2;
     const double ftm = V.tab->ftm_m[0];  // single element
     for_batches(V, [&](int p0, int nb, const Rep &R) {
         fp64_walk<SrcPos4, Q, U>(V, R, p0, nb, smem, pr);
@@ -504,9 +517,9 @@ __global__ void k_bwd_pack(View V, const double *grad_f) {
 
 // dL/dx of a batch's atoms, straight to the caller's order
 __device__ __forceinline__ void grad_out(const View &V, const Rep &R, int p0, int nb, const char *smem,
-                                         double *grad_x) {
+                                         double *grad_x, double sign = 1.0) {
     if (!grad_x) return;
-    for_sums(3, nb, [&](int s, int i) { grad_x[3 * (R.orig0 + V.id[p0 + i]) + s] = lane_total(smem, s, i); });
+    for_sums(3, nb, [&](int s, int i) { grad_x[3 * (R.orig0 + V.id[p0 + i]) + s] = sign * lane_total(smem, s, i); });
 }
 
 // LJ.  dL/dx_i = sum_j M_ij (g_i - g_j),  M = s(r) I + (s'(r)/r) d d^T, s = -U'(r)/r.
@@ -633,7 +646,7 @@ __global__ void __launch_bounds__(512) k_gp_reduce(View V, int nblocks, double *
 // r = |d|, u = d/r, G = g_i - g_j, w = G.u, s = phi' + (F'_i + F'_j) rho' and
 // k = phi'' + (F'_i + F'_j) rho'':
 //   pass 1: rho_i and lambda_i = sum_j w rho'(r); then F'_i, mu_i = lambda_i F''(rho_i)
-//           (into the record's free fields) and the atom's share -lambda_i dF'_i/dA of dL/dA;
+//           (kept as -2 mu_i) and the atom's share -lambda_i dF'_i/dA of dL/dA;
 //   pass 2: dL/dx_i = -sum_j [(s/r) G + (w (k - s/r) + (mu_i + mu_j) rho') u]
 //           and dL/dc_q = -sum_j (g_i.u) dphi'/dc_q, where (as for LJ) half of w
 //           stands for g_i.u over the two orders of a pair.
@@ -680,7 +693,7 @@ __global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_eam_bwd1(View 
             const double rho = lane_total(smem, 0, threadIdx.x), lam = -2.0 * lane_total(smem, 1, threadIdx.x);
             const double sq = rho > 0.0 ? sqrt(rho) : 0.0;
             V.bw[p] = rho > 0.0 ? -0.5 * Aem / sq : 0.0;
-            V.bw[n + p] = rho > 0.0 ? lam * (0.25 * Aem / (rho * sq)) : 0.0;
+            V.bw[n + p] = rho > 0.0 ? -2.0 * lam * (0.25 * Aem / (rho * sq)) : 0.0;
             partA += rho > 0.0 ? lam * (0.5 / sq) : 0.0;
         }
     });
@@ -691,7 +704,7 @@ __global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_eam_bwd1(View 
 struct EamBwd2 {
     double gx, gy, gz, g0, g1, g2;
     double gix, giy, giz, fpi, mui;
-    double rc, rc2, c0, c1, c2, c2x2;
+    double rc, rc2, d0, d1, d2, q0, q1, q2;  // d: 2 p0, 3 p1, 4 p2 (phi'); q: 2 p0, 6 p1, 12 p2 (phi'')
     __device__ __forceinline__ void begin(const View &V, int p) {
         gx = 0.0; gy = 0.0; gz = 0.0;
         const double4_32a g = V.bpack[2 * (size_t)p + 1];
@@ -712,18 +725,17 @@ struct EamBwd2 {
         const double t = rc - r;
         const double Gx = gix - gj.x, Gy = giy - gj.y, Gz = giz - gj.z;
         const double w = fma(Gz, dz, fma(Gy, dy, Gx * dx)) * ir;  // G.u
-        const double P = fma(r, fma(r, c2, c1), c0), tdP = t * fma(c2x2, r, c1);
-        const double m = fma(-2.0, P, tdP);  // phi' = t m
-        // phi'' = 2P - 4 t dP + 2 c2 t^2
-        const double d2phi = fma(c2x2 * t, t, fma(-3.0, tdP, -m));
+        const double m = fma(t, fma(t, d2, d1), d0);      // phi' = -t m
+        const double d2phi = fma(t, fma(t, q2, q1), q0);
         const double fs = fpi + fpj;
-        const double sir = t * fma(-2.0, fs, m) * ir;    // s / r
+        const double tir = t * ir;
+        const double sir = -tir * fma(2.0, fs, m);       // s / r
         const double kv = fma(2.0, fs, d2phi);
-        const double t2 = -2.0 * t;                      // rho'
-        const double b = fma(t2, mui + muj, w * (kv - sir)) * ir;
-        gx -= fma(sir, Gx, b * dx);
-        gy -= fma(sir, Gy, b * dy);
-        gz -= fma(sir, Gz, b * dz);
+        // (w (k - s/r) + (mu_i + mu_j) rho') / r with rho' = -2t; the pass before left -2 mu
+        const double b = fma(w, kv - sir, t * (mui + muj)) * ir;
+        gx = fma(sir, Gx, fma(b, dx, gx));
+        gy = fma(sir, Gy, fma(b, dy, gy));
+        gz = fma(sir, Gz, fma(b, dz, gz));
         // dphi'/dc = (-2t, t (t - 2r), 2 r t (t - r)), with t = rc - r
         const double wt = w * t;
         g0 += wt;
@@ -741,11 +753,12 @@ __global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_eam_bwd2(View 
     EamBwd2 pr{};
     pr.rc = V.tab->eam[0];
     pr.rc2 = pr.rc * pr.rc;
-    pr.c0 = V.tab->eam[2]; pr.c1 = V.tab->eam[3]; pr.c2 = V.tab->eam[4];
-    pr.c2x2 = 2.0 * pr.c2;
+    const EamPoly poly(V.tab);
+    pr.d0 = 2.0 * poly.p0; pr.d1 = 3.0 * poly.p1; pr.d2 = 4.0 * poly.p2;
+    pr.q0 = 2.0 * poly.p0; pr.q1 = 6.0 * poly.p1; pr.q2 = 12.0 * poly.p2;
     for_batches(V, [&](int p0, int nb, const Rep &R) {
         fp64_walk<SrcPack, Q, U>(V, R, p0, nb, smem, pr);
-        grad_out(V, R, p0, nb, smem, grad_x);
+        grad_out(V, R, p0, nb, smem, grad_x, -1.0);
     });
     const double g0 = warp_sum(pr.g0), g1 = warp_sum(-0.5 * pr.g1), g2 = warp_sum(-pr.g2);
     if (threadIdx.x == 0) {

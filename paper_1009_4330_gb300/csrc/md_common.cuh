@@ -148,7 +148,7 @@ struct View {
     double *ev_seg;       // [kEvSegments][8] partial sums of segments of a replica's tiles
     // backward
     double4_32a *bpack;   // [n_pad][2] x, y, z, type | dL/dF, 0
-    double *bw;           // [2][n_pad] EAM backward: F'(rho_i), mu_i = lambda_i F''(rho_i)
+    double *bw;           // [2][n_pad] EAM backward: F'(rho_i), -2 mu_i with mu_i = lambda_i F''(rho_i)
     double *gp_part;      // per block partial parameter gradients
     // block-local lists (tile_atoms = 0: every list entry holds a slot)
     int tile_atoms, n_ftiles;
