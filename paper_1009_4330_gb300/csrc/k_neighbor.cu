@@ -8,6 +8,8 @@
 // for cache reuse (Sec. III.B, texture-cache discussion).  The build
 // algorithm itself is not described there; this one bins atoms into cells of
 // edge >= cutoff + skin and scans the 27 surrounding cells.
+#include <algorithm>
+
 #include "md_common.cuh"
 #include "md_kernels.h"
 
@@ -576,7 +578,8 @@ constexpr int kBuf = 36;    // rows of the append buffer: a multiple of 4, >= 3 
 // memory there is no room for more, and at 64 registers the loops spill (work-list build: 735
 // against 702 us per step of 512 replicas).
 constexpr int kBuildWarps = 28;
-// blocks of the work-list build per resident one: a finer deal (702 -> 696 us)
+// blocks of the work-list build per resident one: a finer deal (702 -> 696 us), where the
+// batch has the cells for it (some tenth of the replicas rebuild in a step)
 constexpr int kBuildWlDeal = 4;
 
 template <int PREC, int HALF, int NW>
@@ -1166,7 +1169,8 @@ void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &
     if (wl) {
         const void *kb = fp64 ? (V.half ? (const void *)k_build_wl<MD_PREC_FP64, 1> : (const void *)k_build_wl<MD_PREC_FP64, 0>)
                               : (V.half ? (const void *)k_build_wl<MD_PREC_MIXED, 1> : (const void *)k_build_wl<MD_PREC_MIXED, 0>);
-        seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * kBuildWlDeal), dim3(32), 0, a});
+        seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * std::min(kBuildWlDeal, 1 + V.nbins_total / (V.n_sm * kBuildWarps * 4))), dim3(32), 0,
+                            a});
         return;
     }
     const void *kb;
