@@ -18,6 +18,8 @@
 // adds the round sum with Kahan compensation (forces, energy and virial
 // alike), and folds the compensated sums into FP64 for the group reduction,
 // kick and store.
+#include <cooperative_groups.h>
+
 #include "md_common.cuh"
 #include "md_kernels.h"
 
@@ -27,6 +29,11 @@ namespace md {
 
 __device__ __forceinline__ void load_rec(const View &V, int j, float &x, float &y, float &z, int &t) {
     const float4 r = __ldg(&V.rec[j]);
+    x = r.x; y = r.y; z = r.z; t = __float_as_int(r.w);
+}
+// the same by an ordinary load: where the records change during the kernel (k_steps)
+__device__ __forceinline__ void load_rec_now(const View &V, int j, float &x, float &y, float &z, int &t) {
+    const float4 r = V.rec[j];
     x = r.x; y = r.y; z = r.z; t = __float_as_int(r.w);
 }
 __device__ __forceinline__ float rcp32(float x) {
@@ -159,12 +166,12 @@ struct Wide {
     int sub, g;   // its thread of the atom's T, its lane of that thread's G
 };
 
-__device__ __forceinline__ Wide wide_lane(const View &V, int lg) {
+// lane of the pass's warp number gw
+__device__ __forceinline__ Wide wide_lane(const View &V, int lg, int gw) {
     Wide w;
     w.lt = V.ltpa;
     w.lg = lg;
     const int ll = w.lt + lg, lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     w.p = (gw << (5 - ll)) + (lane >> ll);
     const int i = lane & ((1 << ll) - 1);
     w.sub = i >> lg;
@@ -198,7 +205,7 @@ __device__ __forceinline__ WideAtom<Q> load_wide(const View &V, const Wide &w) {
     a.lp = V.nlist + (size_t)(w.p >> la) * ((size_t)V.maxneigh << la) +
            (size_t)(((w.p & ((1 << la) - 1)) << w.lt) + w.sub) * Q;
     if (w.g < (V.maxneigh >> w.lt) / Q) load_entries<Q>(a.lp + (size_t)w.g * 32 * Q, a.cur);
-    load_rec(V, w.p, a.x, a.y, a.z, a.t);
+    load_rec_now(V, w.p, a.x, a.y, a.z, a.t);
     a.count = V.ncount[w.p];
     a.err = V.ctl->err;
     a.remaining = V.ctl->remaining;
@@ -226,7 +233,7 @@ __device__ __forceinline__ void walk_wide(const View &V, const Wide &w, const Re
         int tj[Q];
 #pragma unroll
         for (int q = 0; q < Q; ++q)
-            if (q < left) load_rec(V, entry_j(cur[q]), xj[q], yj[q], zj[q], tj[q]);
+            if (q < left) load_rec_now(V, entry_j(cur[q]), xj[q], yj[q], zj[q], tj[q]);
         pair.round_begin();
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
@@ -452,7 +459,8 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV
         const int cnt = V.ncount[p];
         float xi, yi, zi;
         int ti;
-        load_rec(V, p, xi, yi, zi, ti);
+        if constexpr (kWide) load_rec_now(V, p, xi, yi, zi, ti);
+        else load_rec(V, p, xi, yi, zi, ti);
         const float hx = R.hf[0], hy4 = R.hf[1] * 0.25f, hz16 = R.hf[2] * 0.0625f;
         const uint32_t *base = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + a * L * Q;
         float cx = 0.f, cy = 0.f, cz = 0.f, ce = 0.f, cw[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -464,6 +472,8 @@ __device__ __forceinline__ void fix_near_warp(const View &V, LJPair<MT, HALF, EV
             if (tmode == 1) {
                 const float4 r4 = srec[entry_j(e) & (kTileCap - 1)];
                 xj = r4.x; yj = r4.y; zj = r4.z; tj = __float_as_int(r4.w);
+            } else if constexpr (kWide) {
+                load_rec_now(V, entry_j(e), xj, yj, zj, tj);
             } else {
                 load_rec(V, entry_j(e), xj, yj, zj, tj);
             }
@@ -629,29 +639,40 @@ __global__ void __maxnreg__((LjRegs<T, Q, HALF, EV>::value)) k_lj(View V, KArgs 
     }
 }
 
-// the full-list pass of a small system (see walk_wide); a.aux = log2 of G
-template <int Q, int EV, int MT>
-__global__ void __launch_bounds__(kWideBlock) k_lj_wide(View V, KArgs a) {
-    constexpr int NT = EV ? 10 : 3, KT = (NT + 1) / 2;
-    __shared__ float s_round[kWideBlock / 32][NT][32];
-    __shared__ float s_tab[5][kMaxTypes * kMaxTypes];
+// Coefficients of an LJ wide pass: the tables of several types in shared memory
+template <int MT>
+struct WideTab {
+    const float *lj1, *lj2, *lj3, *lj4, *off;
+    float c1, c2, c3, c4, c0;
+};
+
+// stage (several types; ends with a block barrier) or load the coefficients
+template <int MT>
+__device__ __forceinline__ WideTab<MT> wide_tab(const View &V, float (*s_tab)[kMaxTypes * kMaxTypes]) {
+    WideTab<MT> t;
     if (MT) {
         for (int k = threadIdx.x; k < V.ntypes * V.ntypes; k += blockDim.x) {
             s_tab[0][k] = V.tab->lj1f[k]; s_tab[1][k] = V.tab->lj2f[k];
             s_tab[2][k] = V.tab->lj3f[k]; s_tab[3][k] = V.tab->lj4f[k]; s_tab[4][k] = V.tab->offf[k];
         }
         __syncthreads();
+        t.lj1 = s_tab[0]; t.lj2 = s_tab[1]; t.lj3 = s_tab[2]; t.lj4 = s_tab[3]; t.off = s_tab[4];
+    } else {
+        t.c1 = V.tab->lj1f[0]; t.c2 = V.tab->lj2f[0];
+        t.c3 = V.tab->lj3f[0]; t.c4 = V.tab->lj4f[0]; t.c0 = V.tab->offf[0];
     }
-    const Wide w = wide_lane(V, a.aux);
-    if (w.p >= V.n_pad) return;  // whole warps: n_pad is a multiple of 32
-    WideAtom<Q> at = load_wide<Q>(V, w);
+    return t;
+}
+
+// one warp's atoms of the full-list pass (gw: the warp's number); all 32 lanes
+template <int Q, int EV, int MT>
+__device__ __forceinline__ void lj_wide_warp(const View &V, int mode, int rem, int gw, const Wide &w, WideAtom<Q> &at,
+                                             const Rep &R, const WideTab<MT> &tab, float (*s_round)[32]) {
+    constexpr int NT = EV ? 10 : 3, KT = (NT + 1) / 2;
     LJPair<MT, 0, EV> pr;
     pr.V = &V;
-    pr.lj1 = s_tab[0]; pr.lj2 = s_tab[1]; pr.lj3 = s_tab[2]; pr.lj4 = s_tab[3]; pr.off = s_tab[4];
-    if (!MT) {
-        pr.c1 = V.tab->lj1f[0]; pr.c2 = V.tab->lj2f[0];
-        pr.c3 = V.tab->lj3f[0]; pr.c4 = V.tab->lj4f[0]; pr.c0 = V.tab->offf[0];
-    }
+    pr.lj1 = tab.lj1; pr.lj2 = tab.lj2; pr.lj3 = tab.lj3; pr.lj4 = tab.lj4; pr.off = tab.off;
+    pr.c1 = tab.c1; pr.c2 = tab.c2; pr.c3 = tab.c3; pr.c4 = tab.c4; pr.c0 = tab.c0;
     pr.rc2 = V.rc2f;
     pr.nt = V.ntypes;
     pr.n = V.n_pad;
@@ -660,21 +681,33 @@ __global__ void __launch_bounds__(kWideBlock) k_lj_wide(View V, KArgs a) {
     KahanF acc[KT];
     for (int k = 0; k < KT; ++k) acc[k].zero();
     const double ftm = V.tab->ftm_m[MT ? at.t : 0];
-    const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
     const bool valid = (w.p - R.atom0) < R.natoms;
-    if (at.err) return;
-    walk_wide<Q, NT, KT>(V, w, R, valid ? at.count : 0, at, s_round[threadIdx.x >> 5], pr, acc);
-    fix_near_warp<0, Q, MT, 0, EV, KT>(V, pr, pr.near_min < V.rc2f_band, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                                       threadIdx.x & 31, 0, nullptr, &w, acc);
+    walk_wide<Q, NT, KT>(V, w, R, valid ? at.count : 0, at, s_round, pr, acc);
+    fix_near_warp<0, Q, MT, 0, EV, KT>(V, pr, pr.near_min < V.rc2f_band, gw, threadIdx.x & 31, 0, nullptr, &w, acc);
 #pragma unroll
     for (int k = 0; k < KT; ++k) {
         const int term = w.g + (k << w.lg);
         const double x = wide_sum(w, acc[k].value());
         if (!valid || w.sub != 0) continue;
-        if (term < 3) wide_finish(V, a.mode, at.remaining, term, w.p, ftm, x);
+        if (term < 3) wide_finish(V, mode, rem, term, w.p, ftm, x);
         else if (EV && term < NT) V.ev[(size_t)(term == 3 ? 0 : term - 2) * V.n_pad + w.p] = x;
     }
     if (EV && valid && w.sub == 0 && w.g == 0) write_kinetic(V, w.p, ftm);
+}
+
+// the full-list pass of a small system (see walk_wide); a.aux = log2 of G
+template <int Q, int EV, int MT>
+__global__ void __launch_bounds__(kWideBlock) k_lj_wide(View V, KArgs a) {
+    __shared__ float s_round[kWideBlock / 32][EV ? 10 : 3][32];
+    __shared__ float s_tab[5][kMaxTypes * kMaxTypes];
+    const WideTab<MT> tab = wide_tab<MT>(V, s_tab);
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const Wide w = wide_lane(V, a.aux, gw);
+    if (w.p >= V.n_pad) return;  // whole warps: n_pad is a multiple of 32
+    WideAtom<Q> at = load_wide<Q>(V, w);
+    const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
+    if (at.err) return;
+    lj_wide_warp<Q, EV, MT>(V, a.mode, at.remaining, gw, w, at, R, tab, s_round[threadIdx.x >> 5]);
 }
 
 // Cell-list force pass, no Verlet list (the alternative the paper measures
@@ -941,24 +974,31 @@ __global__ void __launch_bounds__(256) k_eam_rho(View V, KArgs a) {
     if (valid && sub == 0) finish_rho(V, a.mode, p, rho);
 }
 
+// one warp's atoms of the density pass
+template <int Q>
+__device__ __forceinline__ void rho_wide_warp(const View &V, int mode, const Wide &w, WideAtom<Q> &at, const Rep &R,
+                                              float (*s_round)[32]) {
+    RhoPair pr;
+    pr.rc = V.tab->eamf[0];
+    pr.rc2 = V.rc2f;
+    const bool valid = (w.p - R.atom0) < R.natoms;
+    KahanF acc[1];
+    acc[0].zero();
+    walk_wide<Q, 1, 1>(V, w, R, valid ? at.count : 0, at, s_round, pr, acc);
+    const double rho = wide_sum(w, acc[0].value());
+    if (valid && w.sub == 0 && w.g == 0) finish_rho(V, mode, w.p, rho);
+}
+
 // the density pass of a small system (see walk_wide)
 template <int Q>
 __global__ void __launch_bounds__(kWideBlock) k_eam_rho_wide(View V, KArgs a) {
     __shared__ float s_round[kWideBlock / 32][1][32];
-    const Wide w = wide_lane(V, a.aux);
+    const Wide w = wide_lane(V, a.aux, (blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (w.p >= V.n_pad) return;
     WideAtom<Q> at = load_wide<Q>(V, w);
-    RhoPair pr;
-    pr.rc = V.tab->eamf[0];
-    pr.rc2 = V.rc2f;
     const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
-    const bool valid = (w.p - R.atom0) < R.natoms;
     if (at.err) return;
-    KahanF acc[1];
-    acc[0].zero();
-    walk_wide<Q, 1, 1>(V, w, R, valid ? at.count : 0, at, s_round[threadIdx.x >> 5], pr, acc);
-    const double rho = wide_sum(w, acc[0].value());
-    if (valid && w.sub == 0 && w.g == 0) finish_rho(V, a.mode, w.p, rho);
+    rho_wide_warp<Q>(V, a.mode, w, at, R, s_round[threadIdx.x >> 5]);
 }
 
 // pass 2: F_i = -sum_j [phi'(r) + (F'_i + F'_j) rho'(r)] d / r
@@ -1073,35 +1113,42 @@ __global__ void __launch_bounds__(256) k_eam_force(View V, KArgs a) {
     }
 }
 
-// the force pass of a small system (see walk_wide)
+// one warp's atoms of the force pass
 template <int Q, int EV>
-__global__ void __launch_bounds__(kWideBlock) k_eam_force_wide(View V, KArgs a) {
+__device__ __forceinline__ void eam_wide_warp(const View &V, int mode, int rem, const Wide &w, WideAtom<Q> &at,
+                                              const Rep &R, float (*s_round)[32]) {
     constexpr int NT = EV ? 10 : 3, KT = (NT + 1) / 2;
-    __shared__ float s_round[kWideBlock / 32][NT][32];
-    const Wide w = wide_lane(V, a.aux);
-    if (w.p >= V.n_pad) return;
-    WideAtom<Q> at = load_wide<Q>(V, w);
     EamPair<EV> pr;
     pr.rc = V.tab->eamf[0]; pr.c0 = V.tab->eamf[2]; pr.c1 = V.tab->eamf[3]; pr.c2 = V.tab->eamf[4];
     pr.rc2 = V.rc2f;
-    const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
     const bool valid = (w.p - R.atom0) < R.natoms;
     const double ftm = V.tab->ftm_m[0];  // single element
-    if (at.err) return;
     pr.fpi = __int_as_float(at.t);
     KahanF acc[KT];
     for (int k = 0; k < KT; ++k) acc[k].zero();
-    walk_wide<Q, NT, KT>(V, w, R, valid ? at.count : 0, at, s_round[threadIdx.x >> 5], pr, acc);
+    walk_wide<Q, NT, KT>(V, w, R, valid ? at.count : 0, at, s_round, pr, acc);
 #pragma unroll
     for (int k = 0; k < KT; ++k) {
         const int term = w.g + (k << w.lg);
         const double x = wide_sum(w, acc[k].value());
         if (!valid || w.sub != 0) continue;
-        if (term < 3) wide_finish(V, a.mode, at.remaining, term, w.p, ftm, x);
+        if (term < 3) wide_finish(V, mode, rem, term, w.p, ftm, x);
         else if (EV && term == 3) V.ev[w.p] = x + V.emb[w.p];
         else if (EV && term < NT) V.ev[(size_t)(term - 2) * V.n_pad + w.p] = x;
     }
     if (EV && valid && w.sub == 0 && w.g == 0) write_kinetic(V, w.p, ftm);
+}
+
+// the force pass of a small system (see walk_wide)
+template <int Q, int EV>
+__global__ void __launch_bounds__(kWideBlock) k_eam_force_wide(View V, KArgs a) {
+    __shared__ float s_round[kWideBlock / 32][EV ? 10 : 3][32];
+    const Wide w = wide_lane(V, a.aux, (blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (w.p >= V.n_pad) return;
+    WideAtom<Q> at = load_wide<Q>(V, w);
+    const Rep &R = V.rep[V.n_rep == 1 ? 0 : V.tile_rep[w.p >> 5]];
+    if (at.err) return;
+    eam_wide_warp<Q, EV>(V, a.mode, at.remaining, w, at, R, s_round[threadIdx.x >> 5]);
 }
 
 // ------------------------------------------------------- drift + control --
@@ -1288,6 +1335,94 @@ __global__ void __launch_bounds__(256) k_drift_done(View V, KArgs a) {
     }
 }
 
+// Whole md_step steps of a small mixed system in one launch: a cluster of
+// kStepsCtas blocks drifts, checks the displacements and evaluates forces step after
+// step, with the cluster's hardware barrier between the phases, and returns when the
+// steps are done or one of them needs a rebuild (which the graph then runs, with that
+// step's force pass: the bookkeeping is k_drift_done's).  One step of a few
+// thousand atoms in separate launches is four of them, each mostly its own
+// start and its first loads.  The phases' arithmetic is k_drift's and
+// the wide passes': the same trajectory bit for bit.  The blocks' flags go
+// through distributed shared memory; positions, velocities and records are read with
+// ordinary loads, ordered by the barriers (release / acquire).
+constexpr int kStepsCtas = 16, kStepsThreads = 512;
+
+template <int Q, int EAM, int MT>
+__global__ void __cluster_dims__(kStepsCtas, 1, 1) __launch_bounds__(kStepsThreads, 1) k_steps(View V, KArgs a) {
+    __shared__ float s_round[kStepsThreads / 32][3][32];
+    __shared__ float s_tab[5][kMaxTypes * kMaxTypes];
+    __shared__ int s_flag[kStepsCtas];
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int lane = threadIdx.x & 31, cta = blockIdx.x;
+    const unsigned err = V.ctl->err;
+    int rem = V.ctl->remaining, first = V.ctl->first;
+    if (err != 0) {  // latched before this launch: the same in every block
+        if (cta == 0 && threadIdx.x == 0) {
+            cudaGraphSetConditional(V.cond_rebuild, 0u);
+            cudaGraphSetConditional(V.cond_loop, 0u);
+        }
+        return;
+    }
+    WideTab<MT> tab;
+    if (!EAM) tab = wide_tab<MT>(V, s_tab);
+    const Rep &R = V.rep[0];
+    const int gtid = cta * kStepsThreads + threadIdx.x, gw0 = gtid >> 5;
+    const int warps = (int)(((long long)V.n_pad << (V.ltpa + a.aux)) >> 5);
+    constexpr int kThreads = kStepsCtas * kStepsThreads;
+    cluster.sync();  // every block runs before its shared memory is written
+    int done = 0, flags = 0;
+    while (true) {
+        float d2 = 0.f;
+        for (int p = 2 * gtid; p < V.n_pad; p += 2 * kThreads) {
+            int rep;
+            d2 = fmaxf(d2, drift_pair(V, p, 0u, first, rep));
+        }
+        first = 0;
+        // 1: an atom beyond skin/2, 2: a non-finite one (d2 = +Inf)
+        int f = __syncthreads_or(d2 > V.skin_half2f) ? 1 : 0;
+        if (f) f |= __syncthreads_or(__float_as_uint(d2) >= 0x7f800000u) ? 2 : 0;
+        if (threadIdx.x < kStepsCtas) *cluster.map_shared_rank(&s_flag[cta], threadIdx.x) = f;
+        cluster.sync();
+        flags = __reduce_or_sync(0xffffffffu, lane < kStepsCtas ? s_flag[lane] : 0);
+        if (flags) break;
+        ++done;
+        --rem;
+        if constexpr (EAM) {
+            for (int gw = gw0; gw < warps; gw += kThreads / 32) {
+                const Wide w = wide_lane(V, a.aux, gw);
+                WideAtom<Q> at = load_wide<Q>(V, w);
+                rho_wide_warp<Q>(V, kModeStep, w, at, R, s_round[threadIdx.x >> 5]);
+            }
+            cluster.sync();
+        }
+        for (int gw = gw0; gw < warps; gw += kThreads / 32) {
+            const Wide w = wide_lane(V, a.aux, gw);
+            WideAtom<Q> at = load_wide<Q>(V, w);
+            if constexpr (EAM) eam_wide_warp<Q, 0>(V, kModeStep, rem, w, at, R, s_round[threadIdx.x >> 5]);
+            else lj_wide_warp<Q, 0, MT>(V, kModeStep, rem, gw, w, at, R, tab, s_round[threadIdx.x >> 5]);
+        }
+        cluster.sync();
+        if (rem <= 0) break;
+    }
+    if (cta == 0 && threadIdx.x == 0) {
+        const bool bad = flags & 2, rebuild = (flags & 1) && !bad;
+        if (rebuild) {  // this step is counted; its rebuild and force pass follow
+            ++done;
+            --rem;
+            V.ctl->rebuilds += 1;
+        }
+        if (bad) latch_error(V.ctl, kErrNonfinite);
+        V.rep_flag[0] = flags ? 1 : 0;
+        V.rep_disp[0] = 0u;
+        V.ctl->first = 0;
+        V.ctl->steps += done;
+        V.ctl->remaining = rem;
+        cudaGraphSetConditional(V.cond_rebuild, rebuild ? 1u : 0u);
+        cudaGraphSetConditional(V.cond_loop, (rem > 0 && !bad) ? 1u : 0u);
+    }
+}
+
 // before the WHILE node: loop while steps remain and no error is latched
 __global__ void k_loop_init(View V, KArgs a) {
     if (threadIdx.x == 0 && blockIdx.x == 0)
@@ -1365,12 +1500,14 @@ static const void *pick_eamf(int T, int Q, int ev) {
 // sixteen.  us per step at 512 / 640 / 880-1024 / 2048 threads per SM: 4,000
 // atoms 26.2 (8 lanes) / 26.0 (16), 16,000 atoms 28.9 (4) / 29.4 (8), 32,771 atoms 34.6 (2) / 32.5 (4) / 36
 // (8); one lane: 31 .. 33.  32 lanes for the smallest systems measured the same as 16.
-constexpr int kWideThreads = 880, kWideMost = 4;
+// Two lanes pay up to 640 threads per SM only (60,000 atoms: 36.9 us with one, 38.0 with two).
+constexpr int kWideThreads = 880, kWideThreads2 = 640, kWideMost = 4;
 
 static int wide_log(const View &V) {
     int lg = 0;
     while (lg < kWideMost && V.ltpa + lg < 5 && ((long long)V.n_pad << (V.ltpa + lg + 1)) <= (long long)V.n_sm * kWideThreads)
         ++lg;
+    if (lg == 1 && ((long long)V.n_pad << (V.ltpa + 1)) > (long long)V.n_sm * kWideThreads2) lg = 0;
     return lg;
 }
 
@@ -1435,6 +1572,50 @@ void drift_sequence(const View &V, bool in_graph, std::vector<KCall> &seq) {
     else  // two atoms per thread
         seq.push_back(KCall{(const void *)k_drift<MD_PREC_MIXED>, dim3((V.n_pad / 2 + 255) / 256), dim3(256), 0, a});
     seq.push_back(KCall{(const void *)k_drift_done, dim3(1), dim3(256), 0, a});
+}
+
+// Systems with at most so many list slots run their steps in k_steps (the list's capacity is 128 at
+// rc 2.5).  us per step, separate launches -> k_steps (a rebuild every ~8): 500 atoms
+// 21.5 -> 13.3, 2,000 21.4 -> 15.5, 4,000 23.3 -> 20.6, 5,000 23.5 -> 28.1; EAM 864 19.5 -> 12.8, 2,048
+// 19.6 -> 15.5, 8,000 25.1 -> 36.7.  Clusters of eight blocks: 13.5, 19.2, 28.6.
+constexpr int kStepsMost = 4096 * 128;
+
+bool steps_sequence(const View &V, std::vector<KCall> &seq) {
+    // (at least two lanes per thread of the list layout)
+    if (V.prec != MD_PREC_MIXED || V.n_rep != 1 || V.half || V.tile_atoms > 0 || V.ltpa >= 5 ||
+        (long long)V.n_pad * V.maxneigh > kStepsMost)
+        return false;
+    KArgs a{};
+    a.in_graph = 1;
+    a.aux = 1;
+    while (a.aux < kWideMost && V.ltpa + a.aux < 5 &&
+           ((long long)V.n_pad << (V.ltpa + a.aux + 1)) <= kStepsCtas * kStepsThreads)
+        ++a.aux;
+    const void *fn = V.pot == MD_POT_EAM_FS ? PICK_WIDE(k_steps, 1, 0)
+                     : V.ntypes > 1         ? PICK_WIDE(k_steps, 0, 1)
+                                            : PICK_WIDE(k_steps, 0, 0);
+    // a cluster of 16 needs the function's consent and a GPU that can place it
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kStepsCtas);
+    cfg.blockDim = dim3(kStepsThreads);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kStepsCtas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess || clusters < 1) {
+        cudaGetLastError();
+        return false;
+    }
+    seq.push_back(KCall{fn, dim3(kStepsCtas), dim3(kStepsThreads), 0, a});
+    return true;
 }
 
 void kick_sequence(const View &V, int mode, std::vector<KCall> &seq) {

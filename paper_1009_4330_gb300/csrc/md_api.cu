@@ -11,6 +11,10 @@
 //           scan, scatter, gather, build } --> force pass(es)
 //   }
 //
+// For a small mixed system k_steps stands for drift, bookkeeping and force
+// pass of every step that needs no rebuild, and the IF body ends with the force
+// pass of the one that does.
+//
 // k_drift_done (one block) sets cond_rebuild from the per-replica
 // displacement check, counts the step, decrements the remaining step count
 // and sets cond_loop; neither the drift nor the force pass takes a ticket.
@@ -166,9 +170,11 @@ static md_status build_step_graph(md_system *h) {
     cudaGraphNode_t init_last;
     CK(h, add_chain(h, g, seq, nullptr, &init_last));
     CK(h, cudaGraphAddDependencies(g, &init_last, &wnode, nullptr, 1));
-    // body: drift -> IF(rebuild) -> force
+    // body: drift -> IF(rebuild) -> force; or, for a small system, its steps up to
+    // one that needs a rebuild -> IF(rebuild with that step's force pass)
     seq.clear();
-    drift_sequence(h->V, true, seq);
+    const bool whole_steps = steps_sequence(h->V, seq);
+    if (!whole_steps) drift_sequence(h->V, true, seq);
     cudaGraphNode_t drift_last;
     CK(h, add_chain(h, body, seq, nullptr, &drift_last));
     cudaGraphNode_t inode;
@@ -177,12 +183,14 @@ static md_status build_step_graph(md_system *h) {
     seq.clear();
     rebuild_sequence(h->V, false, false, seq);
     for (auto &k : seq) k.args.in_graph = 1;
-    cudaGraphNode_t rlast;
+    cudaGraphNode_t rlast, flast;
+    if (whole_steps) force_sequence(h->V, kModeStep, h->block, true, seq);
     CK(h, add_chain(h, rbody, seq, nullptr, &rlast));
-    seq.clear();
-    force_sequence(h->V, kModeStep, h->block, true, seq);
-    cudaGraphNode_t flast;
-    CK(h, add_chain(h, body, seq, &inode, &flast));
+    if (!whole_steps) {
+        seq.clear();
+        force_sequence(h->V, kModeStep, h->block, true, seq);
+        CK(h, add_chain(h, body, seq, &inode, &flast));
+    }
     CK(h, cudaGraphInstantiate(&h->exec, g, 0));
     return MD_OK;
 }

@@ -25,6 +25,10 @@ void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &
 // md_step call, record refresh, displacement check, rebuild decision)
 void drift_sequence(const View &V, bool in_graph, std::vector<KCall> &seq);
 
+// whole steps of a small system in one launch, up to one that needs a rebuild;
+// false (and nothing added) where the step runs as drift, rebuild and force launches
+bool steps_sequence(const View &V, std::vector<KCall> &seq);
+
 // force evaluation for the current potential / precision / list kind /
 // threads per atom, ending with the epilogue `mode` (kModeStoreF, kModeStep,
 // kModeEV).  `block` = threads per block.
