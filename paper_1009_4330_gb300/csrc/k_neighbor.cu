@@ -922,18 +922,18 @@ __global__ void __launch_bounds__(32 * NW, kBuildWarps / NW) k_build(View V, KAr
 // (rows of more than 32 kRowKeep candidates) are tested again.
 constexpr int kRowKeep = 4;
 
+// one (cell, part) by the nine warps of a block
 template <int PREC, int HALF>
-__global__ void __launch_bounds__(288) k_build_rows(View V, KArgs a) {
+__device__ __forceinline__ void build_rows(const View &V, int gb, int part, int hsplit) {
     __shared__ __align__(16) float s_h[16][8];  // home atoms 2k, 2k + 1: {x, x, y, y}, {z, z, |x|^2, |x|^2}
     __shared__ int s_cnt[9][32];                // accepted per row and home atom
     __shared__ uint32_t s_t[9][kRowKeep][32], s_e[9][kRowKeep][32];
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
-    const int gb = blockIdx.x / V.hsplit, part = blockIdx.x - gb * V.hsplit;
     const int r = V.bin_rep[gb];
     const Rep &R = V.rep[r];
     int my_max = 0;
     long long my_sum = 0;
-    const int hs = V.bin_start[gb], hn = (a.all || V.rep_flag[r]) ? V.bin_count[gb] : 0;  // 0: nothing to do
+    const int hs = V.bin_start[gb], hn = V.bin_count[gb];
     const int xyz = V.bin2xyz[gb];
     const int dy = row % 3 - 1, dz = row / 3 - 1;
     // the row's three cells, one lane each (the other lanes repeat the last)
@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(288) k_build_rows(View V, KArgs a) {
     const float rl2f = 0.5f * (V.rl2f_lo + V.rl2f_hi), margin = 0.5f * (V.rl2f_hi - V.rl2f_lo);
     const int maxn = V.maxneigh, lt = V.ltpa, lq = V.lvec;
     const int la = 5 - lt, ltq = lt + lq, tq = 1 << ltq;
-    for (int h0 = 32 * part; h0 < hn; h0 += 32 * V.hsplit) {
+    for (int h0 = 32 * part; h0 < hn; h0 += 32 * hsplit) {
         const int nh = min(32, hn - h0);
         const int hbase = hs + h0;  // slot of home atom 0 of this chunk
         __syncthreads();
@@ -1067,6 +1067,12 @@ __global__ void __launch_bounds__(288) k_build_rows(View V, KArgs a) {
         }
     }
     if (row == 0) build_stats(V, r, my_max, my_sum, lane);
+}
+
+template <int PREC, int HALF>
+__global__ void __launch_bounds__(288) k_build_rows(View V, KArgs a) {
+    const int gb = blockIdx.x / V.hsplit, part = blockIdx.x - gb * V.hsplit;
+    if (a.all || V.rep_flag[V.bin_rep[gb]]) build_rows<PREC, HALF>(V, gb, part, V.hsplit);
     if (a.all && last_block(&V.ctl->ticket_build)) {
         if (threadIdx.x == 0) {
             V.ctl->ticket_build = 0;
@@ -1109,6 +1115,32 @@ __global__ void __launch_bounds__(1024) k_worklist(View V, KArgs a) {
     }
 }
 
+struct Unit {  // a cell and one of the parts it is shared out in
+    int gb, part, hsplit;
+};
+
+// unit u of the work list: in the last flagged replica f with wl_u0[f] <= u
+__device__ __forceinline__ Unit wl_unit(const View &V, int nf, int u) {
+    int lo = 0, hi = nf - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (__ldg(&V.wl_u0[mid]) <= u) lo = mid;
+        else hi = mid - 1;
+    }
+    const int local = u - __ldg(&V.wl_u0[lo]), hs = __ldg(&V.wl_hs[lo]);
+    return Unit{__ldg(&V.wl_bin[lo]) + local / hs, local % hs, hs};
+}
+
+// the work list's units by rows (see build_rows), for batches of few cells
+template <int PREC, int HALF>
+__global__ void __launch_bounds__(288, 3) k_build_rows_wl(View V, KArgs a) {
+    const int nf = *V.wl_n, total = V.wl_u0[nf];
+    for (int u = blockIdx.x; u < total; u += gridDim.x) {
+        const Unit q = wl_unit(V, nf, u);
+        build_rows<PREC, HALF>(V, q.gb, q.part, q.hsplit);
+    }
+}
+
 // Batched rebuild: a fixed grid walks the work list's units (k_worklist), so
 // that the bins of replicas keeping their lists cost no block launches.
 template <int PREC, int HALF>
@@ -1117,20 +1149,11 @@ __global__ void __launch_bounds__(32, kBuildWarps) k_build_wl(View V, KArgs a) {
     const int nf = *V.wl_n;
     const int total = V.wl_u0[nf];
     for (int u = blockIdx.x; u < total; u += gridDim.x) {
-        // the flagged replica holding unit u: the last f with wl_u0[f] <= u
-        int lo = 0, hi = nf - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(&V.wl_u0[mid]) <= u) lo = mid;
-            else hi = mid - 1;
-        }
-        const int local = u - __ldg(&V.wl_u0[lo]);
-        const int hs = __ldg(&V.wl_hs[lo]);
-        const int gb = __ldg(&V.wl_bin[lo]) + local / hs, part = local % hs;
+        const Unit q = wl_unit(V, nf, u);
         int my_max = 0;
         long long my_sum = 0;
-        build_cell<PREC, HALF, 1>(V, gb, part, hs, lane, w, my_max, my_sum);
-        build_stats(V, V.bin_rep[gb], my_max, my_sum, lane);
+        build_cell<PREC, HALF, 1>(V, q.gb, q.part, q.hsplit, lane, w, my_max, my_sum);
+        build_stats(V, V.bin_rep[q.gb], my_max, my_sum, lane);
     }
 }
 
@@ -1140,6 +1163,10 @@ __global__ void __launch_bounds__(32, kBuildWarps) k_build_wl(View V, KArgs a) {
 // ~8): LJ 500 atoms 20.7 -> 18.7, 4,000 22.4 -> 20.1, 4,000 FP64 31.6 -> 29.3, 8,000 at rc 4.0 43.8 -> 36.9;
 // 32,771 atoms (11 units per SM) 29.3 -> 29.9, 65,536 (21) 38.1 -> 41.8.
 constexpr int kRowBuild = 6;
+// Batches of at most so many cells per SM (about one replica in seven rebuilds in a step).  us per
+// step: 4 replicas (2,554 atoms) 39.2 -> 32.3, 16 (22,829) 70.3 -> 55.3, 60 (169,745, 54 cells per SM) 107.2 ->
+// 104.6; 90 (79 cells per SM) 126.5 -> 143.5.
+constexpr int kRowBuildWl = 64;
 
 void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &seq) {
     KArgs a{};
@@ -1167,10 +1194,16 @@ void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &
     if (V.tile_atoms > 0)
         seq.push_back(KCall{(const void *)k_tiles, dim3((V.n_ftiles + 3) / 4), dim3(128), 0, a});
     if (wl) {
+        if (V.tile_atoms == 0 && V.nbins_total <= V.n_sm * kRowBuildWl) {
+            const void *kr = fp64 ? (V.half ? (const void *)k_build_rows_wl<MD_PREC_FP64, 1> : (const void *)k_build_rows_wl<MD_PREC_FP64, 0>)
+                                  : (V.half ? (const void *)k_build_rows_wl<MD_PREC_MIXED, 1> : (const void *)k_build_rows_wl<MD_PREC_MIXED, 0>);
+            seq.push_back(KCall{kr, dim3(std::min(V.n_sm * 6, V.nbins_total * V.hsplit)), dim3(288), 0, a});
+            return;
+        }
         const void *kb = fp64 ? (V.half ? (const void *)k_build_wl<MD_PREC_FP64, 1> : (const void *)k_build_wl<MD_PREC_FP64, 0>)
                               : (V.half ? (const void *)k_build_wl<MD_PREC_MIXED, 1> : (const void *)k_build_wl<MD_PREC_MIXED, 0>);
-        seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * std::min(kBuildWlDeal, 1 + V.nbins_total / (V.n_sm * kBuildWarps * 4))), dim3(32), 0,
-                            a});
+        const int deal = std::min(kBuildWlDeal, 1 + V.nbins_total / (V.n_sm * kBuildWarps * 4));
+        seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * deal), dim3(32), 0, a});
         return;
     }
     const void *kb;
