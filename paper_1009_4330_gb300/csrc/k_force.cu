@@ -98,6 +98,8 @@ __device__ __forceinline__ float pair_r2(float dx, float dy, float dz) {
 // terms of one round (at most Q) are summed plainly and the round's sum is
 // added to the running total with compensation (blocked Kahan summation:
 // error ~ (Q + 2) u sum |terms| instead of ~n u for n plain additions).
+// Pair::kPacked: the x and y components' operations go two to an instruction, and pair gets
+// d_x and d_y packed as well: the same values from ~10 % fewer instructions (EAM).
 // LOCAL: the entries are block-local and the records come from the block's
 // staging in shared memory (srec).
 template <int T, int Q, bool LOCAL, class Pair>
@@ -111,32 +113,57 @@ __device__ __forceinline__ void walk_list(const View &V, const uint32_t *lp, int
     for (int r = 0; r < nr; ++r) {
         if (r + 1 < nr) load_entries<Q>(lp + (size_t)(r + 1) * 32 * Q, nxt);
         const int left = cnt - (r * PER + sub * Q);
-        float xj[Q], yj[Q], zj[Q];
-        int tj[Q];
+        if constexpr (Pair::kPacked) {
+            ulonglong2 rj[Q];  // the records: {x, y}, {z, type}
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            if (q < left) {
-                if constexpr (LOCAL) {
-                    const float4 r4 = srec[entry_j(cur[q]) & (kTileCap - 1)];
-                    xj[q] = r4.x; yj[q] = r4.y; zj[q] = r4.z; tj[q] = __float_as_int(r4.w);
-                } else {
-                    load_rec(V, entry_j(cur[q]), xj[q], yj[q], zj[q], tj[q]);
+            for (int q = 0; q < Q; ++q)
+                if (q < left) {
+                    const float4 *at = LOCAL ? &srec[entry_j(cur[q]) & (kTileCap - 1)] : &V.rec[entry_j(cur[q])];
+                    rj[q] = LOCAL ? *reinterpret_cast<const ulonglong2 *>(at) : __ldg(reinterpret_cast<const ulonglong2 *>(at));
+                }
+            pair.round_begin();
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if (q < left) {
+                    const uint32_t e = cur[q];
+                    // the scalar form's operations (see below), x and y side by side
+                    const f32x2 c = add2(pack2(__int_as_float(0x4B400000u | (e & 0x3u)), __int_as_float(0x4B400000u | (e & 0xCu))),
+                                         pack2(-12582913.0f, -12582916.0f));
+                    const f32x2 dxy = fma2(c, pack2(-hx, -hy4), sub2(pack2(xi, yi), rj[q].x));
+                    const float2 zt = unpack2(rj[q].y), d = unpack2(dxy);
+                    const float dz = fmaf(-code_z16(e), hz16, zi - zt.x);
+                    pair(dxy, d.x, d.y, dz, pair_r2(d.x, d.y, dz), __float_as_int(zt.y));
                 }
             }
-        }
-        pair.round_begin();
+            pair.round_end();
+        } else {
+            float xj[Q], yj[Q], zj[Q];
+            int tj[Q];
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            if (q < left) {
-                const uint32_t e = cur[q];
-                const float dx = fmaf(-code_x(e), hx, xi - xj[q]);
-                const float dy = fmaf(-code_y4(e), hy4, yi - yj[q]);
-                const float dz = fmaf(-code_z16(e), hz16, zi - zj[q]);
-                const float r2 = pair_r2(dx, dy, dz);
-                pair(e, dx, dy, dz, r2, tj[q]);
+            for (int q = 0; q < Q; ++q) {
+                if (q < left) {
+                    if constexpr (LOCAL) {
+                        const float4 r4 = srec[entry_j(cur[q]) & (kTileCap - 1)];
+                        xj[q] = r4.x; yj[q] = r4.y; zj[q] = r4.z; tj[q] = __float_as_int(r4.w);
+                    } else {
+                        load_rec(V, entry_j(cur[q]), xj[q], yj[q], zj[q], tj[q]);
+                    }
+                }
             }
+            pair.round_begin();
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if (q < left) {
+                    const uint32_t e = cur[q];
+                    const float dx = fmaf(-code_x(e), hx, xi - xj[q]);
+                    const float dy = fmaf(-code_y4(e), hy4, yi - yj[q]);
+                    const float dz = fmaf(-code_z16(e), hz16, zi - zj[q]);
+                    const float r2 = pair_r2(dx, dy, dz);
+                    pair(e, dx, dy, dz, r2, tj[q]);
+                }
+            }
+            pair.round_end();
         }
-        pair.round_end();
 #pragma unroll
         for (int q = 0; q < Q; ++q) cur[q] = nxt[q];
     }
@@ -338,6 +365,7 @@ __device__ __forceinline__ bool in_cut_fp64(const View &V, int p, uint32_t e) {
 //       per component at the end (F zeroed beforehand; kick in k_kick).
 template <int MT, int HALF, int EV>
 struct LJPair {
+    static constexpr bool kPacked = false;
     const View *V;
     const float *lj1, *lj2, *lj3, *lj4, *off;
     float c3, c4, c0;  // one atom type: the energy coefficients and shift, likewise
@@ -812,6 +840,7 @@ void cells_force_sequence(const View &V, int mode, std::vector<KCall> &seq) {
 // same velocity read/write (with a zero increment), but three additions per
 // pair instead of the pair arithmetic and compensated sums.
 struct GatherPair {
+    static constexpr bool kPacked = false;
     float acc;
     __device__ __forceinline__ void round_begin() {}
     __device__ __forceinline__ void round_end() {}
@@ -915,6 +944,7 @@ __global__ void k_kick(View V, KArgs a) {
 // pass 1: host density rho_i = sum_j (rc - r)^2 and the embedding derivative
 // F'(rho_i) = -A / (2 sqrt(rho_i)) (0 at rho = 0), FP64 per atom
 struct RhoPair {
+    static constexpr bool kPacked = true;
     KahanF acc;
     float rc, rc2, part;
     __device__ __forceinline__ void round_begin() { part = 0; }
@@ -925,6 +955,9 @@ struct RhoPair {
         const float r = r2 * rsqrtf(r2);  // branch-free: t = 0 beyond rc
         const float t = (r2 < rc2) ? rc - r : 0.f;
         part += t * t;
+    }
+    __device__ __forceinline__ void operator()(f32x2, float dx, float dy, float dz, float r2, int t) {
+        (*this)(0u, dx, dy, dz, r2, t);
     }
 };
 
@@ -1004,6 +1037,7 @@ __global__ void __launch_bounds__(kWideBlock) k_eam_rho_wide(View V, KArgs a) {
 // pass 2: F_i = -sum_j [phi'(r) + (F'_i + F'_j) rho'(r)] d / r
 template <int EV>
 struct EamPair {
+    static constexpr bool kPacked = false;
     float rc, rc2, c0, c1, c2, fpi;
     KahanF ax, ay, az, e;
     KahanF w[6];
@@ -1028,16 +1062,20 @@ struct EamPair {
     __device__ __forceinline__ float term(int k) const {
         return k == 0 ? rx : k == 1 ? ry : k == 2 ? rz : k == 3 ? re : rw[k - 4];
     }
+    // -(phi' + (F'_i + F'_j) rho') / r, branch-free: t = 0 beyond rc zeroes the term
+    __device__ __forceinline__ float coefficient(float r2, int wj) const {
+        const float fpj = __int_as_float(wj);
+        const float rinv = rsqrtf(r2);
+        const float r = r2 * rinv;
+        const float t = (r2 < rc2) ? rc - r : 0.f;
+        const float poly = c0 + r * (c1 + r * c2);
+        const float dpoly = c1 + 2.f * c2 * r;
+        return -t * (-2.f * poly + t * dpoly - 2.f * (fpi + fpj)) * rinv;
+    }
     // wj: F'_j, which came with the record (rec.w, set by the density pass)
     __device__ __forceinline__ void operator()(uint32_t, float dx, float dy, float dz, float r2, int wj) {
-        if constexpr (!EV) {  // branch-free: t = 0 beyond rc zeroes the term
-            const float fpj = __int_as_float(wj);
-            const float rinv = rsqrtf(r2);
-            const float r = r2 * rinv;
-            const float t = (r2 < rc2) ? rc - r : 0.f;
-            const float poly = c0 + r * (c1 + r * c2);
-            const float dpoly = c1 + 2.f * c2 * r;
-            const float coef = -t * (-2.f * poly + t * dpoly - 2.f * (fpi + fpj)) * rinv;
+        if constexpr (!EV) {
+            const float coef = coefficient(r2, wj);
             rx += dx * coef; ry += dy * coef; rz += dz * coef;
             return;
         }
@@ -1059,6 +1097,36 @@ struct EamPair {
                 rw[3] += h * dx * fyp; rw[4] += h * dx * fzp; rw[5] += h * dy * fzp;
             }
         }
+    }
+};
+
+// The force-only pass with the x and y components' sums packed; what the
+// walk leaves in the wrapped pair are the same sums.  Density and force passes of 500,000 atoms
+// 117.0 -> 114.8 us.  (The LJ pass, which its gathers bound, is slower packed: 124.8 -> 135.2 us on
+// 864,000 atoms, 126.1 .. 132 with only part of it packed or with more registers.)
+struct PackedForce {
+    using Base = EamPair<0>;
+    static constexpr bool kPacked = true;
+    Base &b;
+    f32x2 rxy;
+    KahanF2 axy;
+    __device__ __forceinline__ explicit PackedForce(Base &base) : b(base) { axy.zero(); }
+    __device__ __forceinline__ void round_begin() {
+        rxy = 0ull;
+        b.rz = 0.f;
+    }
+    __device__ __forceinline__ void round_end() {
+        axy.add(rxy);
+        b.az.add(b.rz);
+    }
+    __device__ __forceinline__ void operator()(f32x2 dxy, float, float, float dz, float r2, int tj) {
+        const float f = b.coefficient(r2, tj);
+        rxy = fma2(dxy, pack2(f, f), rxy);
+        b.rz = fmaf(dz, f, b.rz);
+    }
+    __device__ __forceinline__ void finish() {
+        b.ax = axy.first();
+        b.ay = axy.second();
     }
 };
 
@@ -1094,7 +1162,13 @@ __global__ void __launch_bounds__(256) k_eam_force(View V, KArgs a) {
             load_rec(V, p, xi, yi, zi, ti);
             pr.fpi = __int_as_float(ti);
             const uint32_t *lp = V.nlist + (size_t)gw * (size_t)(A * V.maxneigh) + lane * Q;
-            walk_mode<T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
+            if constexpr (!EV) {
+                PackedForce pk(pr);
+                walk_mode<T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pk);
+                pk.finish();
+            } else {
+                walk_mode<T, Q>(V, tmode, lp, sub, cnt, xi, yi, zi, R, s_rec, pr);
+            }
         }
     }
     const double fx = group_sum<T>(pr.ax.value());

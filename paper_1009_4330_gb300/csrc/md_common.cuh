@@ -245,6 +245,32 @@ __device__ __forceinline__ double widen_bits(float y) {
     return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
+// Two FP32 operations in one instruction (sm_100 and later), each rounded as
+// the scalar one: half the issue slots of a pair of operations.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 d) {
+    float2 v;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(d));
+    return v;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// a - b: the product with -1 is exact
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xBF800000BF800000ull, a); }
+
 // FP64 reciprocal and reciprocal square root from the FP32 hardware
 // approximations y0 (relative error < 2^-21, the truncation of x included) by
 // one third-order step each (the series of 1/(1 - e) and (1 - e)^-1/2 to e^2):
@@ -309,6 +335,19 @@ struct KahanF {
         s = t;
     }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+};
+
+// Two such sums side by side, every operation of both in one instruction: the same values.
+struct KahanF2 {
+    f32x2 s, c;
+    __device__ __forceinline__ void zero() { s = 0ull; c = 0ull; }
+    __device__ __forceinline__ void add(f32x2 y) {
+        const f32x2 yc = sub2(y, c), t = add2(s, yc);
+        c = sub2(sub2(t, s), yc);
+        s = t;
+    }
+    __device__ __forceinline__ KahanF first() const { return KahanF{unpack2(s).x, unpack2(c).x}; }
+    __device__ __forceinline__ KahanF second() const { return KahanF{unpack2(s).y, unpack2(c).y}; }
 };
 
 __device__ __forceinline__ void latch_error(Ctl *ctl, unsigned bit) { atomicOr(&ctl->err, bit); }
