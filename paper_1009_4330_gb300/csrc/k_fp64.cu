@@ -20,9 +20,9 @@
 //     double.
 // 17 FP64 instructions per evaluated LJ pair instead of 28 per list entry, with the
 // FP64 pipe 80-86 % busy.  Against one pass of FP64 arithmetic over every
-// entry (time per pass): LJ 256,000 atoms, half list 994 -> 463 us; LJ 4,000
-// atoms 30.6 -> 18 us; EAM 108,000 atoms (density + force) 863 -> 412 us; backward
-// LJ 32,768 atoms, two types 534 -> 200 us, EAM 108,000 atoms 1,337 -> 830 us.
+// entry (time per pass): LJ 256,000 atoms, half list 994 -> 456 us; LJ 4,000
+// atoms 30.6 -> 18.5 us; EAM 108,000 atoms (density + force) 863 -> 360 us; backward
+// LJ 32,768 atoms, two types 534 -> 198 us, EAM 108,000 atoms 1,337 -> 731 us.
 //
 // The atoms are dealt out evenly, in units of four, to one wave of one-warp
 // blocks (at most 16 per SM): a second, partly filled wave cost up to 30 % of
@@ -153,9 +153,12 @@ __device__ __forceinline__ void fp64_walk(const View &V, const Rep &R, int p0, i
     if (active) start();
 
     while (true) {
-        // fill: one chunk per lane until every group has U entries per lane or its list is used up
+        // fill: one chunk per lane until every group has U entries per lane or its list is used up;
+        // groups that have room for a chunk join in, and so fill less often on their own (LJ, 32,000
+        // / 256,000 atoms, half list: 81.7 -> 77.6 / 464.7 -> 456.5 us)
         bool need = active && k0 < cnt && fill - head < kGrp * U;
         while (__any_sync(kFull, need)) {
+            need = active && k0 < cnt && fill - head <= kRing - kGrp * Q;
             const int left = need ? cnt - (k0 + cls * Q) : 0;
             uint32_t e[Q];
             float4 rj[Q];
