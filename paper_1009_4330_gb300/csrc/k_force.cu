@@ -18,6 +18,8 @@
 // adds the round sum with Kahan compensation (forces, energy and virial
 // alike), and folds the compensated sums into FP64 for the group reduction,
 // kick and store.
+#include <type_traits>
+
 #include <cooperative_groups.h>
 
 #include "md_common.cuh"
@@ -944,7 +946,7 @@ __global__ void k_kick(View V, KArgs a) {
 // pass 1: host density rho_i = sum_j (rc - r)^2 and the embedding derivative
 // F'(rho_i) = -A / (2 sqrt(rho_i)) (0 at rho = 0), FP64 per atom
 struct RhoPair {
-    static constexpr bool kPacked = true;
+    static constexpr bool kPacked = false;
     KahanF acc;
     float rc, rc2, part;
     __device__ __forceinline__ void round_begin() { part = 0; }
@@ -956,8 +958,12 @@ struct RhoPair {
         const float t = (r2 < rc2) ? rc - r : 0.f;
         part += t * t;
     }
+};
+// the same with x and y packed
+struct PackedRho : RhoPair {
+    static constexpr bool kPacked = true;
     __device__ __forceinline__ void operator()(f32x2, float dx, float dy, float dz, float r2, int t) {
-        (*this)(0u, dx, dy, dz, r2, t);
+        RhoPair::operator()(0u, dx, dy, dz, r2, t);
     }
 };
 
@@ -975,7 +981,7 @@ __device__ __forceinline__ void finish_rho(const View &V, int mode, int p, doubl
     if (mode == kModeEV) V.emb[p] = rho > 0.0 ? -Aemb * sqrt(rho) : 0.0;
 }
 
-template <int T, int Q>
+template <int T, int Q, int PACK>
 __global__ void __launch_bounds__(256) k_eam_rho(View V, KArgs a) {
     extern __shared__ float4 s_rec[];
     const int tmode = begin_tile(V, T, s_rec);
@@ -986,7 +992,7 @@ __global__ void __launch_bounds__(256) k_eam_rho(View V, KArgs a) {
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int p = gw * A + lane / T;
     const int sub = lane & (T - 1);
-    RhoPair pr;
+    std::conditional_t<PACK, PackedRho, RhoPair> pr;
     pr.acc.zero();
     pr.rc = V.tab->eamf[0];
     pr.rc2 = V.rc2f;
@@ -1101,8 +1107,9 @@ struct EamPair {
 };
 
 // The force-only pass with the x and y components' sums packed; what the
-// walk leaves in the wrapped pair are the same sums.  Density and force passes of 500,000 atoms
-// 117.0 -> 114.8 us.  (The LJ pass, which its gathers bound, is slower packed: 124.8 -> 135.2 us on
+// walk leaves in the wrapped pair are the same sums.  Density and force passes of 80,000 atoms with the force
+// pass scalar / packed 33.0 / 32.0 us, 500,000 with both scalar / packed 117.0 / 114.8 us.  (The
+// LJ pass, which its gathers bound, is slower packed: 124.8 -> 135.2 us on
 // 864,000 atoms, 126.1 .. 132 with only part of it packed or with more registers.)
 struct PackedForce {
     using Base = EamPair<0>;
@@ -1533,22 +1540,28 @@ static const void *pick_lj(int T, int Q, int half, int ev, int mt) {
     return pick_lj_q<1>(T, half, ev, mt);
 }
 
-template <int Q>
+template <int Q, int PACK>
 static const void *pick_rho_q(int T) {
     switch (T) {
-        case 1: return (const void *)k_eam_rho<1, Q>;
-        case 2: return (const void *)k_eam_rho<2, Q>;
-        case 4: return (const void *)k_eam_rho<4, Q>;
-        case 8: return (const void *)k_eam_rho<8, Q>;
-        case 16: return (const void *)k_eam_rho<16, Q>;
-        default: return (const void *)k_eam_rho<32, Q>;
+        case 1: return (const void *)k_eam_rho<1, Q, PACK>;
+        case 2: return (const void *)k_eam_rho<2, Q, PACK>;
+        case 4: return (const void *)k_eam_rho<4, Q, PACK>;
+        case 8: return (const void *)k_eam_rho<8, Q, PACK>;
+        case 16: return (const void *)k_eam_rho<16, Q, PACK>;
+        default: return (const void *)k_eam_rho<32, Q, PACK>;
     }
 }
 
-static const void *pick_rho(int T, int Q) {
-    if (Q == 4) return pick_rho_q<4>(T);
-    if (Q == 2) return pick_rho_q<2>(T);
-    return pick_rho_q<1>(T);
+// The density pass with x and y packed has fewer instructions in a longer chain: from this many threads per SM
+// (about the resident ones). Density plus force pass, scalar -> packed: 60,000 atoms 29.5 -> 30.4 us, 80,000 32.0 ->
+// 33.2, 108,000 36.8 -> 36.8 (a step 46.0 -> 46.4), 150,000 62.7 -> 62.2 per step, 256,000 69.4 -> 67.7,
+// 500,000 117.0 -> 115.0.
+constexpr int kPackThreads = 900;
+
+static const void *pick_rho(int T, int Q, bool pack) {
+    if (Q == 4) return pack ? pick_rho_q<4, 1>(T) : pick_rho_q<4, 0>(T);
+    if (Q == 2) return pack ? pick_rho_q<2, 1>(T) : pick_rho_q<2, 0>(T);
+    return pack ? pick_rho_q<1, 1>(T) : pick_rho_q<1, 0>(T);
 }
 
 template <int Q, int EV>
@@ -1617,7 +1630,7 @@ static void mixed_force_sequence(const View &V, int mode, int block, KArgs a, st
     } else {
         KArgs ar = a;
         ar.in_graph = 0;
-        seq.push_back(KCall{pick_rho(T, V.vec), grid, dim3(block), sm, ar});
+        seq.push_back(KCall{pick_rho(T, V.vec, threads >= (long long)V.n_sm * kPackThreads), grid, dim3(block), sm, ar});
         seq.push_back(KCall{pick_eamf(T, V.vec, ev), grid, dim3(block), sm, a});
     }
 }
