@@ -369,10 +369,11 @@ K_LJ_TRAFFIC_VARIANT = {"tpa": 1, "vec": 4, "list": "full", "block": 128, "tile_
 # the pair coefficient 4, the cut-off test and band minimum 2, the three
 # force sums 6, the compensated round sums 3 (12 additions per 4 entries).
 FP32_OPS_PER_ENTRY = 35
-# FP64 operations per list entry of the FP64 pair loop, counted the same way:
-# separation 9, r^2 5, Newton reciprocal 7, r^-6 2, coefficient 4, cut-off 1,
-# force sums 6.
-FP64_OPS_PER_ENTRY = 34
+# FP64 operations per evaluated pair of the FP64 LJ pass, counted the same way:
+# separation 3, r^2 5, reciprocal 6, r^-6 2, coefficient 4, force sums 6. The pass
+# tests its list entries in FP32 and evaluates those within the cut-off, of a
+# uniform liquid's list the fraction (rc / (rc + skin))^3.
+FP64_OPS_PER_PAIR = 26
 
 
 def load_peaks():
@@ -517,15 +518,16 @@ def step_arm(s, n, k, W):
             "vec": inf["vec"], "block": inf["block"], "rebuilds": i1["rebuilds"] - i0["rebuilds"]}
 
 
-def force_arm(s, ceil, prec):
-    """The force pass alone (md_step form), with its pipe fraction for the precision's pipe."""
+def force_arm(s, ceil, prec, within=1.0):
+    """The force pass alone (md_step form), with its pipe fraction for the precision's pipe;
+    within: the fraction of the list entries that lie within the cut-off."""
     fms, fby = s.time_force(3, 10)
     inf = s.info()
     out = {"force_ms": fms, "force_GBs": fby / (fms / 1000) / 1e9}
     if ceil and s.potential == "lj":
         # per list entry the pair term is evaluated once, full or half list
         if prec == "fp64":
-            tf = FP64_OPS_PER_ENTRY * inf["list_entries"] / (fms / 1000) / 1e12
+            tf = FP64_OPS_PER_PAIR * within * inf["list_entries"] / (fms / 1000) / 1e12
             out["fp64_TFLOPs"] = tf
             out["fp64_pipe_frac"] = tf / ceil["fp64_fma_tflops"]
         else:
@@ -564,7 +566,7 @@ def lj_pair(synth, cells, rc, K, W, ceil, tune=None):
     s, _ = make_lj(synth, cells, rc, "fp64", tpa=0)
     k64 = max(20, k // 10)
     f = step_arm(s, n, k64, 3)
-    f.update(force_arm(s, ceil, "fp64"))
+    f.update(force_arm(s, ceil, "fp64", (rc / (rc + d["skin"])) ** 3))
     out["fp64"] = f
     out["fp64_autotune"] = s.autotune_table()
     s.close()
@@ -606,7 +608,7 @@ def side_runs(synth, cells, K, W, ceil, tune_rc25=None):
                          precision=prec, tpa=0)
         k = max(50, K // 4) if prec == "mixed" else max(20, K // 40)
         a = step_arm(s, nb, k, 5)
-        a.update(force_arm(s, ceil, prec))
+        a.update(force_arm(s, ceil, prec, (2.5 / 2.8) ** 3))
         a["atoms"] = nb
         bat[prec] = a
         s.close()
