@@ -37,6 +37,20 @@ def _dev(a, dtype, shape=None):
     return t.contiguous()
 
 
+def _rows(t, n, what):
+    """t, which has to have a row for each of n atoms: the kernels read (or write) that many."""
+    if t.shape[0] < n:
+        raise MDError(int(L.MD_ERR_INVALID), f"{what}: {t.shape[0]} rows for {n} atoms")
+    return t
+
+
+def _out(t, n, what):
+    """t, a caller's output buffer: written as n rows of three doubles through its pointer."""
+    if not t.is_cuda or t.dtype != torch.float64 or not t.is_contiguous() or t.numel() < 3 * n:
+        raise MDError(int(L.MD_ERR_INVALID), f"{what}: a contiguous float64 CUDA tensor of {n} x 3 values is needed")
+    return t
+
+
 def _ptr(t):
     return ctypes.c_void_p(t.data_ptr()) if t is not None else None
 
@@ -63,8 +77,8 @@ class System:
         _require_cuda()
         self._lib = L.load()
         x = _dev(x, torch.float64, (-1, 3))
-        v = _dev(v, torch.float64, (-1, 3))
         n = x.shape[0]
+        v = _rows(_dev(v, torch.float64, (-1, 3)), n, "v")
         t = _dev(types if types is not None else np.zeros(n, np.int32), torch.int32, (n,))
         self._keep = []
         cfg = self._config(n, box, potential, params, cutoff, skin, dt, mass, n_types, ftm2v, energy_shift,
@@ -133,8 +147,8 @@ class System:
         xs, vs, ts = [], [], []
         for r, rep in enumerate(replicas):
             x = _dev(rep["x"], torch.float64, (-1, 3))
-            v = _dev(rep["v"], torch.float64, (-1, 3))
             n = x.shape[0]
+            v = _rows(_dev(rep["v"], torch.float64, (-1, 3)), n, f"v of replica {r}")
             t = _dev(rep.get("types", np.zeros(n, np.int32)), torch.int32, (n,))
             xs.append(x); vs.append(v); ts.append(t)
             cfgs[r] = self._config(n, rep["box"], potential, params, cutoff, skin, dt, mass, n_types, ftm2v,
@@ -187,7 +201,7 @@ class System:
         self._call("md_build_neighbors")
 
     def compute_forces(self, out=None):
-        f = out if out is not None else torch.empty((self.n, 3), dtype=torch.float64, device="cuda")
+        f = _out(out, self.n, "out") if out is not None else torch.empty((self.n, 3), dtype=torch.float64, device="cuda")
         self._call("md_compute_forces", _ptr(f))
         return f
 
@@ -210,8 +224,8 @@ class System:
         return x, v, f
 
     def set_state(self, x=None, v=None):
-        xd = _dev(x, torch.float64, (-1, 3)) if x is not None else None
-        vd = _dev(v, torch.float64, (-1, 3)) if v is not None else None
+        xd = _rows(_dev(x, torch.float64, (-1, 3)), self.n, "x") if x is not None else None
+        vd = _rows(_dev(v, torch.float64, (-1, 3)), self.n, "v") if v is not None else None
         self._version += 1
         self._call("md_set_state", _ptr(xd), _ptr(vd))
         torch.cuda.current_stream().synchronize()
@@ -220,24 +234,38 @@ class System:
         """Replace every atom (n <= capacity): new positions, velocities and types,
         same box, parameters, kernel variant and device memory."""
         x = _dev(x, torch.float64, (-1, 3))
-        v = _dev(v, torch.float64, (-1, 3))
         n = x.shape[0]
+        v = _rows(_dev(v, torch.float64, (-1, 3)), n, "v")
         t = _dev(types if types is not None else np.zeros(n, np.int32), torch.int32, (n,))
         self._version += 1
         self._call("md_reset", ctypes.c_int64(n), _ptr(x), _ptr(v), _ptr(t))
         self.n = n
 
-    def set_params(self, params):
+    def _params(self, params):
+        """params as the library reads them: a flat host array, at least as long as the potential's."""
         p = np.ascontiguousarray(params, dtype=np.float64).ravel()
+        if p.size < self.n_params:
+            raise MDError(int(L.MD_ERR_INVALID), f"params: {p.size} values, the potential has {self.n_params}")
+        return p
+
+    @property
+    def n_params(self):
+        """Potential parameters in the ABI layout: 2 n_types^2 for LJ, 5 for EAM."""
+        return 5 if self.potential == "eam" else 2 * self.n_types * self.n_types
+
+    def set_params(self, params):
+        p = self._params(params)
         self._version += 1
         self._call("md_set_params", p.ctypes.data_as(ctypes.POINTER(ctypes.c_double)))
 
     def eval_forces(self, params=None, x=None, out=None):
         """Forces (n,3) at new parameters and/or positions, which the system keeps: set_params,
         set_state(x=x) and compute_forces in one call, the forces evaluated once."""
-        f = out if out is not None else torch.empty((self.n, 3), dtype=torch.float64, device="cuda")
-        p = np.ascontiguousarray(params, dtype=np.float64).ravel() if params is not None else None
-        xd = _dev(x, torch.float64, (-1, 3)) if x is not None else None
+        f = _out(out, self.n, "out") if out is not None else torch.empty((self.n, 3), dtype=torch.float64, device="cuda")
+        p = self._params(params) if params is not None else None
+        xd = _rows(_dev(x, torch.float64, (-1, 3)), self.n, "x") if x is not None else None
+        if (xd is not None and xd.shape[0] != self.n) or (p is not None and p.size != self.n_params) or f.numel() != 3 * self.n:
+            raise MDError(int(L.MD_ERR_INVALID), "eval_forces: x, params or out does not have the system's size")
         self._version += 1
         self._call("md_eval_forces", p.ctypes.data_as(ctypes.POINTER(ctypes.c_double)) if p is not None else None,
                    _ptr(xd), _ptr(f))
@@ -246,10 +274,9 @@ class System:
     def backward(self, grad_f):
         """dL/dx (n,3) and dL/dparams (ABI layout: 2 n_types^2 for LJ; 5 for EAM, the cut-off slot 0)
         for dL/dF = grad_f."""
-        g = _dev(grad_f, torch.float64, (-1, 3))
+        g = _rows(_dev(grad_f, torch.float64, (-1, 3)), self.n, "grad_f")
         gx = torch.empty_like(g)
-        npar = 5 if self.potential == "eam" else 2 * self.n_types * self.n_types
-        gp = torch.empty(npar, dtype=torch.float64, device="cuda")
+        gp = torch.empty(self.n_params, dtype=torch.float64, device="cuda")
         self._call("md_forces_backward", _ptr(g), _ptr(gx), _ptr(gp))
         return gx, gp
 
