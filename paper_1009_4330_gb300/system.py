@@ -433,7 +433,7 @@ def _to_host(a, b):
     a, b = a.detach(), b.detach()
     if a.is_cuda and a.device == b.device:
         both = torch.cat([a.double().reshape(-1), b.double().reshape(-1)]).cpu().numpy()
-        return both[:a.numel()], both[a.numel():]
+        return both[:a.numel()].reshape(a.shape), both[a.numel():].reshape(b.shape)
     return a.cpu().double().numpy(), b.cpu().double().numpy()
 
 
