@@ -1669,16 +1669,24 @@ void drift_sequence(const View &V, bool in_graph, std::vector<KCall> &seq) {
     seq.push_back(KCall{(const void *)k_drift_done, dim3(1), dim3(256), 0, a});
 }
 
-// Systems with at most so many list slots run their steps in k_steps (the list's capacity is 128 at
-// rc 2.5).  us per step, separate launches -> k_steps (a rebuild every ~8): 500 atoms
-// 21.5 -> 13.3, 2,000 21.4 -> 15.5, 4,000 23.3 -> 20.6, 5,000 23.5 -> 28.1; EAM 864 19.5 -> 12.8, 2,048
-// 19.6 -> 15.5, 8,000 25.1 -> 36.7.  Clusters of eight blocks: 13.5, 19.2, 28.6.
-constexpr int kStepsMost = 4096 * 128;
+// Which systems run their steps in k_steps.  Two things decide, since the rest of the chip stands idle meanwhile:
+//   * the turns that the cluster's 8,192 threads take through a pass, at two lanes or more per thread of the list
+//     layout: at most two.  us per step in separate launches / in k_steps (a rebuild every ~8), LJ at rc 2.5, one
+//     turn: 500 atoms 20.4 / 12.5, 4,096 22.8 / 20.3; two: 2,000 atoms with 4 threads per atom 21.1 / 18.2, 4,096
+//     with 2 23.3 / 21.7, 1,000 with 8 21.4 / 18.7 (rc 4.0 30.4 / 30.2); three: 1,500 with 8 21.2 / 21.6 (rc 3.2
+//     25.1 / 26.1), 3,000 with 4 22.8 / 23.0; four: 4,096 with 4 24.0 / 26.3; 4,096 with 16 24.5 / 60.7;
+//   * the list slots of all its passes, two for EAM (the list's capacity is 128 per atom at rc 2.5): with more of them
+//     the lanes left per thread get few and walk longer lists.  EAM 2,048 atoms 19.6 / 15.5, with 4 threads per atom
+//     21.1 / 19.7, 2,916 20.0 / 21.5, 4,000 21.1 / 21.6; LJ 5,000 atoms 23.5 / 28.1.
+// Clusters of eight blocks: LJ 500, 4,000 and 5,000 atoms 13.5, 19.2 and 28.6.
+constexpr int kStepsMost = 4096 * 128, kStepsTurns = 2;
 
 bool steps_sequence(const View &V, std::vector<KCall> &seq) {
     // (at least two lanes per thread of the list layout)
+    const int passes = V.pot == MD_POT_EAM_FS ? 2 : 1;
     if (V.prec != MD_PREC_MIXED || V.n_rep != 1 || V.half || V.tile_atoms > 0 || V.ltpa >= 5 ||
-        (long long)V.n_pad * V.maxneigh > kStepsMost)
+        (long long)V.n_pad * V.maxneigh * passes > kStepsMost ||
+        ((long long)V.n_pad << (V.ltpa + 1)) > (long long)kStepsTurns * kStepsCtas * kStepsThreads)
         return false;
     KArgs a{};
     a.in_graph = 1;
