@@ -1595,11 +1595,15 @@ static const void *pick_eamf(int T, int Q, int ev) {
 // atoms 26.2 (8 lanes) / 26.0 (16), 16,000 atoms 28.9 (4) / 29.4 (8), 32,771 atoms 34.6 (2) / 32.5 (4) / 36
 // (8); one lane: 31 .. 33.  32 lanes for the smallest systems measured the same as 16.
 // Two lanes pay up to 640 threads per SM only (60,000 atoms: 36.9 us with one, 38.0 with two).
+// More lanes than the longest list has rounds would only stand by and add to the terms' sums: EAM 4,000 atoms with 8
+// threads per atom (two rounds) 25.2 (4 lanes) -> 21.8 us per step, LJ 4,096 with 4 at rc 1.12 22.8 (8) -> 20.3 (1).
 constexpr int kWideThreads = 880, kWideThreads2 = 640, kWideMost = 4;
 
 static int wide_log(const View &V) {
     int lg = 0;
-    while (lg < kWideMost && V.ltpa + lg < 5 && ((long long)V.n_pad << (V.ltpa + lg + 1)) <= (long long)V.n_sm * kWideThreads)
+    const int rounds = (V.list_most + (V.vec << V.ltpa) - 1) >> (V.ltpa + V.lvec);  // of the longest list
+    while (lg < kWideMost && V.ltpa + lg < 5 && (1 << lg) < rounds &&
+           ((long long)V.n_pad << (V.ltpa + lg + 1)) <= (long long)V.n_sm * kWideThreads)
         ++lg;
     if (lg == 1 && ((long long)V.n_pad << (V.ltpa + 1)) > (long long)V.n_sm * kWideThreads2) lg = 0;
     return lg;

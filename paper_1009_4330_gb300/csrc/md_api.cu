@@ -254,6 +254,7 @@ static md_status settle_overflow(md_system *h, bool all) {
         if (c.err & kErrNonfinite) return fail(h, MD_ERR_NONFINITE, "non-finite position or velocity");
         if (!(c.err & kErrOverflow)) return MD_OK;
         const int need = round_up((int)std::ceil(c.need_maxneigh * 1.2) + 8, 128);
+        h->V.list_most = std::max(h->V.list_most, h->V.half ? 2 * c.need_maxneigh : c.need_maxneigh);
         st = alloc_list(h, need);
         if (st) return st;
         unsigned zero = 0;
@@ -668,6 +669,13 @@ static md_status create_impl(int n_rep, const md_config *cfgs, const double *con
     set_tiles(h);
     st = full_rebuild(h, true);
     if (st) { md_destroy(h); return st; }
+    {
+        int most = 0;
+        long long entries = 0;
+        st = read_stats(h, &most, &entries);
+        if (st) { md_destroy(h); return st; }
+        V.list_most = V.half ? 2 * most : most;
+    }
     st = compute_forces(h, kModeStoreF);
     if (st) { md_destroy(h); return st; }
     if (h->cfg.tpa == 0) {

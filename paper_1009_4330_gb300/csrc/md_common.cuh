@@ -101,6 +101,7 @@ struct View {
     int tpa;          // threads per atom the list is laid out for
     int vec;          // entries per thread per list load (1, 2 or 4)
     int ltpa, lvec;   // log2 of tpa and vec
+    int list_most;    // longest full list at creation, or that the list has grown for since
     int half;         // 1: half list (each pair once, Newton-3 atomics)
     int prec;         // md_precision
     int pot;          // md_potential
