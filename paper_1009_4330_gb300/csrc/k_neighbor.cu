@@ -1163,10 +1163,11 @@ __device__ __forceinline__ Unit wl_unit(const View &V, int nf, int u) {
     return Unit{__ldg(&V.wl_bin[lo]) + local / hs, local % hs, hs};
 }
 
-// the work list's units by rows (see build_rows), for batches of few cells
+// the work list's units by rows (see build_rows), where there are at most a.aux of them
 template <int PREC, int HALF>
 __global__ void __launch_bounds__(288, 3) k_build_rows_wl(View V, KArgs a) {
     const int nf = *V.wl_n, total = V.wl_u0[nf];
+    if (total > a.aux) return;
     for (int u = blockIdx.x; u < total; u += gridDim.x) {
         const Unit q = wl_unit(V, nf, u);
         build_rows<PREC, HALF>(V, q.gb, q.part, q.hsplit);
@@ -1174,12 +1175,14 @@ __global__ void __launch_bounds__(288, 3) k_build_rows_wl(View V, KArgs a) {
 }
 
 // Batched rebuild: a fixed grid walks the work list's units (k_worklist), so
-// that the bins of replicas keeping their lists cost no block launches.
+// that the bins of replicas keeping their lists cost no block launches.  a.aux: as
+// many units or fewer are left to k_build_rows_wl.
 template <int PREC, int HALF>
 __global__ void __launch_bounds__(32, kBuildWarps) k_build_wl(View V, KArgs a) {
     const int lane = threadIdx.x & 31, w = 0;
     const int nf = *V.wl_n;
     const int total = V.wl_u0[nf];
+    if (total <= a.aux) return;
     for (int u = blockIdx.x; u < total; u += gridDim.x) {
         const Unit q = wl_unit(V, nf, u);
         int my_max = 0;
@@ -1195,10 +1198,15 @@ __global__ void __launch_bounds__(32, kBuildWarps) k_build_wl(View V, KArgs a) {
 // ~8): LJ 500 atoms 20.7 -> 18.7, 4,000 22.4 -> 20.1, 4,000 FP64 31.6 -> 29.3, 8,000 at rc 4.0 43.8 -> 36.9;
 // 32,771 atoms (11 units per SM) 29.3 -> 29.9, 65,536 (21) 38.1 -> 41.8.
 constexpr int kRowBuild = 6;
-// Batches of at most so many cells per SM (about one replica in seven rebuilds in a step).  us per
-// step: 4 replicas (2,554 atoms) 39.2 -> 32.3, 16 (22,829) 70.3 -> 55.3, 60 (169,745, 54 cells per SM) 107.2 ->
-// 104.6; 90 (79 cells per SM) 126.5 -> 143.5.
-constexpr int kRowBuildWl = 64;
+// In a batch the units that count are those of the replicas that rebuild in the step, which only the GPU knows: both
+// builds are launched, and one of them returns.  us per step by cells / by rows / so decided: 40 replicas of 8,000
+// atoms at rc 5.0 (36 units per SM, one in seven rebuilding) 882 / 902 / 791, all rebuilding together 577 / 865 /
+// 522; 4 of 40,000 at rc 2.5 (45) 72 / 82 / 71, together 57 / 70 / 56; 20 of 8,000 at rc 4.0 264 / 257 / 243 (with the
+// line at 3 and 12 units per SM 244 and 258).  Batches of at most kRowBuildOnly units per SM in all are built by
+// rows only, which saves the second launch (10 replicas of 2,000 atoms at rc 2.5, 8.4 units, 52.7 -> 50.3; at 11.4 of
+// denser cells, 8 of 8,000 at rc 5.0 together, it costs 197 -> 238), those of more than kRowBuildWl cells per SM by
+// cells only.
+constexpr int kRowBuildOnly = 9, kRowBuildWl = 64;
 
 // threads per block of the per-slot passes (k_prepare, k_scatter, k_gather), as the drift's: evaluation of 100,003 atoms at
 // new coordinates 225 (256) -> 222 us
@@ -1234,12 +1242,22 @@ void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &
                         dim3(kSortBlock), 0, as});
     if (V.tile_atoms > 0)
         seq.push_back(KCall{(const void *)k_tiles, dim3((V.n_ftiles + 3) / 4), dim3(128), 0, a});
-    if (wl) {
-        if (V.tile_atoms == 0 && V.nbins_total <= V.n_sm * kRowBuildWl) {
+    list_build_sequence(V, all, seq);
+}
+
+void list_build_sequence(const View &V, bool all, std::vector<KCall> &seq) {
+    KArgs a{};
+    a.all = all ? 1 : 0;
+    const bool fp64 = V.prec == MD_PREC_FP64;
+    if (V.n_rep > 1 && !all) {
+        const bool rows = V.tile_atoms == 0 && V.nbins_total <= V.n_sm * kRowBuildWl;
+        const bool only = V.nbins_total * V.hsplit <= V.n_sm * kRowBuildOnly;
+        a.aux = !rows ? 0 : only ? V.nbins_total * V.hsplit : V.n_sm * kRowBuild;
+        if (rows) {
             const void *kr = fp64 ? (V.half ? (const void *)k_build_rows_wl<MD_PREC_FP64, 1> : (const void *)k_build_rows_wl<MD_PREC_FP64, 0>)
                                   : (V.half ? (const void *)k_build_rows_wl<MD_PREC_MIXED, 1> : (const void *)k_build_rows_wl<MD_PREC_MIXED, 0>);
-            seq.push_back(KCall{kr, dim3(std::min(V.n_sm * 6, V.nbins_total * V.hsplit)), dim3(288), 0, a});
-            return;
+            seq.push_back(KCall{kr, dim3(std::min(V.n_sm * kRowBuild, V.nbins_total * V.hsplit)), dim3(288), 0, a});
+            if (only) return;
         }
         const void *kb = fp64 ? (V.half ? (const void *)k_build_wl<MD_PREC_FP64, 1> : (const void *)k_build_wl<MD_PREC_FP64, 0>)
                               : (V.half ? (const void *)k_build_wl<MD_PREC_MIXED, 1> : (const void *)k_build_wl<MD_PREC_MIXED, 0>);

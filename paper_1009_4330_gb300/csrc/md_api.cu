@@ -239,9 +239,8 @@ static int ilog2(int x) {
 // run the list build kernel again (after growing the list)
 static md_status rebuild_list_only(md_system *h, bool all) {
     std::vector<KCall> seq;
-    rebuild_sequence(h->V, all, false, seq);
-    std::vector<KCall> last(seq.end() - 1, seq.end());  // k_build
-    CK(h, run_seq(h, last));
+    list_build_sequence(h->V, all, seq);
+    CK(h, run_seq(h, seq));
     return MD_OK;
 }
 

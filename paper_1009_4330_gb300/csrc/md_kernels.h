@@ -21,6 +21,9 @@ struct KCall {
 // staged in the scratch arrays (create / set_state).
 void rebuild_sequence(const View &V, bool all, bool staged, std::vector<KCall> &seq);
 
+// its last part, the list build alone, on the bins of the last rebuild (for the replicas flagged by it, or all)
+void list_build_sequence(const View &V, bool all, std::vector<KCall> &seq);
+
 // one drift (x += dt v, half kick from the stored F on the first step of an
 // md_step call, record refresh, displacement check, rebuild decision)
 void drift_sequence(const View &V, bool in_graph, std::vector<KCall> &seq);
