@@ -629,6 +629,10 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
     __shared__ uint4 s_row[NW][9];
     __shared__ int4 s_row2[NW][9];
     __shared__ int s_delta[NW][2][64];  // per tile of the chunk, per stencil code: entry shift
+    const int hs = V.bin_start[gb], hn = V.bin_count[gb];
+    // nothing to do here: in a gas most cells are empty (256,000 atoms at density 0.005, 2.3 M cells: a build with its sort
+    // 1,886 -> 1,675 us; where no cell is empty the early look costs nothing, 864,000 atoms of liquid 580 us)
+    if (hn <= 32 * part) return;
     const int r = V.bin_rep[gb];
     const Rep &R = V.rep[r];
     const int maxn = V.maxneigh, lt = V.ltpa, lq = V.lvec;
@@ -658,7 +662,6 @@ __device__ __forceinline__ void build_cell(const View &V, int gb, int part, int 
             s_row2[w][row] = make_int4(cnt, cnt + c1, __float_as_int(dy * hy), __float_as_int(dz * hz));
         }
     }
-    const int hs = V.bin_start[gb], hn = V.bin_count[gb];
     const float rl2f = 0.5f * (V.rl2f_lo + V.rl2f_hi), margin = 0.5f * (V.rl2f_hi - V.rl2f_lo);
     // box pre-test bound: above every squared distance the margin band can hold
     const float keep2 = V.rl2f_hi + margin;
