@@ -49,6 +49,7 @@ constexpr int kBatchAtoms = 32;
 constexpr int kSumStride = kBatchAtoms + 1;
 constexpr int kUnit = 4;      // atoms per dealt unit
 constexpr unsigned kFull = 0xffffffffu;
+constexpr float kScreen = 1.0009765625f;  // entries are screened at 2^-10 above rc^2: far beyond the FP32 error of r^2
 // Warps per SM of the one wave: 20 (at most 96 registers) for the LJ and EAM
 // density passes without energies, 16 for the others.  32,000 / 256,000-atom LJ pass: 84.4 /
 // 523 us with 16, 74.4 / 515 with 20, 91.0 / 596 with 12 (EAM backward: 844, 863, 818).
@@ -93,11 +94,86 @@ __device__ __forceinline__ bool below(double r2, double rc2) {
     return (unsigned long long)__double_as_longlong(r2) < (unsigned long long)__double_as_longlong(rc2);
 }
 
+// first entry of slot p's list
+__device__ __forceinline__ const uint32_t *list_of(const View &V, int p, int Q) {
+    const int la = 5 - V.ltpa;
+    return V.nlist + (size_t)(p >> la) * ((size_t)V.maxneigh << la) + (size_t)((p & ((1 << la) - 1)) << V.ltpa) * Q;
+}
+
+// The walk of a batch with short lists (a gas): at most eight entries an atom, kShortPairs in all.  Each lane tests its own atom's
+// entries, all atoms' accepted ones share one queue, and the warp evaluates it 32 pairs at a time.  As pair k of an
+// atom is the only one of its partial sum k, each is stored as it comes: the same bits as the groups' walk below, which such
+// lists leave mostly idle (eight lanes for one or two pairs, ~75 instructions an atom).  us per LJ pass of 256,000 atoms at
+// density 0.005 / 0.02 / 0.05 (full list) groups 30.3 / 63.5 / 95.8, so 24.6 /
+// 36.8 / 71.7.  The backward passes keep to the groups: the second walk cost them registers (EAM 6,912 atoms 80 -> 95 us).
+constexpr int kShortPairs = kGroups * kRing / 2;
+template <class Src, int Q, class Pair>
+__device__ __forceinline__ void short_walk(const View &V, const Rep &R, int p0, int cnt, int most, char *smem, Pair &pair) {
+    const int lane = threadIdx.x;
+    uint2 *const queue = reinterpret_cast<uint2 *>(smem);  // entry; atom of the batch and index among its accepted
+    const double *const xs = reinterpret_cast<const double *>(smem + kGroups * kRing * 4);
+    double *const sums = reinterpret_cast<double *>(smem + kSumsAt);
+#pragma unroll
+    for (int k = 0; k < Pair::kSums * kGrp; ++k) sums[k * kSumStride + lane] = 0.0;
+    const float hx = R.hf[0], hy4 = R.hf[1] * 0.25f, hz16 = R.hf[2] * 0.0625f;
+    const float keep2 = V.rc2f * kScreen;
+    const int p = p0 + lane, lt = V.ltpa;
+    const uint32_t *const lp = list_of(V, p, Q);
+    float4 ri = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (cnt > 0) ri = V.rec[p];
+    int mine = 0, total = 0;
+    for (int k0 = 0; k0 < most; k0 += Q) {
+        uint32_t e[Q];
+        float4 rj[Q];
+        const int left = cnt - k0;
+        if (left > 0) {
+            const int c = k0 / Q;
+            load_chunk<Q>(lp + (size_t)(c >> lt) * (32 * Q) + (c & ((1 << lt) - 1)) * Q, e);
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (q < left) {
+                    if (V.tile_atoms) e[q] = ((uint32_t)entry_slot(V, p, e[q]) << 6) | (e[q] & 63u);
+                    rj[q] = __ldg(&V.rec[entry_j(e[q])]);
+                }
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            bool acc = false;
+            if (q < left) {
+                const float dx = fmaf(-code_x(e[q]), hx, ri.x - rj[q].x);
+                const float dy = fmaf(-code_y4(e[q]), hy4, ri.y - rj[q].y);
+                const float dz = fmaf(-code_z16(e[q]), hz16, ri.z - rj[q].z);
+                acc = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < keep2;
+            }
+            const unsigned b = __ballot_sync(kFull, acc);
+            if (acc) {
+                queue[total + __popc(b & ((1u << lane) - 1u))] = make_uint2(e[q], (unsigned)(mine << 5 | lane));
+                ++mine;
+            }
+            total += __popc(b);
+        }
+    }
+    __syncwarp();
+    for (int i = lane; i - lane < total; i += 32) {
+        const bool on = i < total;
+        const uint2 q = on ? queue[i] : make_uint2(((uint32_t)p0 << 6) | kSelfCode, 0u);
+        const int a = q.y & 31u;
+        pair.begin(V, p0 + a);
+        const double4_32a xj = load_pos<Src>(V, entry_j(q.x));
+        const double *const x = xs + a * 9;
+        const double dx = x[q.x & 3u] - xj.x, dy = x[3 + ((q.x >> 2) & 3u)] - xj.y, dz = x[6 + ((q.x >> 4) & 3u)] - xj.z;
+        pair(V, q.x, on, dx, dy, dz, fma(dz, dz, fma(dy, dy, dx * dx)), xj.w);
+        if (on) pair.store(sums + a, (int)(q.y >> 5));
+    }
+    __syncwarp();
+}
+
 // The walk over the lists of a batch: atoms p0 .. p0 + nb - 1 (nb <= 32, one replica).
 // U: pairs in flight per lane.  A lane's FP64 chain is ~13 dependent
 // instructions; with 16 warps per SM other warps fill the pipe (U = 1), a system
 // too small for that evaluates up to four pairs per lane at once.
 // Pair, zero-initialised (a group that gets no atom evaluates its lanes' idle pairs all the same), supplies
+//   kSums                                  sums per lane
 //   begin(V, p)                            per-atom values of slot p, sums zeroed
 //   operator()(V, e, on, dx, dy, dz, r2, w)   one pair per lane (on: this lane has one)
 //   store(sums, cls)                       this lane's partial sums -> shared memory
@@ -116,9 +192,17 @@ __device__ __forceinline__ void fp64_walk(const View &V, const Rep &R, int p0, i
         xs[3 * k + 2] = x - R.h[c];
     }
     __syncwarp();
+    if constexpr (!Src::packed) {
+        const int c = lane < nb ? V.ncount[p0 + lane] : 0;
+        const int most = __reduce_max_sync(kFull, c);
+        if (most <= kGrp && __reduce_add_sync(kFull, c) <= kShortPairs) {
+            short_walk<Src, Q>(V, R, p0, c, most, smem, pair);
+            return;
+        }
+    }
     const float hx = R.hf[0], hy4 = R.hf[1] * 0.25f, hz16 = R.hf[2] * 0.0625f;
-    const float keep2 = V.rc2f * 1.0009765625f;  // 2^-10 above rc^2: far beyond the FP32 error of r^2
-    const int lt = V.ltpa, la = 5 - lt, maxn = V.maxneigh;
+    const float keep2 = V.rc2f * kScreen;
+    const int lt = V.ltpa;
     const unsigned gmask = 0xffu << (grp * kGrp), lower = (1u << cls) - 1u;
 
     int a = grp, next = kGroups;  // this group's atom; the first atom not taken yet
@@ -143,7 +227,7 @@ __device__ __forceinline__ void fp64_walk(const View &V, const Rep &R, int p0, i
         cnt = V.ncount[p];
         const float4 r = V.rec[p];
         xi = r.x; yi = r.y; zi = r.z;
-        lp = V.nlist + (size_t)(p >> la) * ((size_t)maxn << la) + (size_t)((p & ((1 << la) - 1)) << lt) * Q;
+        lp = list_of(V, p, Q);
         k0 = 0;
         head = 0;
         fill = 0;
@@ -283,6 +367,7 @@ __device__ __forceinline__ void for_sums(int ns, int nb, F &&f) {
 
 template <int HALF, int EV, int MT>
 struct Lj64 {
+    static constexpr int kSums = EV ? 10 : 3;
     double ax, ay, az, e, w[6];
     double c1, c2, c3, c4, c0, rc2;
     int ti;
@@ -380,6 +465,7 @@ __global__ void __launch_bounds__(32, U == 4 ? 8 : EV ? kWarpsFew : kWarpsMany) 
 // ------------------------------------------------------------------- EAM --
 
 struct Rho64 {
+    static constexpr int kSums = 1;
     double rho, rc, rc2;
     __device__ __forceinline__ void begin(const View &, int) { rho = 0.0; }
     __device__ __forceinline__ void operator()(const View &, uint32_t, bool on, double, double, double, double r2,
@@ -426,6 +512,7 @@ struct EamPoly {
 
 template <int EV>
 struct Eam64 {
+    static constexpr int kSums = EV ? 10 : 3;
     double ax, ay, az, e, w[6];
     double rc, rc2, p0, p1, p2, d0, d1, d2, fpi;  // d: 2 p0, 3 p1, 4 p2
     __device__ __forceinline__ void begin(const View &V, int p) {
