@@ -759,14 +759,11 @@ struct EamBwd1 {
     __device__ __forceinline__ void operator()(const View &V, uint32_t ent, bool on, double dx, double dy, double dz,
                                                double r2, double) {
         const bool in = on && below(r2, rc2);
-        // g only: the second half of the record, whose last field pass 1 itself writes
-        const double *gj = reinterpret_cast<const double *>(&V.bpack[2 * (size_t)entry_j(ent) + 1]);
-        const double2 gxy = *reinterpret_cast<const double2 *>(gj);
-        const double gzj = gj[2];
+        const double4_32a gj = V.bpack[2 * (size_t)entry_j(ent) + 1];
         const double ir = rsqrt64(r2), r = r2 * ir;
         const double t = rc - r, tir = t * ir;
         // w rho'(r) with w = (g_i - g_j).d / r and rho' = -2 (rc - r); the -2 at the atom's end
-        const double Gd = fma(giz - gzj, dz, fma(giy - gxy.y, dy, (gix - gxy.x) * dx));
+        const double Gd = fma(giz - gj.z, dz, fma(giy - gj.y, dy, (gix - gj.x) * dx));
         add_if(in, t, t, rho);
         add_if(in, tir, Gd, lam);
     }
