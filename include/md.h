@@ -434,7 +434,8 @@ md_status md_probe_ceilings(void *stream, md_ceilings *out);
  * a third-order step each from the FP32 hardware approximations, used by the
  * FP64 force passes -- applied to x[n] (device), results in y[n] (device), on
  * `stream`.  For tests that hold them to an error bound against the
- * correctly rounded operations; valid for FLT_MIN < x < FLT_MAX.
+ * correctly rounded operations; valid for FLT_MIN <= x <= 2^126 (op 0, beyond
+ * which the FP32 approximation flushes to zero) and FLT_MIN <= x < FLT_MAX (op 1).
  * Cite: no paper passage -- test hook.
  */
 md_status md_probe_fp64_math(int32_t op, int64_t n, const double *x, double *y, void *stream);

@@ -280,7 +280,8 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xBF800
 // both below 2^-62, so that only the last roundings are left; the residuals
 // are single fused multiply-adds of exact products (y0 has 24 bits).  3 and 5
 // FP64 instructions; the two-step Newton forms with conversions took 6 and 9.
-// For FLT_MIN <= x < FLT_MAX; below (x = 0 included) the result is NaN.
+// For FLT_MIN <= x < FLT_MAX, and x <= 2^126 for the reciprocal, whose approximation is flushed to zero beyond (the
+// squared distances here are far below); under FLT_MIN (x = 0 included) the result is NaN.
 __device__ __forceinline__ double seed64(float y0, double x) {
     const double y = widen_bits(y0);
     return __double2hiint(x) < 0x38100000 ? __hiloint2double(0x7ff80000, 0) : y;
