@@ -40,3 +40,47 @@ def test_short_lists(rho, rc, tpa, vec):
     """Lists of no entry to a few dozen: fewer rounds than the size alone allows lanes."""
     r, kw = _lj(999, rho, rc, 1)
     _same_bits(kw, r, 160, tpa, vec)
+
+
+def _atoms(per_sm):
+    """Sizes follow the GPU's, as the rule for the lanes does (threads per SM)."""
+    import torch
+    return per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+
+
+@pytest.mark.parametrize("nt", [1, 2])
+@pytest.mark.parametrize("tpa,vec,per_sm,copies", [(1, 4, 270, 2),   # two lanes
+                                                   (1, 1, 160, 3),   # four
+                                                   (1, 4, 80, 6),    # eight
+                                                   (2, 2, 135, 2),   # two
+                                                   (2, 4, 90, 3),    # four
+                                                   (4, 4, 66, 2),    # two
+                                                   (4, 1, 45, 3),    # four
+                                                   (8, 4, 35, 2),    # two
+                                                   (16, 1, 16, 3)])  # two
+def test_lj_lanes(tpa, vec, per_sm, copies, nt):
+    r, kw = _lj(_atoms(per_sm) + 3, 0.8442, 2.5, nt)
+    _same_bits(kw, r, copies, tpa, vec)
+
+
+def _eam(n):
+    cells = int(round((n / 4) ** (1 / 3)))
+    x, box = synth.fcc_lattice(cells, cells, cells, 3.615)
+    x = synth.displace(x, box, 0.08, 41)
+    return ({"x": x, "v": np.ones_like(x), "box": box, "types": np.zeros(len(x), np.int32)},
+            dict(potential="eam", params=np.array(synth.EAM_PARAMS), cutoff=float(synth.EAM_PARAMS[0]), skin=0.5, dt=1.0,
+                 mass=63.55, ftm2v=synth.FTM2V_METAL, precision="mixed", tpa=1))
+
+
+@pytest.mark.parametrize("tpa,vec,per_sm,copies", [(1, 4, 270, 2), (1, 2, 160, 3), (2, 4, 135, 2), (4, 4, 66, 2), (8, 1, 35, 2)])
+def test_eam_lanes(tpa, vec, per_sm, copies):
+    r, kw = _eam(_atoms(per_sm))
+    _same_bits(kw, r, copies, tpa, vec)
+
+
+@pytest.mark.parametrize("vec", [1, 2, 4])
+def test_eam_scalar_and_packed_density_pass(vec):
+    """Sizes too large for several lanes take the scalar density pass up to 900 threads per SM, larger ones the packed one."""
+    r, kw = _eam(_atoms(600))
+    assert _atoms(330) < len(r["x"]) < _atoms(880)
+    _same_bits(kw, r, 2, 1, vec)
