@@ -296,18 +296,6 @@ __device__ __forceinline__ void walk_wide(const View &V, const Wide &w, const Re
     }
 }
 
-// force component c of atom p: kick or store
-__device__ __forceinline__ void wide_finish(const View &V, int mode, int rem, int c, int p, double ftm, double f) {
-    const size_t i = (size_t)c * V.n_pad + p;
-    if (mode == kModeStep || mode == kModeKickDry) {
-        const bool last = (mode == kModeStep && rem == 0);
-        const double k = (mode == kModeKickDry) ? 0.0 : (last ? 0.5 : 1.0) * V.dt * ftm;
-        V.v[i] += k * f;
-        if (!last) return;
-    }
-    V.f[i] = f;
-}
-
 // stage the block's tile when its entries are block-local (before the
 // kernel's first block barrier)
 __device__ __forceinline__ int begin_tile(const View &V, int T, float4 *srec) {
@@ -334,12 +322,6 @@ __device__ __forceinline__ void epilogue(const View &V, int mode, int rem, int p
     } else {
         V.f[p] = fx; V.f[n + p] = fy; V.f[2 * n + p] = fz;
     }
-}
-
-__device__ __forceinline__ void write_kinetic(const View &V, int p, double ftm) {
-    const int n = V.n_pad;
-    const double vx = V.v[p], vy = V.v[n + p], vz = V.v[2 * n + p];
-    V.ev[n + p] = 0.5 * (vx * vx + vy * vy + vz * vz) / ftm;
 }
 
 __device__ __forceinline__ void write_ev(const View &V, int p, int t, double e, const double *w, const double *s_ftm) {
@@ -403,7 +385,6 @@ struct LJPair {
         }
     }
     // the round's sums, in the order of the wide passes' terms
-    static constexpr int kTerms = EV ? 10 : 3;
     __device__ __forceinline__ float term(int k) const {
         return k == 0 ? rx : k == 1 ? ry : k == 2 ? rz : k == 3 ? re : rw[k - 4];
     }
@@ -722,7 +703,7 @@ __device__ __forceinline__ void lj_wide_warp(const View &V, int mode, int rem, i
         const int term = w.g + (k << w.lg);
         const double x = wide_sum(w, acc[k].value());
         if (!valid || w.sub != 0) continue;
-        if (term < 3) wide_finish(V, mode, rem, term, w.p, ftm, x);
+        if (term < 3) finish_component(V, mode, rem, term, w.p, ftm, x);
         else if (EV && term < NT) V.ev[(size_t)(term == 3 ? 0 : term - 2) * V.n_pad + w.p] = x;
     }
     if (EV && valid && w.sub == 0 && w.g == 0) write_kinetic(V, w.p, ftm);
@@ -954,7 +935,6 @@ struct RhoPair {
     float rc, rc2, part;
     __device__ __forceinline__ void round_begin() { part = 0; }
     __device__ __forceinline__ void round_end() { acc.add(part); }
-    static constexpr int kTerms = 1;
     __device__ __forceinline__ float term(int) const { return part; }
     __device__ __forceinline__ void operator()(uint32_t, float, float, float, float r2, int) {
         const float r = r2 * rsqrtf(r2);  // branch-free: t = 0 beyond rc
@@ -1067,7 +1047,6 @@ struct EamPair {
         }
     }
     // the round's sums, in the order of the wide passes' terms
-    static constexpr int kTerms = EV ? 10 : 3;
     __device__ __forceinline__ float term(int k) const {
         return k == 0 ? rx : k == 1 ? ry : k == 2 ? rz : k == 3 ? re : rw[k - 4];
     }
@@ -1216,7 +1195,7 @@ __device__ __forceinline__ void eam_wide_warp(const View &V, int mode, int rem, 
         const int term = w.g + (k << w.lg);
         const double x = wide_sum(w, acc[k].value());
         if (!valid || w.sub != 0) continue;
-        if (term < 3) wide_finish(V, mode, rem, term, w.p, ftm, x);
+        if (term < 3) finish_component(V, mode, rem, term, w.p, ftm, x);
         else if (EV && term == 3) V.ev[w.p] = x + V.emb[w.p];
         else if (EV && term < NT) V.ev[(size_t)(term - 2) * V.n_pad + w.p] = x;
     }
@@ -1238,13 +1217,10 @@ __global__ void __launch_bounds__(kWideBlock) k_eam_force_wide(View V, KArgs a) 
 // ------------------------------------------------------- drift + control --
 
 // x += dt v (after v += dt/2 a(F) on the first step of an md_step call);
-// refresh the FP32 record; per-replica max displacement since the build;
-// the last block turns it into per-replica rebuild flags and sets the
-// rebuild conditional of the step graph.  Mixed precision: two adjacent
+// refresh the FP32 record; per-replica max displacement since the build, which
+// k_drift_done turns into rebuild flags.  Mixed precision: two adjacent
 // atoms per thread with 16-byte loads and stores (measured faster than one
 // atom per thread, and half the blocks' atomics); FP64: one atom per thread.
-constexpr int kDriftPer = 1;
-
 template <int PREC>
 __device__ __forceinline__ float drift_one(const View &V, int p, unsigned err, int first, int &rep) {
     const int n = V.n_pad;
@@ -1342,26 +1318,15 @@ __global__ void __launch_bounds__(kDriftBlock) k_drift(View V, KArgs a) {
     const unsigned err = V.ctl->err;
     const int first = V.ctl->first;
     if (blockIdx.x == 0 && threadIdx.x == 0) V.ctl->err_at_drift = err;  // for k_drift_done
-    float d2[kDriftPer];
-    int rep[kDriftPer];
+    float d2 = 0.f;
+    int rep = -1;
+    const int t = blockIdx.x * kDriftBlock + threadIdx.x;
     if constexpr (PREC == MD_PREC_MIXED) {
-        // two adjacent atoms per thread
-        const int p = 2 * (blockIdx.x * kDriftBlock + threadIdx.x);
-        d2[0] = 0.f;
-        rep[0] = -1;
-        if (p < V.n_pad) d2[0] = drift_pair(V, p, err, first, rep[0]);
+        if (2 * t < V.n_pad) d2 = drift_pair(V, 2 * t, err, first, rep);  // two adjacent atoms per thread
     } else {
-        const int p0 = blockIdx.x * (kDriftBlock * kDriftPer) + threadIdx.x;
-#pragma unroll
-        for (int u = 0; u < kDriftPer; ++u) {
-            const int p = p0 + u * kDriftBlock;
-            d2[u] = 0.f;
-            rep[u] = -1;
-            if (p < V.n_pad) d2[u] = drift_one<PREC>(V, p, err, first, rep[u]);
-        }
+        if (t < V.n_pad) d2 = drift_one<PREC>(V, t, err, first, rep);
     }
-#pragma unroll
-    for (int u = 0; u < kDriftPer; ++u) note_disp(V.rep_disp, V.skin_half2f, d2[u], rep[u]);
+    note_disp(V.rep_disp, V.skin_half2f, d2, rep);
 }
 
 // The step's bookkeeping after the drift, one block: the per-replica maximum
@@ -1666,7 +1631,7 @@ void drift_sequence(const View &V, bool in_graph, std::vector<KCall> &seq) {
     a.in_graph = in_graph ? 1 : 0;
     if (V.prec == MD_PREC_FP64)
         seq.push_back(KCall{(const void *)k_drift<MD_PREC_FP64>,
-                            dim3((V.n_pad + kDriftBlock * kDriftPer - 1) / (kDriftBlock * kDriftPer)), dim3(kDriftBlock), 0, a});
+                            dim3((V.n_pad + kDriftBlock - 1) / kDriftBlock), dim3(kDriftBlock), 0, a});
     else  // two atoms per thread
         seq.push_back(KCall{(const void *)k_drift<MD_PREC_MIXED>, dim3((V.n_pad / 2 + kDriftBlock - 1) / kDriftBlock),
                             dim3(kDriftBlock), 0, a});

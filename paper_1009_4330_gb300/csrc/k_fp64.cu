@@ -419,23 +419,6 @@ struct Lj64 {
     }
 };
 
-// epilogue of force component c of slot p: kick or store (see the modes in md_common.cuh)
-__device__ __forceinline__ void finish64(const View &V, int mode, int rem, int c, int p, double ftm, double f) {
-    const size_t at = (size_t)c * V.n_pad + p;
-    if (mode == kModeStep || mode == kModeKickDry) {
-        const bool last = (mode == kModeStep && rem == 0);
-        V.v[at] += ((mode == kModeKickDry) ? 0.0 : (last ? 0.5 : 1.0) * V.dt * ftm) * f;
-        if (!last) return;
-    }
-    V.f[at] = f;
-}
-
-__device__ __forceinline__ void kinetic64(const View &V, int p, double ftm) {
-    const int n = V.n_pad;
-    const double vx = V.v[p], vy = V.v[n + p], vz = V.v[2 * n + p];
-    V.ev[n + p] = 0.5 * (vx * vx + vy * vy + vz * vz) / ftm;
-}
-
 template <int Q, int U, int HALF, int EV, int MT>
 __global__ void __launch_bounds__(32, U == 4 ? 8 : EV ? kWarpsFew : kWarpsMany) k64_lj(View V, KArgs a) {
     extern __shared__ char smem[];
@@ -454,11 +437,11 @@ __global__ void __launch_bounds__(32, U == 4 ? 8 : EV ? kWarpsFew : kWarpsMany) 
             const int p = p0 + i;
             if (s >= 3) V.ev[(size_t)(s == 3 ? 0 : s - 2) * V.n_pad + p] = (HALF ? 1.0 : 0.5) * x;
             else if (HALF) atomicAdd(&V.f[(size_t)s * V.n_pad + p], x);
-            else finish64(V, a.mode, rem, s, p, V.tab->ftm_m[MT ? V.type[p] : 0], x);
+            else finish_component(V, a.mode, rem, s, p, V.tab->ftm_m[MT ? V.type[p] : 0], x);
         });
         // (half lists: the kinetic term follows in k_kick)
         if (EV && !HALF && (int)threadIdx.x < nb)
-            kinetic64(V, p0 + threadIdx.x, V.tab->ftm_m[MT ? V.type[p0 + threadIdx.x] : 0]);
+            write_kinetic(V, p0 + threadIdx.x, V.tab->ftm_m[MT ? V.type[p0 + threadIdx.x] : 0]);
     });
 }
 
@@ -571,11 +554,11 @@ __global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_eam_force(View
         for_sums(EV ? 10 : 3, nb, [&](int s, int i) {
             const double x = lane_total(smem, s, i);
             const int p = p0 + i;
-            if (s < 3) finish64(V, a.mode, rem, s, p, ftm, x);
+            if (s < 3) finish_component(V, a.mode, rem, s, p, ftm, x);
             else if (s == 3) V.ev[p] = 0.5 * x + V.emb[p];
             else V.ev[(size_t)(s - 2) * V.n_pad + p] = 0.5 * x;
         });
-        if (EV && (int)threadIdx.x < nb) kinetic64(V, p0 + threadIdx.x, ftm);
+        if (EV && (int)threadIdx.x < nb) write_kinetic(V, p0 + threadIdx.x, ftm);
     });
 }
 

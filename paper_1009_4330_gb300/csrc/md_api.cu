@@ -570,7 +570,6 @@ static md_status create_impl(int n_rep, const md_config *cfgs, const double *con
     }
     if (V.pot == MD_POT_EAM_FS) {
         if (V.prec == MD_PREC_FP64) AL(V.fp64, n);
-        else AL(V.fp32, n);
         AL(V.emb, n);
     }
     AL(V.ev, 8 * n);

@@ -140,8 +140,7 @@ struct View {
     int *wl_u0, *wl_bin, *wl_hs, *wl_s0, *wl_a0, *wl_n;
     int n_sm;             // SMs of the device (fixed grids)
     // EAM
-    double *fp64;         // F'(rho) per atom (fp64 path)
-    float *fp32;          // F'(rho) per atom (mixed path)
+    double *fp64;         // F'(rho) per atom (fp64 path; the mixed path keeps it in rec.w)
     double *emb;          // F(rho) per atom (energy)
     // per-atom energy / virial for deterministic reductions: [8][n_pad]
     double *ev;
@@ -430,6 +429,24 @@ __device__ __forceinline__ int tile_mode(const View &V, int T) {
         return -1;
     }
     return V.tile_cnt[blockIdx.x] >= 0 ? 1 : 0;
+}
+
+// epilogue of force component c of slot p, kick or store (see the modes above); ftm: ftm2v / mass
+__device__ __forceinline__ void finish_component(const View &V, int mode, int rem, int c, int p, double ftm, double f) {
+    const size_t i = (size_t)c * V.n_pad + p;
+    if (mode == kModeStep || mode == kModeKickDry) {
+        const bool last = (mode == kModeStep && rem == 0);
+        V.v[i] += ((mode == kModeKickDry) ? 0.0 : (last ? 0.5 : 1.0) * V.dt * ftm) * f;
+        if (!last) return;
+    }
+    V.f[i] = f;
+}
+
+// the kinetic term of slot p for an energy pass
+__device__ __forceinline__ void write_kinetic(const View &V, int p, double ftm) {
+    const int n = V.n_pad;
+    const double vx = V.v[p], vy = V.v[n + p], vz = V.v[2 * n + p];
+    V.ev[n + p] = 0.5 * (vx * vx + vy * vy + vz * vz) / ftm;
 }
 
 // blocks an energy reduction is spread over at most (where a replica takes several)
