@@ -1208,8 +1208,10 @@ constexpr int kRowBuild = 6;
 // line at 3 and 12 units per SM 244 and 258).  Batches of at most kRowBuildOnly units per SM in all are built by
 // rows only, which saves the second launch (10 replicas of 2,000 atoms at rc 2.5, 8.4 units, 52.7 -> 50.3; at 11.4 of
 // denser cells, 8 of 8,000 at rc 5.0 together, it costs 197 -> 238), those of more than kRowBuildWl cells per SM by
-// cells only.
-constexpr int kRowBuildOnly = 9, kRowBuildWl = 64;
+// cells only.  In between, the two run side by side in a step's graph where rows are the likely choice (one
+// replica in seven rebuilding): 16 replicas of 500 .. 4,000 atoms 68.0 -> 65.2 (64.7 by rows only), 30 of 500 .. 3,000
+// 79.3 -> 76.7 (76.2); in larger batches the build by cells loses by it (4 of 60,000 at rc 5.0, 45 units: 430 -> 448).
+constexpr int kRowBuildOnly = 9, kRowBuildLikely = 7 * kRowBuild, kRowBuildWl = 64;
 
 // threads per block of the per-slot passes (k_prepare, k_scatter, k_gather), as the drift's: evaluation of 100,003 atoms at
 // new coordinates 225 (256) -> 222 us
@@ -1265,7 +1267,8 @@ void list_build_sequence(const View &V, bool all, std::vector<KCall> &seq) {
         const void *kb = fp64 ? (V.half ? (const void *)k_build_wl<MD_PREC_FP64, 1> : (const void *)k_build_wl<MD_PREC_FP64, 0>)
                               : (V.half ? (const void *)k_build_wl<MD_PREC_MIXED, 1> : (const void *)k_build_wl<MD_PREC_MIXED, 0>);
         const int deal = std::min(kBuildWlDeal, 1 + V.nbins_total / (V.n_sm * kBuildWarps * 4));
-        seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * deal), dim3(32), 0, a});
+        const bool beside = rows && V.nbins_total * V.hsplit <= V.n_sm * kRowBuildLikely;
+        seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * deal), dim3(32), 0, a, beside});
         return;
     }
     const void *kb;

@@ -118,7 +118,9 @@ static cudaError_t run_seq(md_system *h, const std::vector<KCall> &seq) {
 
 static cudaError_t add_chain(md_system *h, cudaGraph_t g, const std::vector<KCall> &seq, cudaGraphNode_t *dep,
                              cudaGraphNode_t *last) {
-    cudaGraphNode_t prev = dep ? *dep : nullptr;
+    // what the next call waits for, and what the one before it waited for
+    std::vector<cudaGraphNode_t> after, before;
+    if (dep) after.push_back(*dep);
     for (const KCall &k : seq) {
         View Vc = h->V;
         KArgs a = k.args;
@@ -129,12 +131,17 @@ static cudaError_t add_chain(md_system *h, cudaGraph_t g, const std::vector<KCal
         kp.blockDim = k.block;
         kp.sharedMemBytes = (unsigned)k.smem;
         kp.kernelParams = args;
+        const std::vector<cudaGraphNode_t> &deps = k.beside ? before : after;
         cudaGraphNode_t node;
-        cudaError_t e = cudaGraphAddKernelNode(&node, g, prev ? &prev : nullptr, prev ? 1 : 0, &kp);
+        cudaError_t e = cudaGraphAddKernelNode(&node, g, deps.data(), deps.size(), &kp);
         if (e != cudaSuccess) return e;
-        prev = node;
+        if (!k.beside) {
+            before = after;
+            after.clear();
+        }
+        after.push_back(node);
+        *last = node;
     }
-    *last = prev;
     return cudaSuccess;
 }
 

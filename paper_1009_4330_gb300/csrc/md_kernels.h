@@ -14,6 +14,7 @@ struct KCall {
     dim3 grid, block;
     size_t smem;
     KArgs args;
+    bool beside = false;  // independent of the call before it: in a graph they run side by side
 };
 
 // rebuild: zero bins, prepare, scan, scatter, gather, build.  all = every
