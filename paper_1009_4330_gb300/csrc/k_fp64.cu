@@ -53,6 +53,8 @@ constexpr float kScreen = 1.0009765625f;  // entries are screened at 2^-10 above
 // Warps per SM of the one wave: 20 (at most 96 registers) for the LJ and EAM
 // density passes without energies, 16 for the others.  32,000 / 256,000-atom LJ pass: 84.4 /
 // 523 us with 16, 74.4 / 515 with 20, 91.0 / 596 with 12 (EAM backward: 844, 863, 818).
+// Systems of U = 4 fill at most 16 warps per SM and are compiled for as many: with more than 128 registers a
+// part of them made a second wave (LJ backward, two types, 9,700 atoms 92 -> 69 us).
 constexpr int kWarpsMany = 20, kWarpsFew = 16;
 
 // shared memory of a warp with NS sums per lane:
@@ -105,7 +107,8 @@ __device__ __forceinline__ const uint32_t *list_of(const View &V, int p, int Q) 
 // atom is the only one of its partial sum k, each is stored as it comes: the same bits as the groups' walk below, which such
 // lists leave mostly idle (eight lanes for one or two pairs, ~75 instructions an atom).  us per LJ pass of 256,000 atoms at
 // density 0.005 / 0.02 / 0.05 (full list) groups 30.3 / 63.5 / 95.8, so 24.6 /
-// 36.8 / 71.7.  The backward passes keep to the groups: the second walk cost them registers (EAM 6,912 atoms 80 -> 95 us).
+// 36.8 / 71.7.  The backward passes keep to the groups: the second walk cost them registers (EAM 6,912 atoms 80 -> 95
+// us), and so do systems small enough for U = 4.
 constexpr int kShortPairs = kGroups * kRing / 2;
 template <class Src, int Q, class Pair>
 __device__ __forceinline__ void short_walk(const View &V, const Rep &R, int p0, int cnt, int most, char *smem, Pair &pair) {
@@ -183,6 +186,9 @@ __device__ __forceinline__ void fp64_walk(const View &V, const Rep &R, int p0, i
     uint32_t *const ring = reinterpret_cast<uint32_t *>(smem) + grp * kRing;
     double *const xs = reinterpret_cast<double *>(smem + kGroups * kRing * 4);
     double *const sums = reinterpret_cast<double *>(smem + kSumsAt);
+    constexpr bool kShort = !Src::packed && U == 1;  // batches of short lists are walked by short_walk
+    int count = 0;  // (loaded with the positions)
+    if (kShort && lane < nb) count = V.ncount[p0 + lane];
     // x_i shifted into the frames of the neighbouring cells: dx = -1, 0, 1 -> x_i + h, x_i, x_i - h
     for (int k = lane; k < 3 * nb; k += 32) {
         const int i = k / 3, c = k - 3 * i;
@@ -192,11 +198,10 @@ __device__ __forceinline__ void fp64_walk(const View &V, const Rep &R, int p0, i
         xs[3 * k + 2] = x - R.h[c];
     }
     __syncwarp();
-    if constexpr (!Src::packed) {
-        const int c = lane < nb ? V.ncount[p0 + lane] : 0;
-        const int most = __reduce_max_sync(kFull, c);
-        if (most <= kGrp && __reduce_add_sync(kFull, c) <= kShortPairs) {
-            short_walk<Src, Q>(V, R, p0, c, most, smem, pair);
+    if constexpr (kShort) {
+        const int most = __reduce_max_sync(kFull, count);
+        if (most <= kGrp && __reduce_add_sync(kFull, count) <= kShortPairs) {
+            short_walk<Src, Q>(V, R, p0, count, most, smem, pair);
             return;
         }
     }
@@ -420,7 +425,7 @@ struct Lj64 {
 };
 
 template <int Q, int U, int HALF, int EV, int MT>
-__global__ void __launch_bounds__(32, U == 4 ? 8 : EV ? kWarpsFew : kWarpsMany) k64_lj(View V, KArgs a) {
+__global__ void __launch_bounds__(32, U == 4 || EV ? kWarpsFew : kWarpsMany) k64_lj(View V, KArgs a) {
     extern __shared__ char smem[];
     if (V.ctl->err) return;
     const int rem = (a.mode == kModeStep) ? V.ctl->remaining : 0;
@@ -461,7 +466,7 @@ struct Rho64 {
 };
 
 template <int Q, int U>
-__global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsMany) k64_eam_rho(View V, KArgs a) {
+__global__ void __launch_bounds__(32, U == 4 ? kWarpsFew : kWarpsMany) k64_eam_rho(View V, KArgs a) {
     extern __shared__ char smem[];
     if (V.ctl->err) return;
     Rho64 pr{};
@@ -538,7 +543,7 @@ struct Eam64 {
 };
 
 template <int Q, int U, int EV>
-__global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_eam_force(View V, KArgs a) {
+__global__ void __launch_bounds__(32, kWarpsFew) k64_eam_force(View V, KArgs a) {
     extern __shared__ char smem[];
     if (V.ctl->err) return;
     const int rem = (a.mode == kModeStep) ? V.ctl->remaining : 0;
@@ -668,7 +673,7 @@ struct LjBwd64 {
 
 // gp_part: [block][2 per unordered type pair]
 template <int Q, int U, int MT>
-__global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_lj_bwd(View V, KArgs, double *grad_x) {
+__global__ void __launch_bounds__(32, kWarpsFew) k64_lj_bwd(View V, KArgs, double *grad_x) {
     extern __shared__ char smem[];
     const int nt = V.ntypes, npar = nt * (nt + 1);
     const int lane = threadIdx.x;
@@ -757,7 +762,7 @@ struct EamBwd1 {
 };
 
 template <int Q, int U>
-__global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_eam_bwd1(View V, KArgs) {
+__global__ void __launch_bounds__(32, kWarpsFew) k64_eam_bwd1(View V, KArgs) {
     extern __shared__ char smem[];
     EamBwd1 pr{};
     pr.rc = V.tab->eam[0];
@@ -823,7 +828,7 @@ struct EamBwd2 {
 };
 
 template <int Q, int U>
-__global__ void __launch_bounds__(32, U == 4 ? 8 : kWarpsFew) k64_eam_bwd2(View V, KArgs, double *grad_x) {
+__global__ void __launch_bounds__(32, kWarpsFew) k64_eam_bwd2(View V, KArgs, double *grad_x) {
     extern __shared__ char smem[];
     EamBwd2 pr{};
     pr.rc = V.tab->eam[0];
