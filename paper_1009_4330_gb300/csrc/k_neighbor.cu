@@ -1256,18 +1256,18 @@ void list_build_sequence(const View &V, bool all, std::vector<KCall> &seq) {
     const bool fp64 = V.prec == MD_PREC_FP64;
     if (V.n_rep > 1 && !all) {
         const bool rows = V.tile_atoms == 0 && V.nbins_total <= V.n_sm * kRowBuildWl;
-        const bool only = V.nbins_total * V.hsplit <= V.n_sm * kRowBuildOnly;
-        a.aux = !rows ? 0 : only ? V.nbins_total * V.hsplit : V.n_sm * kRowBuild;
+        const bool only = V.n_units <= V.n_sm * kRowBuildOnly;
+        a.aux = !rows ? 0 : only ? V.n_units : V.n_sm * kRowBuild;
         if (rows) {
             const void *kr = fp64 ? (V.half ? (const void *)k_build_rows_wl<MD_PREC_FP64, 1> : (const void *)k_build_rows_wl<MD_PREC_FP64, 0>)
                                   : (V.half ? (const void *)k_build_rows_wl<MD_PREC_MIXED, 1> : (const void *)k_build_rows_wl<MD_PREC_MIXED, 0>);
-            seq.push_back(KCall{kr, dim3(std::min(V.n_sm * kRowBuild, V.nbins_total * V.hsplit)), dim3(288), 0, a});
+            seq.push_back(KCall{kr, dim3(std::min(V.n_sm * kRowBuild, V.n_units)), dim3(288), 0, a});
             if (only) return;
         }
         const void *kb = fp64 ? (V.half ? (const void *)k_build_wl<MD_PREC_FP64, 1> : (const void *)k_build_wl<MD_PREC_FP64, 0>)
                               : (V.half ? (const void *)k_build_wl<MD_PREC_MIXED, 1> : (const void *)k_build_wl<MD_PREC_MIXED, 0>);
         const int deal = std::min(kBuildWlDeal, 1 + V.nbins_total / (V.n_sm * kBuildWarps * 4));
-        const bool beside = rows && V.nbins_total * V.hsplit <= V.n_sm * kRowBuildLikely;
+        const bool beside = rows && V.n_units <= V.n_sm * kRowBuildLikely;
         seq.push_back(KCall{kb, dim3(V.n_sm * kBuildWarps * deal), dim3(32), 0, a, beside});
         return;
     }

@@ -475,6 +475,7 @@ static md_status create_impl(int n_rep, const md_config *cfgs, const double *con
         for (Rep &R : h->reps) {
             const double m = (double)R.natoms / (double)R.nbins;
             R.hsplit = split(m);  // a replica's own cells (work-list builds of a batch)
+            V.n_units += R.nbins * R.hsplit;
             mean = std::max(mean, m);
         }
         V.hsplit = split(mean);
