@@ -11,7 +11,8 @@
 //   * a list entry is first tested in FP32 on the 16-byte records (cut-off
 //     plus a margin far above the FP32 error).  Only the entries that pass, ~70 % (the
 //     list reaches rc + skin), are queued in shared memory and evaluated in FP64, eight
-//     lanes to an atom, so that the FP64 instructions run with full warps;
+//     lanes to an atom (short lists: all of a warp's in one queue), so that the FP64
+//     instructions run with full warps;
 //   * x_i plus the stencil cell's shift is formed once per atom (3 values per
 //     axis, in shared memory), which leaves one FP64 subtraction per
 //     component of d;
@@ -19,13 +20,13 @@
 //     the exact cut-off comparison are integer operations on the words of the
 //     double.
 // 17 FP64 instructions per evaluated LJ pair instead of 28 per list entry, with the
-// FP64 pipe 80-86 % busy.  Against one pass of FP64 arithmetic over every
-// entry (time per pass): LJ 256,000 atoms, half list 994 -> 456 us; LJ 4,000
-// atoms 30.6 -> 18.5 us; EAM 108,000 atoms (density + force) 863 -> 360 us; backward
-// LJ 32,768 atoms, two types 534 -> 198 us, EAM 108,000 atoms 1,337 -> 731 us.
+// FP64 pipe 79-86 % busy.  Against one pass of FP64 arithmetic over every
+// entry (time per pass): LJ 256,000 atoms, half list 994 -> 443 us; LJ 4,000
+// atoms 30.6 -> 19 us; EAM 108,000 atoms (density + force) 863 -> 366 us; backward
+// LJ 32,768 atoms, two types 534 -> 195 us, EAM 108,000 atoms 1,337 -> 728 us.
 //
 // The atoms are dealt out evenly, in units of four, to one wave of one-warp
-// blocks (at most 16 per SM): a second, partly filled wave cost up to 30 % of
+// blocks (at most 20 per SM): a second, partly filled wave cost up to 30 % of
 // a pass.  A warp works through its range in batches of at most 32 atoms, in four
 // groups of eight lanes; a group takes the batch's next atom as soon as it is
 // done with one and does not wait for the others (its lanes' partial sums go

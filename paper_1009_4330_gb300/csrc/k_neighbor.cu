@@ -576,7 +576,7 @@ __device__ __forceinline__ void buf_store(unsigned sa, uint32_t e) {
 // Each row is read as one flat candidate range, 32 candidates at a time, one per
 // lane, the next 32 on their way meanwhile, shifted into the home cell's
 // frame.  A candidate farther than rl from the bounding box of
-// the home atoms cannot be accepted by any of them (about 30 % of the 27-cell
+// the home atoms cannot be accepted by any of them (about 38 % of the 27-cell
 // candidates); the others go to a per-warp queue in shared memory, in
 // candidate order, and are tested in full rounds of 32: each lane
 // tests its candidate against every home atom (records broadcast from shared
@@ -588,7 +588,7 @@ __device__ __forceinline__ void buf_store(unsigned sa, uint32_t e) {
 // written out four entries (16 bytes) at a time.  So the lists are in candidate
 // order (deterministic).
 // The home atoms' tests are two to an instruction (FP32x2).  What bounds it: instruction issue (73 %) and
-// the L1 data pipe (75 %) at rc 2.5, both at ~65 % at rc 5.0.  Against scanning each home
+// the L1 data pipe (77 %) at rc 2.5; at rc 5.0 (55 and 56 %) also the list's partly written sectors.  Against scanning each home
 // atom's masks bit by bit and storing 4-byte entries straight to the list, whose
 // scattered sectors bound the build at rc 5.0 (one launch, 500,000 atoms): rc 2.5 225 ->
 // 220 us (209.6 M -> 187.8 M warp instructions), rc 5.0 1.51 -> 1.09 ms; measured and not kept:
