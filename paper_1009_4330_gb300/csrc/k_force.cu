@@ -1560,15 +1560,18 @@ static const void *pick_eamf(int T, int Q, int ev) {
 // atoms 26.2 (8 lanes) / 26.0 (16), 16,000 atoms 28.9 (4) / 29.4 (8), 32,771 atoms 34.6 (2) / 32.5 (4) / 36
 // (8); one lane: 31 .. 33.  32 lanes for the smallest systems measured the same as 16.
 // Two lanes pay up to 640 threads per SM only (60,000 atoms: 36.9 us with one, 38.0 with two).
-// More lanes than the longest list has rounds would only stand by and add to the terms' sums: EAM 4,000 atoms with 8
-// threads per atom (two rounds) 25.2 (4 lanes) -> 21.8 us per step, LJ 4,096 with 4 at rc 1.12 22.8 (8) -> 20.3 (1).
-constexpr int kWideThreads = 880, kWideThreads2 = 640, kWideMost = 4;
+// Lanes beyond the rounds of the longest list only stand by and add to the terms' sums: none where there are as
+// many lanes as rounds, and up to kWideIdle threads per SM where there would be more (EAM 4,000 atoms with 8 threads per
+// atom, two or three rounds, 4 lanes / 2: 25.2 / 21.8 us per step, LJ 4,096 with 4 at rc 1.12, one round, 8 / 1: 22.8 / 20.3;
+// but 5,000 atoms with lists of five rounds, 4 lanes / 8 21.0 / 19.9).
+constexpr int kWideThreads = 880, kWideThreads2 = 640, kWideIdle = 300, kWideMost = 4;
 
-static int wide_log(const View &V) {
+int wide_lanes(const View &V) {
+    if (V.prec != MD_PREC_MIXED || V.half || V.tile_atoms > 0) return 0;
+    const int rounds = (V.list_most + (V.vec << V.ltpa) - 1) >> (V.ltpa + V.lvec);
     int lg = 0;
-    const int rounds = (V.list_most + (V.vec << V.ltpa) - 1) >> (V.ltpa + V.lvec);  // of the longest list
     while (lg < kWideMost && V.ltpa + lg < 5 && (1 << lg) < rounds &&
-           ((long long)V.n_pad << (V.ltpa + lg + 1)) <= (long long)V.n_sm * kWideThreads)
+           ((long long)V.n_pad << (V.ltpa + lg + 1)) <= (long long)V.n_sm * ((2 << lg) <= rounds ? kWideThreads : kWideIdle))
         ++lg;
     if (lg == 1 && ((long long)V.n_pad << (V.ltpa + 1)) > (long long)V.n_sm * kWideThreads2) lg = 0;
     return lg;
@@ -1581,7 +1584,7 @@ static int wide_log(const View &V) {
 static void mixed_force_sequence(const View &V, int mode, int block, KArgs a, std::vector<KCall> &seq) {
     const int T = V.tpa;
     const int ev = (mode == kModeEV) ? 1 : 0;
-    const int lg = V.half || V.tile_atoms > 0 ? 0 : wide_log(V);
+    const int lg = wide_lanes(V);
     if (lg > 0) {
         a.aux = lg;
         const dim3 grid((unsigned)((((long long)V.n_pad << (V.ltpa + lg)) + kWideBlock - 1) / kWideBlock));

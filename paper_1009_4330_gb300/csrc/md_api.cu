@@ -251,6 +251,16 @@ static md_status rebuild_list_only(md_system *h, bool all) {
     return MD_OK;
 }
 
+// The longest list that the wide mixed passes have lanes for.  It only grows, and graphs are built anew only where the
+// lanes change with it.  (A batch's lists are not looked at: its capacity.)
+static void note_longest(md_system *h, const Ctl &c) {
+    const int most = h->n_rep > 1 ? h->V.maxneigh : h->V.half ? 2 * c.maxcnt : c.maxcnt;
+    if (most <= h->V.list_most) return;
+    const int lanes = wide_lanes(h->V);
+    h->V.list_most = most;
+    if (wide_lanes(h->V) != lanes) drop_graph(h);
+}
+
 // After a build: grow the list and rebuild while it overflowed.
 static md_status settle_overflow(md_system *h, bool all) {
     for (int it = 0; it < 8; ++it) {
@@ -258,9 +268,9 @@ static md_status settle_overflow(md_system *h, bool all) {
         md_status st = read_ctl(h, &c);
         if (st) return st;
         if (c.err & kErrNonfinite) return fail(h, MD_ERR_NONFINITE, "non-finite position or velocity");
+        note_longest(h, c);
         if (!(c.err & kErrOverflow)) return MD_OK;
         const int need = round_up((int)std::ceil(c.need_maxneigh * 1.2) + 8, 128);
-        h->V.list_most = std::max(h->V.list_most, h->V.half ? 2 * c.need_maxneigh : c.need_maxneigh);
         st = alloc_list(h, need);
         if (st) return st;
         unsigned zero = 0;
@@ -531,7 +541,6 @@ static md_status create_impl(int n_rep, const md_config *cfgs, const double *con
     V.tile_rep = d_tile_rep;
     AL(V.rep_disp, (size_t)n_rep);
     AL(V.rep_flag, (size_t)n_rep);
-    AL(V.rep_maxcnt, (size_t)n_rep);
     AL(V.rep_entries, (size_t)n_rep);
     int *d_bin_rep, *d_lin2bin, *d_bin2xyz;
     AL(d_bin_rep, (size_t)V.nbins_total);
@@ -583,6 +592,8 @@ static md_status create_impl(int n_rep, const md_config *cfgs, const double *con
     AL(V.ev, 8 * n);
     AL(h->d_tab, 1);
     AL(h->d_ctl, 1);
+    if (n_rep == 1) V.rep_maxcnt = &h->d_ctl->maxcnt;
+    else AL(V.rep_maxcnt, (size_t)n_rep);
     AL(V.wl_u0, (size_t)n_rep + 1);
     AL(V.wl_bin, (size_t)n_rep);
     AL(V.wl_hs, (size_t)n_rep);
@@ -675,13 +686,6 @@ static md_status create_impl(int n_rep, const md_config *cfgs, const double *con
     set_tiles(h);
     st = full_rebuild(h, true);
     if (st) { md_destroy(h); return st; }
-    {
-        int most = 0;
-        long long entries = 0;
-        st = read_stats(h, &most, &entries);
-        if (st) { md_destroy(h); return st; }
-        V.list_most = V.half ? 2 * most : most;
-    }
     st = compute_forces(h, kModeStoreF);
     if (st) { md_destroy(h); return st; }
     if (h->cfg.tpa == 0) {
@@ -799,6 +803,7 @@ md_status md_step(md_system *h, int64_t nsteps) {
         if (c.err & kErrTimeout) return fail(h, MD_ERR_TIMEOUT, "device wait timed out");
         if (c.err & kErrConfig) return fail(h, MD_ERR_INVALID, "force launch does not match the list's tiles");
         if (!(c.err & kErrOverflow)) {
+            note_longest(h, c);
             if (c.remaining != 0) return fail(h, MD_ERR_CUDA, "step loop ended with %d steps left", c.remaining);
             return MD_OK;
         }
@@ -908,6 +913,7 @@ md_status md_eval_forces(md_system *h, const double *params, const double *x, do
     Ctl c;
     md_status st = read_ctl(h, &c);
     if (st) return st;
+    note_longest(h, c);
     if (!c.err) return MD_OK;
     st = settle_overflow(h, true);
     if (st) return st;

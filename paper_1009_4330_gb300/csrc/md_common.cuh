@@ -77,6 +77,7 @@ struct Ctl {                // device control block of a handle
     unsigned disp_max;      // md_vv MD_VV_DISP: max squared displacement since the build, float bits
     unsigned ticket_ev;     // last-block ticket of the energy reduction (reset by the last block)
     unsigned ticket_scan;   // last-block ticket of the bin-count scan's first pass (reset by the last block)
+    int maxcnt;             // a single system's rep_maxcnt: read with the status, at no copy of its own
 };
 
 // Parameters of the potential, per ordered type pair p = ti * nt + tj.
@@ -102,7 +103,7 @@ struct View {
     int tpa;          // threads per atom the list is laid out for
     int vec;          // entries per thread per list load (1, 2 or 4)
     int ltpa, lvec;   // log2 of tpa and vec
-    int list_most;    // longest full list at creation, or that the list has grown for since
+    int list_most;    // longest full list that a build has reported so far (a batch: the capacity)
     int half;         // 1: half list (each pair once, Newton-3 atomics)
     int prec;         // md_precision
     int pot;          // md_potential

@@ -38,6 +38,9 @@ bool steps_sequence(const View &V, std::vector<KCall> &seq);
 // kModeEV).  `block` = threads per block.
 void force_sequence(const View &V, int mode, int block, bool in_graph, std::vector<KCall> &seq);
 
+// log2 of the lanes that stand in for one thread of the list layout in the mixed passes of this system (see V.list_most)
+int wide_lanes(const View &V);
+
 // its FP64 pair passes ([LJ pass], or [density, force] for EAM); mode: as above,
 // a: the arguments of the launches (half lists: the mode of a pass that only stores)
 void fp64_force_sequence(const View &V, int mode, KArgs a, std::vector<KCall> &seq);

@@ -84,3 +84,25 @@ def test_eam_scalar_and_packed_density_pass(vec):
     r, kw = _eam(_atoms(600))
     assert _atoms(330) < len(r["x"]) < _atoms(880)
     _same_bits(kw, r, 2, 1, vec)
+
+
+def test_lists_that_get_longer():
+    """A system made as a gas and then filled: the lanes follow its lists, in the passes and in the step's graph."""
+    from paper_1009_4330_gb300 import System
+    n = 1500
+    y, _ = synth.fcc_subset(n, 0.8442, 31)
+    y = synth.displace(y, np.full(3, (n / 0.8442) ** (1 / 3)), 0.04, 32)
+    box = np.full(3, 60.0)
+    x = np.random.default_rng(1).random((n, 3)) * box
+    v = synth.maxwell_boltzmann(n, 1.44, 1.0, 33)
+    kw = dict(_lj(64, 0.8442, 2.5, 1)[1], skin=0.3)
+    with System(x, v, None, box, **kw) as a, System(y, v, None, box, **kw) as b:
+        a.step(3)
+        a.set_state(x=y, v=v)
+        for s in (a, b):
+            s.set_kernel(16, "full", 128, 1)  # (more turns than one cluster takes: separate launches)
+        assert np.array_equal(a.compute_forces().cpu().numpy(), b.compute_forces().cpu().numpy())
+        for s in (a, b):
+            s.step(40)
+        for u, w in zip(a.state(), b.state()):
+            assert np.array_equal(u.cpu().numpy(), w.cpu().numpy())
